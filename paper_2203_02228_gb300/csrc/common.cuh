@@ -202,37 +202,49 @@ __device__ __forceinline__ int32_t euc2d_m(uint64_t m) {
   return (int32_t)(r + ((m - rr) > r ? 1u : 0u));
 }
 
-// The same cost of two points, on a short dependency chain.  An FP32
-// estimate d of sqrt(dx^2 + dy^2) is accepted when the exact integer test
-// d^2 - d < m <= d^2 + d holds, which says (d - 1/2)^2 < m < (d + 1/2)^2,
-// i.e. d = nint(sqrt(m)); otherwise the exact integer steps of euc2d_m
-// decide.  The estimate: |dx|, |dy| < 2^22 convert to FP32 exactly by the
-// 1.5 * 2^23 bias (an add on the bit pattern and a float subtract), the
-// hardware's approximate square root (sqrt.approx.f32) follows, and an
-// estimate below 2^22 rounds to the nearest integer by the same bias.  Its
-// relative error is about 2^-21, so the test fails only for costs above
-// ~10^6, next to a half-integer, or with |dx| or |dy| >= 2^22 (where the
-// bias tricks do not hold and the estimate is meaningless): those, and
-// m = 0 (d = 0 fails the test), take the exact path.
+// The same cost of two points without a branch.  An FP32 estimate d of
+// sqrt(dx^2 + dy^2) is off by at most one when dx^2 + dy^2 < 2^42, and the
+// integer remainder q = m - d^2 says which way: d = nint(sqrt(m)) exactly
+// when d^2 - d < m <= d^2 + d (that is (d - 1/2)^2 < m < (d + 1/2)^2; for
+// d = 0: m = 0), so q > d adds one and q <= -d takes one off.
+//   - |dx|, |dy| < 2^22 convert to FP32 exactly by the 1.5 * 2^23 bias (an
+//     add on the bit pattern and a float subtract); beyond that the biased
+//     value only grows in magnitude, so the sum of squares is then >= 2^44
+//     and the guard below catches it;
+//   - below 2^42 the sum of squares is off by a relative 2^-23 at most, its
+//     root by 2^-24, and sqrt.approx adds 2^-23: less than 0.5 in all at
+//     d < 2^21, so the rounded estimate is within one of the truth;
+//   - |q| < 2^24 then, so q is exact in 32-bit wrap-around arithmetic.
+// `big` collects the guard: a caller with several costs runs them side by
+// side and tests it once.  (With a branch per cost -- the estimate accepted
+// or the exact steps -- the costs of one local-search evaluation could not
+// overlap: see eval_both.)
 __device__ __forceinline__ float i2f_biased(int32_t v) {  // exact for |v| < 2^22
   return __fsub_rn(__int_as_float(v + 0x4B400000), 12582912.0f);
 }
 
-__device__ __forceinline__ float sqrt_approx(float x) {
+__device__ __forceinline__ float sqrt_approx(float x) {  // x = 0 or x >= 1: never subnormal
   float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 
-__device__ __forceinline__ int32_t euc2d(int2 a, int2 b) {
+__device__ __forceinline__ int32_t euc2d_near(int2 a, int2 b, bool& big) {
   const int32_t dx = a.x - b.x, dy = a.y - b.y;  // |dx|, |dy| < 2^24
-  const uint64_t m = (uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy);
   const float fx = i2f_biased(dx), fy = i2f_biased(dy);
   const float mf = __fmaf_rn(fx, fx, __fmul_rn(fy, fy));
-  const uint32_t d = (uint32_t)(__float_as_int(__fadd_rn(sqrt_approx(mf), 12582912.0f)) - 0x4B400000);
-  const uint64_t dd = (uint64_t)d * d;
-  if (m > dd - d && m <= dd + d) return (int32_t)d;
-  return euc2d_m(m);
+  big |= !(mf < 4398046511104.0f);  // 2^42
+  const int32_t d = __float_as_int(__fadd_rn(sqrt_approx(mf), 12582912.0f)) - 0x4B400000;
+  const int32_t q = (int32_t)((uint32_t)dx * (uint32_t)dx + (uint32_t)dy * (uint32_t)dy - (uint32_t)d * (uint32_t)d);
+  return d + (q > d ? 1 : 0) - (q + d < min(d, 1) ? 1 : 0);
+}
+
+static __device__ __noinline__ int32_t euc2d_far(int2 a, int2 b) { return euc2d_m(sqdist(a, b)); }
+
+__device__ __forceinline__ int32_t euc2d(int2 a, int2 b) {
+  bool big = false;
+  const int32_t d = euc2d_near(a, b, big);
+  return big ? euc2d_far(a, b) : d;
 }
 
 // ---------------------------------------------------------------------

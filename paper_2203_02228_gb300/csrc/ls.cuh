@@ -150,17 +150,22 @@ __device__ __forceinline__ bool tour_move2(Tour& T, int n1, int n2, int n3, int 
 }
 
 // Both scans from a in one pass over NN(a) (one lookup of a, one of each
-// neighbour b): the best 2-opt move and, when do_or, the best Or-opt move.
-// The search then takes the 2-opt move if it gains, else the Or-opt move --
-// the same decision as scanning one after the other.  Lane layout: with
-// k <= 16, lane = side * 16 + s (side 0: the edge (b, succ b), side 1:
-// (pred b, b)); with k > 16, lane = s and the two sides are two passes.
-// The loads that do not depend on the walk from a (the candidate row, b's
-// coordinates) are issued before it; the move is rebuilt from the winning
-// lane's registers.
+// neighbour b): the best 2-opt move if one gains, else (do_or) the best
+// Or-opt move -- the same decision as scanning one after the other.  Returns
+// the gain (0: none) and the move on every lane: mv[7] = 0 for 2-opt
+// (mv[0..3]), 1 for Or-opt (mv[0..6]).
+// Lane layout: with k <= 16, lane = side * 16 + s (side 0: the edge
+// (b, succ b), side 1: (pred b, b)); with k > 16, lane = s and the two sides
+// are two passes.  The loads that do not depend on the walk from a (the
+// candidate row, b's coordinates) are issued before it; the move is rebuilt
+// from the winning lane's registers.
+// Bound by latency while few warps of an SM evaluate and by instruction
+// issue while all do, so the costs are branch-free (euc2d_near): the seven a
+// lane needs run side by side, both sides share one piece of code (swapping
+// the ends of the edge at b only swaps the two orientations of an Or-opt
+// move), and no index is divided by k.
 template <class Tour>
-__device__ __forceinline__ void eval_both(const Tour& T, int a, bool do_or, int64_t& g2, int mv2[4],
-                                          int64_t& go, int mvo[7]) {
+__device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, int (&mv)[8]) {
   const int n = T.n, k = T.k, lane = lane_id();
   do_or = do_or && n >= 8;
   const bool two = k > 16;
@@ -217,122 +222,121 @@ __device__ __forceinline__ void eval_both(const Tour& T, int a, bool do_or, int6
   // gains in 32 bits: each is a signed sum of at most six EUC_2D costs of
   // coordinates below 2^24 (each cost below 2^25)
   int32_t rem1 = 0, rem2 = 0, rem3 = 0;
-  {
-    const int32_t c2 = __shfl_sync(kFull, cst, 2), c3 = __shfl_sync(kFull, cst, 3),
-                  c4 = __shfl_sync(kFull, cst, 4), c5 = __shfl_sync(kFull, cst, 5),
-                  c6 = __shfl_sync(kFull, cst, 6);
-    if (do_or) {
-      rem1 = d_ap + d_as - c2;
-      rem2 = d_ap + c3 - c4;
-      rem3 = d_ap + c5 - c6;
-    }
+  if (do_or) {
+    rem1 = d_ap + d_as - __shfl_sync(kFull, cst, 2);
+    rem2 = d_ap + __shfl_sync(kFull, cst, 3) - __shfl_sync(kFull, cst, 4);
+    rem3 = d_ap + __shfl_sync(kFull, cst, 5) - __shfl_sync(kFull, cst, 6);
   }
-  int32_t b2 = 0, bo = 0;
-  int i2 = INT_MAX, io = INT_MAX;
+  // the lane's best move: a gaining 2-opt move counts kTwoOpt more than its
+  // gain, so that it beats every Or-opt move; code = l * 4 + orientation * 2
+  // + side (l = 0: 2-opt), idx = its place in the sequential scan
+  constexpr int32_t kTwoOpt = 1 << 28;
+  int32_t best = 0;
+  int bidx = INT_MAX, bcode = 0, bbn = a;
   const int passes = two ? 2 : 1;
   for (int pass = 0; pass < passes; ++pass) {
     const int side = two ? pass : (lane >> 4);
     const int bn = pass == 0 ? bn0 : bn1;
     const int2 xbn = pass == 0 ? xbn0 : xbn1;
-    int32_t g = 0;
-    int32_t lo = 0;
-    int li = INT_MAX;
-    if (live) {
-      const int d_bbn = euc2d(xb, xbn);
-      if (side == 0) {
-        if (d_as > d_ab) g = d_as + d_bbn - d_ab - euc2d(x1, xbn);
-      } else {
-        if (d_ap > d_ab) g = d_ap + d_bbn - d_ab - euc2d(xp, xbn);
-      }
+    bool big = false;
+    int32_t c_bn = euc2d_near(xb, xbn, big);   // d(b, bn)
+    int32_t c_n1 = euc2d_near(xbn, x1, big);   // d(bn, s1)
+    int32_t c_np = euc2d_near(xbn, xp, big);   // d(bn, p)
+    int32_t c_na = 0, c_b1 = 0, c_b2 = 0, c_n2 = 0;
+    if (do_or) {
+      c_na = euc2d_near(xbn, xa, big);
+      c_b1 = euc2d_near(xb, x1, big);
+      c_b2 = euc2d_near(xb, x2, big);
+      c_n2 = euc2d_near(xbn, x2, big);
+    }
+    if (__any_sync(kFull, big)) {  // an edge of 2^21 or more: the exact steps
+      c_bn = euc2d_far(xb, xbn);
+      c_n1 = euc2d_far(xbn, x1);
+      c_np = euc2d_far(xbn, xp);
       if (do_or) {
-        // the tour edge (u, v) at b: (b, succ b) or (pred b, b)
-        const int u = side == 0 ? b : bn, v = side == 0 ? bn : b;
-        const int2 xu = side == 0 ? xb : xbn, xv = side == 0 ? xbn : xb;
-        const int d_uv = d_bbn;
-        const int d_ua = side == 0 ? d_ab : euc2d(xu, xa);
-        const int d_av = side == 0 ? euc2d(xa, xv) : d_ab;
-        const bool base_bad = (u == p || v == p || u == a || v == a);
-#pragma unroll
-        for (int l = 1; l <= 3; ++l) {
-          const int q = l == 1 ? s1 : (l == 2 ? s2 : s3);
-          bool bad = base_bad || u == q || v == q;
-          if (l >= 2) bad |= (u == s1 || v == s1);
-          if (l >= 3) bad |= (u == s2 || v == s2);
-          if (bad) continue;
-          const int32_t rem = l == 1 ? rem1 : (l == 2 ? rem2 : rem3);
-          if (l == 1) {  // one node: only the reversed form, u-a-v
-            const int32_t gg = rem + d_uv - d_ua - d_av;
-            if (gg > lo) {
-              lo = gg;
-              li = (s * 2 + side) * 2;
-            }
-          } else {
-            const int2 xe = l == 2 ? x1 : x2;
-            const int d_ue = euc2d(xu, xe), d_ev = euc2d(xe, xv);
-            const int base = (((l - 1) * k + s) * 2 + side) * 2;
-            const int32_t g0 = rem + d_uv - d_ue - d_av;  // reversed: u-e ... a-v
-            if (g0 > lo) {
-              lo = g0;
-              li = base;
-            }
-            const int32_t g1 = rem + d_uv - d_ua - d_ev;  // kept: u-a ... e-v
-            if (g1 > lo) {
-              lo = g1;
-              li = base + 1;
-            }
-          }
+        c_na = euc2d_far(xbn, xa);
+        c_b1 = euc2d_far(xb, x1);
+        c_b2 = euc2d_far(xb, x2);
+        c_n2 = euc2d_far(xbn, x2);
+      }
+    }
+    int32_t v = 0;
+    int code = 0;
+    if (do_or && live) {
+      // reversed (g0) and kept (g1) insertion of a..e between the ends of the
+      // edge {b, bn}: one joins b to e and bn to a, the other b to a and bn
+      // to e; which of the two is the reversed one depends on the side
+      const bool bad1 = b == p || bn == p || bn == a || b == s1 || bn == s1;
+      const bool bad2 = bad1 || b == s2 || bn == s2;
+      const bool bad3 = bad2 || b == s3 || bn == s3;
+      if (!bad1) {  // one node: one form only
+        const int32_t g = rem1 + c_bn - d_ab - c_na;
+        if (g > v) {
+          v = g;
+          code = 4;
         }
       }
-    }
-    int idx = side * k + s;
-    if (!(g > 0)) {
-      g = 0;
-      idx = INT_MAX;
-    }
-    warp_max_gain(g, idx);
-    if (g > b2) {
-      b2 = g;
-      i2 = idx;
-    }
-    if (do_or) {
-      if (!(lo > 0)) {
-        lo = 0;
-        li = INT_MAX;
+      const int32_t e2 = rem2 + c_bn, e3 = rem3 + c_bn;
+      const int32_t be2 = e2 - c_b1 - c_na, ba2 = e2 - d_ab - c_n1;
+      const int32_t be3 = e3 - c_b2 - c_na, ba3 = e3 - d_ab - c_n2;
+      const int32_t g20 = side ? ba2 : be2, g21 = side ? be2 : ba2;
+      const int32_t g30 = side ? ba3 : be3, g31 = side ? be3 : ba3;
+      if (!bad2 && g20 > v) {
+        v = g20;
+        code = 8;
       }
-      warp_max_gain(lo, li);
-      if (lo > bo || (lo == bo && lo > 0 && li < io)) {
-        bo = lo;
-        io = li;
+      if (!bad2 && g21 > v) {
+        v = g21;
+        code = 10;
+      }
+      if (!bad3 && g30 > v) {
+        v = g30;
+        code = 12;
+      }
+      if (!bad3 && g31 > v) {
+        v = g31;
+        code = 14;
       }
     }
-  }
-  g2 = b2;
-  go = bo;
-  // the winner's b and tour neighbour, from its lane (the side is uniform)
-  int side = 0, sw = 0;
-  if (b2 > 0) {
-    side = i2 / k;
-    sw = i2 % k;
-  } else if (bo > 0) {
-    const int rest = io >> 2;
-    side = (io >> 1) & 1;
-    sw = rest % k;
-  }
-  const int wl = two ? sw : side * 16 + sw;
-  const int bw = __shfl_sync(kFull, b, wl);
-  const int bnw = __shfl_sync(kFull, (two && side == 1) ? bn1 : bn0, wl);
-  if (b2 > 0) {
-    if (side == 0) {
-      mv2[0] = a; mv2[1] = s1; mv2[2] = bw; mv2[3] = bnw;
-    } else {
-      mv2[0] = p; mv2[1] = a; mv2[2] = bnw; mv2[3] = bw;
+    const int32_t d_out = side ? d_ap : d_as;
+    const int32_t g = d_out + c_bn - d_ab - (side ? c_np : c_n1);
+    if (live && d_out > d_ab && g > 0) {
+      v = g + kTwoOpt;
+      code = 0;
     }
-  } else if (bo > 0) {
-    const int kept = io & 1, l = (io >> 2) / k + 1;
-    const int u = side == 0 ? bw : bnw, v = side == 0 ? bnw : bw;
-    mvo[0] = p; mvo[1] = a; mvo[2] = l == 1 ? a : (l == 2 ? s1 : s2);
-    mvo[3] = l == 1 ? s1 : (l == 2 ? s2 : s3); mvo[4] = u; mvo[5] = v; mvo[6] = kept;
+    const int l = code >> 2;
+    const int idx = l == 0 ? side * k + s : (((l - 1) * k + s) * 2 + side) * 2 + ((code >> 1) & 1);
+    if (v > best || (v == best && v > 0 && idx < bidx)) {
+      best = v;
+      bidx = idx;
+      bcode = code | side;
+      bbn = bn;
+    }
   }
+  const int32_t gm = __reduce_max_sync(kFull, best);
+  mv[7] = gm < kTwoOpt;
+  if (gm == 0) return 0;
+  unsigned own = __ballot_sync(kFull, best == gm);
+  if (own & (own - 1)) {  // equal gains: the first in scan order
+    const int im = (int)__reduce_min_sync(kFull, best == gm ? (unsigned)bidx : 0xFFFFFFFFu);
+    own = __ballot_sync(kFull, best == gm && bidx == im);
+  }
+  const int wl = __ffs(own) - 1;
+  const int bw = __shfl_sync(kFull, b, wl), bnw = __shfl_sync(kFull, bbn, wl);
+  const int cw = __shfl_sync(kFull, bcode, wl);
+  const int side = cw & 1;
+  if (gm >= kTwoOpt) {
+    mv[0] = side ? p : a;
+    mv[1] = side ? a : s1;
+    mv[2] = side ? bnw : bw;
+    mv[3] = side ? bw : bnw;
+    return gm - kTwoOpt;
+  }
+  const int l = cw >> 2;
+  mv[0] = p; mv[1] = a; mv[2] = l == 1 ? a : (l == 2 ? s1 : s2);
+  mv[3] = l == 1 ? s1 : (l == 2 ? s2 : s3); mv[4] = side ? bnw : bw; mv[5] = side ? bw : bnw;
+  mv[6] = (cw >> 1) & 1;
+  return gm;
 }
 
 // The 3-opt segment exchange of the initial tour (Sec. 4.3: 2-opt and
@@ -409,14 +413,13 @@ __device__ __forceinline__ int64_t eval_or3(const Tour& T, int a, int mv[6]) {
 // way (a segment table that may move to arrays) provide their own overload
 // that picks one concrete representation per call.
 template <class Tour>
-__device__ __forceinline__ void eval_dispatch(const Tour& T, int a, bool do_or, int64_t& g2, int mv2[4],
-                                              int64_t& go, int mvo[7]) {
-  eval_both(T, a, do_or, g2, mv2, go, mvo);
+__device__ __forceinline__ int32_t eval_dispatch(const Tour& T, int a, bool do_or, int (&mv)[8]) {
+  return eval_both(T, a, do_or, mv);
 }
 
 // Applies an Or-opt move {p,a,e,q,u,v,kept} as edge exchanges.
 template <class Tour>
-__device__ __forceinline__ bool apply_or(Tour& T, const int mv[7], LsStats& S) {
+__device__ __forceinline__ bool apply_or(Tour& T, const int* mv, LsStats& S) {
   if (!tour_move2(T, mv[0], mv[1], mv[4], mv[5], S)) return false;  // {p,a},{u,v} -> {p,u},{a,v}
   if (!tour_move2(T, mv[0], mv[4], mv[3], mv[2], S)) return false;  // {p,u},{q,e} -> {p,q},{u,e}
   if (mv[6] && !tour_move2(T, mv[4], mv[2], mv[1], mv[5], S)) return false;  // {u,e},{a,v} -> {u,a},{e,v}
@@ -499,30 +502,21 @@ __device__ __forceinline__ int64_t ls_run(const LsEnv& E, Tour& T, const int32_t
       if (!(f & 2)) ++nlog;
       __syncwarp();
       S.pops++;
-      int mv[4], mvo[7];
-      int64_t g, go;
-      eval_both(T, a, E.oropt != 0, g, mv, go, mvo);
+      int mv[8];
+      const int32_t g = eval_both(T, a, E.oropt != 0, mv);
       if (g > 0) {
-        ok = T.flip(mv[1], mv[2], S);
+        if (mv[7] == 0) {
+          ok = T.flip(mv[1], mv[2], S);
+          S.moves2++;
+        } else {
+          ok = apply_or(T, mv, S);
+          S.movesor++;
+        }
         if (!ok) break;
-        qn = ls_push_warp(E, mv, 4, qh, qn);
+        qn = ls_push_warp(E, mv, mv[7] == 0 ? 4 : 6, qh, qn);
         total += g;
         ++changes;
         ++moves_round;
-        S.moves2++;
-        continue;
-      }
-      if (E.oropt) {
-        g = go;
-        if (g > 0) {
-          ok = apply_or(T, mvo, S);
-          if (!ok) break;
-          qn = ls_push_warp(E, mvo, 6, qh, qn);
-          total += g;
-          ++changes;
-          ++moves_round;
-          S.movesor++;
-        }
       }
     }
     if (!ok || changes >= n || !E.verify || moves_round == 0) break;
@@ -552,7 +546,7 @@ __device__ __forceinline__ int64_t ls_run(const LsEnv& E, Tour& T, const int32_t
 
 // Shared scratch of the block version below.
 struct LsShared {
-  int64_t gain[32];
+  int32_t gain[32];
   int mv[32][8];
   int qh, qn, nlog, changes, moves_round, win, fail;
   int64_t total;
@@ -603,19 +597,12 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, Tour& T, const i
       int idx = qh + w;
       if (idx >= n) idx -= n;
       const int a = E.queue[idx];
-      int mv2[4], mvo[7];
-      int64_t g2, go;
-      eval_dispatch(T, a, E.oropt != 0, g2, mv2, go, mvo);
+      int mv[8];
+      const int32_t g = eval_dispatch(T, a, E.oropt != 0, mv);
       if (lane == 0) {
-        if (g2 > 0) {
-          sh.gain[w] = g2;
-          for (int t = 0; t < 4; ++t) sh.mv[w][t] = mv2[t];
-          sh.mv[w][7] = 0;
-        } else {
-          sh.gain[w] = go > 0 ? go : 0;
-          for (int t = 0; t < 7; ++t) sh.mv[w][t] = mvo[t];
-          sh.mv[w][7] = 1;
-        }
+        sh.gain[w] = g;
+        if (g > 0)
+          for (int t = 0; t < 8; ++t) sh.mv[w][t] = mv[t];
       }
     }
     __syncthreads();

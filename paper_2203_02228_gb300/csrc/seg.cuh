@@ -739,19 +739,14 @@ struct HybTour {
 // evaluation and reversal stay out of line, so that the table's hot loop
 // keeps its registers and a smaller code footprint (spill stores of the
 // per-ant kernel 620 -> 220 bytes, the kernel 3-4 % faster).
-static __device__ __noinline__ void eval_arrays(const ArrTour& T, int a, bool do_or, int64_t& g2, int* mv2,
-                                                int64_t& go, int* mvo) {
-  int m2[4], mo[7];
-  eval_both(T, a, do_or, g2, m2, go, mo);
-  for (int t = 0; t < 4; ++t) mv2[t] = m2[t];
-  for (int t = 0; t < 7; ++t) mvo[t] = mo[t];
+static __device__ __noinline__ int32_t eval_arrays(const ArrTour& T, int a, bool do_or, int* mv) {
+  int m[8];
+  const int32_t g = eval_both(T, a, do_or, m);
+  for (int t = 0; t < 8; ++t) mv[t] = m[t];
+  return g;
 }
-__device__ __forceinline__ void eval_dispatch(const HybTour& T, int a, bool do_or, int64_t& g2, int mv2[4],
-                                              int64_t& go, int mvo[7]) {
-  if (T.arrays())
-    eval_arrays(T.ar, a, do_or, g2, mv2, go, mvo);
-  else
-    eval_both(T.sg, a, do_or, g2, mv2, go, mvo);
+__device__ __forceinline__ int32_t eval_dispatch(const HybTour& T, int a, bool do_or, int (&mv)[8]) {
+  return T.arrays() ? eval_arrays(T.ar, a, do_or, mv) : eval_both(T.sg, a, do_or, mv);
 }
 
 }  // namespace faco

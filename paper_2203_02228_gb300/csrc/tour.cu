@@ -314,28 +314,24 @@ __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int i
       const int my_node = __shfl_sync(kFull, node, w & 31);
       const int my_slot = (base + w) & (kWin - 1);
       if (w < R && ((bmiss >> w) & 1u)) {
-        int mv2[4], mvo[7], mv3[6];
-        int64_t g2, go, g3 = 0;
-        eval_both(T, my_node, oropt != 0, g2, mv2, go, mvo);
+        int mv[8], mv3[6];
+        const int32_t g = eval_both(T, my_node, oropt != 0, mv);
+        int64_t g3 = 0;
         // the 3-opt exchange only when neither 2-opt nor Or-opt improves
-        // (g2, go are the warp's reductions: the branch is warp-uniform)
-        const bool try3 = init3 && !(g2 > 0) && !(go > 0);
+        // (g is the warp's reduction: the branch is warp-uniform)
+        const bool try3 = init3 && g == 0;
         if (try3) g3 = eval_or3(T, my_node, mv3);
         if (lane < k) s_dep[my_slot][1 + lane] = T.pos_of(T.cand(my_node, lane));
         if (lane == 0) {
           s_dep[my_slot][0] = T.pos_of(my_node);
-          if (g2 > 0) {
-            s_gain[my_slot] = g2;
-            for (int t = 0; t < 4; ++t) s_mv[my_slot][t] = mv2[t];
-            s_mv[my_slot][7] = 0;
-          } else if (g3 > 0) {
+          if (g3 > 0) {
             s_gain[my_slot] = g3;
             for (int t = 0; t < 6; ++t) s_mv[my_slot][t] = mv3[t];
             s_mv[my_slot][7] = 2;
           } else {
-            s_gain[my_slot] = go > 0 ? go : 0;
-            for (int t = 0; t < 7; ++t) s_mv[my_slot][t] = mvo[t];
-            s_mv[my_slot][7] = 1;
+            s_gain[my_slot] = g;
+            if (g > 0)
+              for (int t = 0; t < 8; ++t) s_mv[my_slot][t] = mv[t];
           }
           s_any[my_slot] = try3 ? 1 : 0;
           s_node[my_slot] = my_node;
