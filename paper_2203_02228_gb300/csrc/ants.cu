@@ -55,9 +55,9 @@ cudaError_t launch_ants(const Colony& C, const Ants& A, cudaStream_t s) {
   const dim3 grid((A.m + warps - 1) / warps), block(32 * warps);
   const size_t smem = A.smem_vis ? warps * ants_smem_per_warp(C.n, 0, false) : 0;
   if (C.kw == 16)
-    k_ants<16, false><<<grid, block, smem, s>>>(C, A);
+    k_ants<16><<<grid, block, smem, s>>>(C, A);
   else
-    k_ants<32, false><<<grid, block, smem, s>>>(C, A);
+    k_ants<32><<<grid, block, smem, s>>>(C, A);
   return cudaGetLastError();
 }
 
@@ -153,10 +153,10 @@ cudaError_t prepare_ants_kernel(int kw, size_t smem_seg, size_t smem_arr) {
   cudaError_t e;
   if (kw == 16) {
     e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants_blk<16>), smem_seg);
-    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<16, false>), smem_arr);
+    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<16>), smem_arr);
   } else {
     e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants_blk<32>), smem_seg);
-    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<32, false>), smem_arr);
+    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<32>), smem_arr);
   }
   return e;
 }

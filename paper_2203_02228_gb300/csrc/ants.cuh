@@ -166,11 +166,11 @@ struct FbBlock {
 // construction needs this search -- late in the walk, with few nodes left
 // -- and cost several times the scan.)  Must be called by every thread of
 // the block; returns the source position (the same on every thread).
-__device__ __noinline__ int block_nearest(const Colony& C, const uint32_t* vis, FbBlock& fb) {
+__device__ __forceinline__ int block_nearest(int n, const int2* xy, const int32_t* src_route, const int32_t* src_pos,
+                                          DevState* st, const uint32_t* vis, FbBlock& fb) {
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  const int n = C.n;
   const int pc = fb.pc;
-  const int2 xu = C.XYsrc[pc];
+  const int2 xu = xy[pc];
   uint64_t bk = ~0ull;
   int32_t bi = INT_MAX;
   const int words = (n + 31) >> 5;
@@ -180,9 +180,9 @@ __device__ __noinline__ int block_nearest(const Colony& C, const uint32_t* vis, 
     while (fr) {
       const int q = wi * 32 + __ffs(fr) - 1;
       fr &= fr - 1;
-      const uint64_t m = sqdist(xu, C.XYsrc[q]);
+      const uint64_t m = sqdist(xu, xy[q]);
       if (m <= bk) {  // the node id only decides ties
-        const int32_t nd = C.src_route[q];
+        const int32_t nd = src_route[q];
         if (m < bk || nd < bi) {
           bk = m;
           bi = nd;
@@ -209,10 +209,10 @@ __device__ __noinline__ int block_nearest(const Colony& C, const uint32_t* vis, 
   // (the next request reaches the slots only after the barrier that posts
   // it, which every thread passes after these reads)
   if (best_i < 0 || best_i >= n) {  // cannot happen while a node is unvisited
-    if (tid == 0) atomicOr(&C.st->error, kErrInternal);
+    if (tid == 0) atomicOr(&st->error, kErrInternal);
     return pc == 0 ? n - 1 : pc - 1;
   }
-  return C.src_pos[best_i];
+  return src_pos[best_i];
 }
 
 struct Walk {
@@ -224,51 +224,38 @@ struct Walk {
   int first_q;     // source position of route[0]
   int new_edges, nchk;
   int64_t len;     // length of the closed runs and connecting edges
-  int64_t aco, backup, global;
+  int32_t aco, backup, global;
   int64_t fall_ns;  // time in global nearest-unvisited scans
-  bool segs;       // emit a segment table instead of route/pos arrays
-  bool overflow;   // the segment table is full
-  SegTab tab;
+  bool segs;       // emit a list of runs instead of route/pos arrays
+  bool overflow;   // the list is full
+  Seg* runs;       // [cap] the closed runs in tour order
+  int cap, nruns;
 };
 
-// Closes the current run: appends its segment(s) to the table.  The run
-// occupies ant positions [kf - run_len, kf).
+// Closes the current run: appends it to the list (as two runs when it
+// passes the source's end).  The run occupies ant positions
+// [kf - run_len, kf).
 __device__ __forceinline__ void close_run(const Colony& C, Walk& W) {
   if (!W.segs || W.overflow) return;
   const int n = C.n, len = W.run_len, off = W.kf - len;
-  const int S = *W.tab.S;
-  if (S + 2 > W.tab.cap) {
+  const int S = W.nruns;
+  if (S + 2 > W.cap) {
     W.overflow = true;
     return;
   }
+  const int f = W.run_first, rev = W.dir < 0 ? 1 : 0;
+  const int l1 = rev ? f + 1 : n - f;  // nodes before the source's end
+  const bool two = len > l1;
   if (lane_id() == 0) {
-    Seg* sg = W.tab.sg;
-    int add = 1;
-    if (W.dir >= 0) {
-      const int f = W.run_first;
-      if (f + len <= n) {
-        sg[S] = Seg{f, len, off, 0};
-      } else {
-        const int l1 = n - f;
-        sg[S] = Seg{f, l1, off, 0};
-        sg[S + 1] = Seg{0, len - l1, off + l1, 0};
-        add = 2;
-      }
+    if (!rev) {
+      W.runs[S] = Seg{f, two ? l1 : len, off, 0};
+      if (two) W.runs[S + 1] = Seg{0, len - l1, off + l1, 0};
     } else {
-      const int f = W.run_first;
-      if (f - len + 1 >= 0) {
-        sg[S] = Seg{f - len + 1, len, off, 1};
-      } else {
-        const int l1 = f + 1;
-        sg[S] = Seg{0, l1, off, 1};
-        sg[S + 1] = Seg{n - (len - l1), len - l1, off + l1, 1};
-        add = 2;
-      }
+      W.runs[S] = Seg{two ? 0 : f - len + 1, two ? l1 : len, off, 1};
+      if (two) W.runs[S + 1] = Seg{n - (len - l1), len - l1, off + l1, 1};
     }
-    W.tab.A[S] = (uint16_t)S;
-    if (add == 2) W.tab.A[S + 1] = (uint16_t)(S + 1);
-    *W.tab.S = S + add;
   }
+  W.nruns = S + (two ? 2 : 1);
   __syncwarp();
 }
 
@@ -297,10 +284,10 @@ __device__ __forceinline__ void place_run(const Colony& C, int32_t* route, int32
   }
 }
 
-// Backup list, then global nearest unvisited node (warp).  Returns the
-// source position of the chosen node.
-__device__ __noinline__ int fallback_pick(const Colony& C, const uint32_t* vis, int pc, Walk& W, FbBlock* fb) {
-  const int n = C.n, lane = lane_id();
+// First unvisited node of the backup list of source position pc (warp):
+// its source position, or -1.
+__device__ __forceinline__ int backup_pick(const Colony& C, const uint32_t* vis, int pc) {
+  const int lane = lane_id();
   const int u = C.src_route[pc];
   for (int j0 = 0; j0 < C.bl; j0 += 32) {
     const int j = j0 + lane;
@@ -310,35 +297,21 @@ __device__ __noinline__ int fallback_pick(const Colony& C, const uint32_t* vis, 
       if (vis_get(vis, q)) q = -1;
     }
     const unsigned bal = __ballot_sync(kFull, q >= 0);
-    if (bal) {
-      W.backup++;
-      return __shfl_sync(kFull, q, __ffs(bal) - 1);
-    }
+    if (bal) return __shfl_sync(kFull, q, __ffs(bal) - 1);
   }
-  // global nearest unvisited node: rings of grid cells around u, else a
-  // scan of the visited words that skips full ones
-  const uint64_t t0 = global_ns();
-  if (fb) {  // with the whole block (the block kernel: the other warps wait for this)
-    if (lane == 0) {
-      fb->cmd = 1;
-      fb->pc = pc;
-    }
-    __syncwarp();
-    __syncthreads();
-    const int q = block_nearest(C, vis, *fb);
-    W.global++;
-    W.fall_ns += (int64_t)(global_ns() - t0);
-    return q;
-  }
+  return -1;
+}
+
+// The nearest unvisited node of source position pc, by one warp: rings of
+// grid cells around it, else a scan of the visited words that skips full
+// ones.  Returns its source position.
+__device__ __noinline__ int warp_nearest(const Colony& C, const uint32_t* vis, int pc) {
+  const int n = C.n, lane = lane_id();
   const int2 xu = C.XYsrc[pc];
   int qn;
   const int near = ring_nearest(C.cell_src, C.grid, C.cell_start, xu, 24,
                                 [&](const int4& P) { return vis_get(vis, P.x); }, qn);
-  if (near >= 0) {
-    W.global++;
-    W.fall_ns += (int64_t)(global_ns() - t0);
-    return qn;
-  }
+  if (near >= 0) return qn;
   uint64_t bk = ~0ull;
   int32_t bi = INT_MAX;
   const int words = (n + 31) >> 5;
@@ -373,13 +346,37 @@ __device__ __noinline__ int fallback_pick(const Colony& C, const uint32_t* vis, 
     }
   }
   warp_min_key(bk, bi);
-  W.global++;
-  W.fall_ns += (int64_t)(global_ns() - t0);
   if (bi < 0 || bi >= n) {  // cannot happen while a node is unvisited
     if (lane == 0) atomicOr(&C.st->error, kErrInternal);
     return pc == 0 ? n - 1 : pc - 1;
   }
   return C.src_pos[bi];
+}
+
+// Backup list, then the globally nearest unvisited node -- with the whole
+// block when it helps (fb; the other warps wait for this request), else by
+// the warp.  Returns the source position of the chosen node.
+__device__ __forceinline__ int fallback_pick(const Colony& C, const uint32_t* vis, Walk& W, FbBlock* fb) {
+  int q = backup_pick(C, vis, W.pc);
+  if (q >= 0) {
+    W.backup++;
+    return q;
+  }
+  const uint64_t t0 = global_ns();
+  if (fb) {
+    if (lane_id() == 0) {
+      fb->cmd = 1;
+      fb->pc = W.pc;
+    }
+    __syncwarp();
+    __syncthreads();
+    q = block_nearest(C.n, C.XYsrc, C.src_route, C.src_pos, C.st, vis, *fb);
+  } else {
+    q = warp_nearest(C, vis, W.pc);
+  }
+  W.global++;
+  W.fall_ns += (int64_t)(global_ns() - t0);
+  return q;
 }
 
 // One ACO step (already chosen source position q) from the current end.
@@ -454,7 +451,7 @@ __device__ __forceinline__ bool spec_step(const Colony& C, const uint32_t* vis, 
     }
     if (any) {
       const float u = u01(draw(C.seed, (uint32_t)(kf + o), ant, iter, 0));
-      q = c[roulette<KW>(w, u)];
+      q = C.Csrc[(size_t)pt * KW + roulette<KW>(w, u)];  // (not c[]: a local array would spill)
     }
   }
   return valid && any && dir != 0 && q == wrapn(pt + dir, n);
@@ -526,7 +523,7 @@ __device__ __forceinline__ void aco_steps(const Colony& C, int32_t* route, int32
     W.aco += f;
   }
   if (f < nspec && W.kf < n) {
-    if (!anyf) qf = fallback_pick(C, vis, W.pc, W, fb);
+    if (!anyf) qf = fallback_pick(C, vis, W, fb);
     W.aco++;
     place_step(C, route, pos, vis, chk, W, qf);
   }
@@ -558,6 +555,7 @@ __device__ __forceinline__ int64_t construct(const Colony& C, int32_t* route, in
   W.kf = 1; W.pc = q0; W.dir = 0; W.run_first = q0; W.run_len = 1; W.first_q = q0;
   W.new_edges = 0; W.nchk = 0; W.len = 0; W.aco = 0; W.backup = 0; W.global = 0;
   W.overflow = false;
+  W.nruns = 0;
   while (W.kf < n && !W.overflow) {
     if (W.new_edges >= C.min_new_edges) {
       // complete along the source: forward, then backward
@@ -591,46 +589,38 @@ __device__ __forceinline__ int64_t construct(const Colony& C, int32_t* route, in
   return L;
 }
 
-// Writes the table's tour as node ids (source order -> node ids).
-__device__ void seg_materialize(const Colony& C, const SegTab& T, int32_t* route) {
-  const int S = *T.S;
-  const int n = C.n;
+// Writes a list of runs as node ids (warp).
+__device__ void runs_materialize(const Colony& C, const Seg* runs, int S, int32_t* route) {
   for (int r = 0; r < S; ++r) {
-    const Seg s = T.sg[T.A[r]];
-    for (int d = lane_id(); d < s.len; d += 32) {
-      const int q = s.rev ? s.lo + s.len - 1 - d : s.lo + d;
-      const int t = s.off + d;
-      if ((unsigned)q < (unsigned)n && (unsigned)t < (unsigned)n) route[t] = C.src_route[q];
+    const Seg s = runs[r];
+    for (int d = lane_id(); d < s.len; d += 32)
+      route[s.off + d] = C.src_route[s.rev ? s.lo + s.len - 1 - d : s.lo + d];
+  }
+  __syncwarp();
+}
+
+// Writes the table's tour as node ids (warp).
+__device__ void seg_materialize(const Colony& C, const SegView& V, int32_t* route) {
+  for (int r = 0; r < V.S; ++r) {
+    const SegRec s = V.rec(r);
+    for (int q = s.lo + lane_id(); q <= s.hi; q += 32) {
+      const int t = s.pos(q, C.n);
+      if ((unsigned)t < (unsigned)C.n) route[t] = C.src_route[q];
     }
   }
   __syncwarp();
 }
 
-// B = ids by lo (ranks by counting: lo values are distinct); keys.
-__device__ void seg_finish_construction(const SegTab& T) {
-  const int S = *T.S;
-  for (int id = lane_id(); id < S; id += 32) {
-    const int lo = T.sg[id].lo;
-    int r = 0;
-    for (int o = 0; o < S; ++o) r += T.sg[o].lo < lo;
-    T.B[r] = (uint16_t)id;
-  }
-  __syncwarp();
-  segtab_keys(T);
-}
-
 // Array kernel body: one warp runs ant `ant` with explicit route/pos;
-// `mine` is the warp's own shared memory (visited bits, and the segment
-// table when SEGS).
-template <int KW, bool SEGS>
+// `mine` is the warp's own shared memory (visited bits).
+template <int KW>
 __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, int ant, char* mine) {
   const int lane = lane_id();
   if (ant >= A.m) return;
-  if (!SEGS && A.redo && !A.redo[ant]) return;  // array kernel: only the ants the table could not hold
+  if (A.redo && !A.redo[ant]) return;  // only the ants the table could not hold
   const int n = C.n;
   const int words = (n + 31) >> 5;
-  const size_t vis_bytes = ((size_t)words * 4 + 15) & ~(size_t)15;
-  uint32_t* vis = (SEGS || A.smem_vis) ? reinterpret_cast<uint32_t*>(mine) : A.vis_g + (size_t)ant * words;
+  uint32_t* vis = A.smem_vis ? reinterpret_cast<uint32_t*>(mine) : A.vis_g + (size_t)ant * words;
   const uint32_t iter = (uint32_t)(C.st->iter + 1);
   const uint64_t t_start = global_ns();
   int32_t* route = A.route + (size_t)ant * n;
@@ -638,28 +628,15 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
   int32_t* chk = A.chk + (size_t)ant * n;
 
   Walk W;
-  W.segs = SEGS;
-  if (SEGS) {
-    W.tab = segtab_at(mine + vis_bytes, A.seg_cap);
-    if (lane == 0) *W.tab.S = 0;
-    __syncwarp();
-  }
+  W.segs = false;
+  W.runs = nullptr;
+  W.cap = 0;
   W.fall_ns = 0;
   const int64_t pre_len = construct<KW>(C, route, pos, vis, chk, W, (uint32_t)ant, iter);
   const uint64_t t_cons = global_ns();
-  if (SEGS && W.overflow) {
-    if (lane == 0) A.redo[ant] = 1;
-    return;
-  }
-  if (SEGS) seg_finish_construction(W.tab);
   if (A.pre_route) {
-    if (SEGS) {
-      seg_materialize(C, W.tab, A.pre_route + (size_t)ant * n);
-      for (int i = lane; i < W.nchk; i += 32) A.pre_chk[(size_t)ant * n + i] = C.src_route[chk[i]];
-    } else {
-      for (int i = lane; i < n; i += 32) A.pre_route[(size_t)ant * n + i] = route[i];
-      for (int i = lane; i < W.nchk; i += 32) A.pre_chk[(size_t)ant * n + i] = chk[i];
-    }
+    for (int i = lane; i < n; i += 32) A.pre_route[(size_t)ant * n + i] = route[i];
+    for (int i = lane; i < W.nchk; i += 32) A.pre_chk[(size_t)ant * n + i] = chk[i];
     if (lane == 0) {
       A.pre_len[ant] = pre_len;
       A.pre_nchk[ant] = W.nchk;
@@ -669,29 +646,10 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
   LsEnv E{n, C.oropt, C.verify, A.queue + (size_t)ant * n, A.flags + (size_t)ant * n,
           A.logb + (size_t)ant * n};
   LsStats S{0, 0, 0, 0, 0};
-  int64_t gain;
-  if (SEGS) {
-    SegTour T{n, C.k, C.kw, W.tab, C.XYsrc, C.Csrc, C.Dcsrc};
-    gain = C.ls ? ls_run(E, T, chk, W.nchk, S) : 0;
-    if (gain < 0) {  // the table filled up during the search
-      if (lane == 0) A.redo[ant] = 1;
-      return;
-    }
-    // hand the tour over: segments in ant order
-    const int Sn = *W.tab.S;
-    int4* out = A.segs + (size_t)ant * A.seg_cap_ls;
-    for (int r = lane; r < Sn; r += 32) {
-      const Seg s = W.tab.sg[W.tab.A[r]];
-      out[r] = make_int4(s.lo, s.len, s.off, s.rev);
-    }
-    if (lane == 0) A.nseg[ant] = Sn;
-    if (A.keep_tours) seg_materialize(C, W.tab, route);
-  } else {
-    ArrTour T{n, C.k, route, pos, C.xy, C.cand, C.k, C.dcand};
-    gain = C.ls ? ls_run(E, T, chk, W.nchk, S) : 0;
-    if (lane == 0 && A.nseg) A.nseg[ant] = -1;  // tour is in route/pos
-  }
+  ArrTour T{n, C.k, route, pos, C.xy, C.cand, C.k, C.dcand};
+  const int64_t gain = C.ls ? ls_run(E, T, chk, W.nchk, S) : 0;
   if (lane == 0) {
+    if (A.nseg) A.nseg[ant] = -1;  // tour is in route/pos
     A.len[ant] = pre_len - gain;
     if (A.redo) A.redo[ant] = 0;
     int64_t* st = A.stats + (size_t)ant * kNStats;
@@ -700,7 +658,7 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
     st[kStGlobal] += W.global; st[kStCheck] += W.nchk; st[kStPops] += S.pops;
     st[kStMoves2] += S.moves2; st[kStMovesOr] += S.movesor; st[kStFlip] += S.flip;
     st[kStVerify] += S.verify;
-    if (!SEGS && A.segs) st[kStRedo] += 1;
+    if (A.segs) st[kStRedo] += 1;
     st[kStStartNs] = (int64_t)t_start;
     st[kStDurNs] = (int64_t)(global_ns() - t_start);
     st[kStConsNs] = (int64_t)(t_cons - t_start);
@@ -719,25 +677,19 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 constexpr int kAntWarps = 8;
 constexpr int kAntMaxRegs = 64;
 
-__device__ __forceinline__ void st_redo_add(const Ants& A, int ant) {
-  A.stats[(size_t)ant * kNStats + kStRedo] += 1;
-}
-
-
 // ---------------------------------------------------------------------
 // Kernels.  One colony: the Colony and Ants descriptors are kernel
 // parameters.  A batch of colonies: every block reads its (colony, ant)
 // from a block map and the colony's descriptors from device tables into
 // shared memory; the bodies are the same.
 // ---------------------------------------------------------------------
-template <int KW, bool SEGS>
+template <int KW>
 __global__ void __launch_bounds__(128, 1) k_ants(Colony C, Ants A) {
   extern __shared__ __align__(16) char smem[];
   const int wib = threadIdx.x >> 5;
   const int ant = blockIdx.x * (blockDim.x >> 5) + wib;
   const size_t vis_bytes = ((size_t)((C.n + 31) >> 5) * 4 + 15) & ~(size_t)15;
-  const size_t per_warp = SEGS ? vis_bytes + segtab_bytes(A.seg_cap) : (A.smem_vis ? vis_bytes : 0);
-  ants_arr_body<KW, SEGS>(C, A, ant, smem + (size_t)wib * per_warp);
+  ants_arr_body<KW>(C, A, ant, smem + (A.smem_vis ? (size_t)wib * vis_bytes : 0));
 }
 
 template <int KW>
@@ -802,7 +754,7 @@ __global__ void __launch_bounds__(128, MB)
     copy_words(&sC[wib], cols + e.x, sizeof(Colony), wib * 32, 32);
     copy_words(&sA[wib], ants + e.x, sizeof(Ants), wib * 32, 32);
     __syncwarp();
-    ants_arr_body<KW, false>(sC[wib], sA[wib], e.y, smem + (size_t)wib * per_warp);
+    ants_arr_body<KW>(sC[wib], sA[wib], e.y, smem + (size_t)wib * per_warp);
     __syncwarp();
     if (mapped) break;
   }

@@ -192,8 +192,8 @@ __device__ __forceinline__ void best_body(const Colony& C, const Ants& A) {
 }
 
 // The iteration-best tour as explicit route/pos (into tmp): from its
-// segment table (source positions -> node ids of the current source), or
-// from the ant's arrays when it was built with them.  Skipped when neither
+// segments (a thread per source position of the current source), or from
+// the ant's arrays when it was built with them.  Skipped when neither
 // the global best nor the source will take it.
 __device__ __forceinline__ void best_tour_body(const Colony& C, const Ants& A, int t) {
   int32_t* tmp_route = C.tmp_route;
@@ -202,33 +202,30 @@ __device__ __forceinline__ void best_tour_body(const Colony& C, const Ants& A, i
   const DevState* st = C.st;
   if (t >= n || (!st->gb_improved && st->use_gb)) return;
   const int a = st->it_best_ant;
-  int node;
+  int node, at = t;  // the node at tour position `at`
   const int S = A.nseg ? A.nseg[a] : -1;
-  if (S == -1) {  // node ids
+  if (S < 0) {  // arrays, as node ids
     node = A.route[(size_t)a * n + t];
-  } else if (S < 0) {  // source positions
-    node = C.src_route[A.route[(size_t)a * n + t]];
-  } else {
-    const int4* sg = A.segs + (size_t)a * A.seg_cap_ls;
+  } else {  // t is a source position: its segment's map gives its tour position
+    const int2* sg = A.segs + (size_t)a * A.seg_cap_ls;
     int lo = 0, hi = S - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (sg[mid].z <= t)
+      if (sg[mid].x <= t)
         lo = mid;
       else
         hi = mid - 1;
     }
-    const int4 s = sg[lo];
-    const int d = t - s.z;
-    int q = s.w ? s.x + s.y - 1 - d : s.x + d;
-    if ((unsigned)q >= (unsigned)n) {  // inconsistent table: a library bug, flagged
+    const int map = sg[lo].y, base = map & 0x7fffffff;
+    at = wrapn(map < 0 ? base - t : base + t, n);
+    if ((unsigned)at >= (unsigned)n) {  // inconsistent table: a library bug, flagged
       atomicOr(&C.st->error, kErrInternal);
-      q = 0;
+      at = 0;
     }
-    node = C.src_route[q];
+    node = C.src_route[t];
   }
-  tmp_route[t] = node;
-  tmp_pos[node] = t;
+  tmp_route[at] = node;
+  tmp_pos[node] = at;
 }
 
 // Global best <- iteration best when improved; source <- global best or

@@ -132,7 +132,8 @@ struct Ants {
   int32_t seg_cap;       // segments per ant table during construction (0: arrays only)
   int32_t seg_cap_ls;    // during the local search, which also takes the visited bits' room;
                          // the stride of segs
-  int4* segs;            // [m][seg_cap] final tours as (lo, len, off, rev), or null
+  int2* segs;            // [m][seg_cap_ls] final tours as segments in source order: first node and
+                         // map to tour positions (seg.cuh), or null
   int32_t* nseg;         // [m] segment count, -1 when the tour is in route/pos
   int32_t* redo;         // [m] 1: the table overflowed, the array kernel redoes the ant
   int32_t keep_tours;    // 1: also write every tour to route[] (inspection)
@@ -239,12 +240,10 @@ __device__ __forceinline__ int32_t euc2d_near(int2 a, int2 b, bool& big) {
   return d + (q > d ? 1 : 0) - (q + d < min(d, 1) ? 1 : 0);
 }
 
-static __device__ __noinline__ int32_t euc2d_far(int2 a, int2 b) { return euc2d_m(sqdist(a, b)); }
-
 __device__ __forceinline__ int32_t euc2d(int2 a, int2 b) {
   bool big = false;
   const int32_t d = euc2d_near(a, b, big);
-  return big ? euc2d_far(a, b) : d;
+  return big ? euc2d_m(sqdist(a, b)) : d;
 }
 
 // ---------------------------------------------------------------------
@@ -324,18 +323,6 @@ __device__ __forceinline__ void warp_max_gain(int32_t& g, int32_t& idx) {
   const int32_t gm = __reduce_max_sync(kFull, g);
   idx = (int32_t)__reduce_min_sync(kFull, g == gm ? (unsigned)idx : 0xFFFFFFFFu);
   g = gm;
-}
-
-__device__ __forceinline__ void warp_max_gain(int64_t& g, int32_t& idx) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const int64_t g2 = shfl64_xor(g, o);
-    const int32_t i2 = __shfl_xor_sync(kFull, idx, o);
-    if (g2 > g || (g2 == g && i2 < idx)) {
-      g = g2;
-      idx = i2;
-    }
-  }
 }
 
 __device__ __forceinline__ int wrapn(int x, int n) {  // x in (-n, 2n)

@@ -45,7 +45,8 @@ struct LsEnv {
 };
 
 struct LsStats {
-  int64_t pops, moves2, movesor, flip, verify;
+  int32_t pops, moves2, movesor, verify;
+  int64_t flip;
   int64_t t_eval, t_confirm, t_flip, t_push;  // device ns per phase (block search)
 };
 
@@ -217,16 +218,8 @@ __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, i
     cu = xp;
     cv = x3;
   }
-  const int32_t cst = euc2d(cu, cv);
-  const int d_as = __shfl_sync(kFull, cst, 0), d_ap = __shfl_sync(kFull, cst, 1);
-  // gains in 32 bits: each is a signed sum of at most six EUC_2D costs of
-  // coordinates below 2^24 (each cost below 2^25)
-  int32_t rem1 = 0, rem2 = 0, rem3 = 0;
-  if (do_or) {
-    rem1 = d_ap + d_as - __shfl_sync(kFull, cst, 2);
-    rem2 = d_ap + __shfl_sync(kFull, cst, 3) - __shfl_sync(kFull, cst, 4);
-    rem3 = d_ap + __shfl_sync(kFull, cst, 5) - __shfl_sync(kFull, cst, 6);
-  }
+  bool big = false;
+  int32_t cst = euc2d_near(cu, cv, big);
   // the lane's best move: a gaining 2-opt move counts kTwoOpt more than its
   // gain, so that it beats every Or-opt move; code = l * 4 + orientation * 2
   // + side (l = 0: 2-opt), idx = its place in the sequential scan
@@ -238,7 +231,6 @@ __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, i
     const int side = two ? pass : (lane >> 4);
     const int bn = pass == 0 ? bn0 : bn1;
     const int2 xbn = pass == 0 ? xbn0 : xbn1;
-    bool big = false;
     int32_t c_bn = euc2d_near(xb, xbn, big);   // d(b, bn)
     int32_t c_n1 = euc2d_near(xbn, x1, big);   // d(bn, s1)
     int32_t c_np = euc2d_near(xbn, xp, big);   // d(bn, p)
@@ -249,16 +241,30 @@ __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, i
       c_b2 = euc2d_near(xb, x2, big);
       c_n2 = euc2d_near(xbn, x2, big);
     }
-    if (__any_sync(kFull, big)) {  // an edge of 2^21 or more: the exact steps
-      c_bn = euc2d_far(xb, xbn);
-      c_n1 = euc2d_far(xbn, x1);
-      c_np = euc2d_far(xbn, xp);
-      if (do_or) {
-        c_na = euc2d_far(xbn, xa);
-        c_b1 = euc2d_far(xb, x1);
-        c_b2 = euc2d_far(xb, x2);
-        c_n2 = euc2d_far(xbn, x2);
+    if (__any_sync(kFull, big)) {  // an edge of 2^21 or more: the exact steps, one cost after the other
+#pragma unroll 1
+      for (int j = 0; j < 8; ++j) {
+        const int2 u = j == 7 ? cu : ((j == 0 || j == 4 || j == 5) ? xb : xbn);
+        const int2 t = j == 7 ? cv : j == 0 ? xbn : (j == 1 || j == 4) ? x1 : j == 2 ? xp : j == 3 ? xa : x2;
+        const int32_t d = euc2d_m(sqdist(u, t));
+        if (j == 0) c_bn = d;
+        if (j == 1) c_n1 = d;
+        if (j == 2) c_np = d;
+        if (j == 3) c_na = d;
+        if (j == 4) c_b1 = d;
+        if (j == 5) c_b2 = d;
+        if (j == 6) c_n2 = d;
+        if (j == 7) cst = d;
       }
+    }
+    const int d_as = __shfl_sync(kFull, cst, 0), d_ap = __shfl_sync(kFull, cst, 1);
+    // gains in 32 bits: each is a signed sum of at most six EUC_2D costs of
+    // coordinates below 2^24 (each cost below 2^25)
+    int32_t rem1 = 0, rem2 = 0, rem3 = 0;
+    if (do_or) {
+      rem1 = d_ap + d_as - __shfl_sync(kFull, cst, 2);
+      rem2 = d_ap + __shfl_sync(kFull, cst, 3) - __shfl_sync(kFull, cst, 4);
+      rem3 = d_ap + __shfl_sync(kFull, cst, 5) - __shfl_sync(kFull, cst, 6);
     }
     int32_t v = 0;
     int code = 0;
@@ -409,14 +415,6 @@ __device__ __forceinline__ int64_t eval_or3(const Tour& T, int a, int mv[6]) {
   return g;
 }
 
-// Evaluation from a on any tour; representations that can change on the
-// way (a segment table that may move to arrays) provide their own overload
-// that picks one concrete representation per call.
-template <class Tour>
-__device__ __forceinline__ int32_t eval_dispatch(const Tour& T, int a, bool do_or, int (&mv)[8]) {
-  return eval_both(T, a, do_or, mv);
-}
-
 // Applies an Or-opt move {p,a,e,q,u,v,kept} as edge exchanges.
 template <class Tour>
 __device__ __forceinline__ bool apply_or(Tour& T, const int* mv, LsStats& S) {
@@ -424,16 +422,6 @@ __device__ __forceinline__ bool apply_or(Tour& T, const int* mv, LsStats& S) {
   if (!tour_move2(T, mv[0], mv[4], mv[3], mv[2], S)) return false;  // {p,u},{q,e} -> {p,q},{u,e}
   if (mv[6] && !tour_move2(T, mv[4], mv[2], mv[1], mv[5], S)) return false;  // {u,e},{a,v} -> {u,a},{e,v}
   return true;
-}
-
-// apply_or called rather than inlined in the block search's round loop
-// (about one move in six is an Or-opt move): the loop keeps a smaller code
-// footprint and fewer spills (per-ant kernel 1.6 % faster).
-template <class Tour>
-__device__ __noinline__ bool apply_or_call(Tour& T, const int* mv, LsStats& S) {
-  int m[7];
-  for (int t = 0; t < 7; ++t) m[t] = mv[t];
-  return apply_or(T, m, S);
 }
 
 // Queue the np (<= 32) nodes x[0..np) in order, each only if it is not
@@ -542,140 +530,6 @@ __device__ __forceinline__ int64_t ls_run(const LsEnv& E, Tour& T, const int32_t
   for (int i = lane; i < nlog; i += 32) E.flags[E.logb[i]] = 0;
   __syncwarp();
   return ok ? total : -1;
-}
-
-// Shared scratch of the block version below.
-struct LsShared {
-  int32_t gain[32];
-  int mv[32][8];
-  int qh, qn, nlog, changes, moves_round, win, fail;
-  int64_t total;
-};
-
-// The same search run by a block of W warps on one tour: each round, warp w
-// evaluates the w-th queued node; entries are popped in queue order up to
-// and including the first one whose evaluation found a move, which warp 0
-// applies.  Nothing changes the tour between the confirmed evaluations, so
-// the result equals popping one node at a time.  Must be called by every
-// thread of the block.  Returns the gain, or -1 (capacity).
-template <class Tour>
-__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, Tour& T, const int32_t* init, int ninit,
-                                                LsStats& S, LsShared& sh) {
-  const int n = E.n, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int W = blockDim.x >> 5;
-  for (int i = tid; i < ninit; i += blockDim.x) {
-    const int x = init[i];
-    E.queue[i] = x;
-    E.flags[x] = 1;
-  }
-  if (tid == 0) {
-    sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.fail = 0;
-    sh.total = 0;
-  }
-  __syncthreads();
-  for (;;) {
-    const int qh = sh.qh, qn = sh.qn;
-    if (qn == 0 || sh.changes >= n || sh.fail) {
-      if (sh.fail || sh.changes >= n || !E.verify || sh.moves_round == 0) break;
-      const int nl = sh.nlog;  // verify round: queue again the nodes popped
-      for (int i = tid; i < nl; i += blockDim.x) {
-        const int x = E.logb[i];
-        E.queue[i] = x;
-        E.flags[x] = 1;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        sh.qh = 0; sh.qn = nl; sh.nlog = 0; sh.moves_round = 0;
-      }
-      if (w == 0) S.verify++;
-      __syncthreads();
-      continue;
-    }
-    const int R = qn < W ? qn : W;
-    const uint64_t t0 = (w == 0) ? global_ns() : 0;
-    if (w < R) {
-      int idx = qh + w;
-      if (idx >= n) idx -= n;
-      const int a = E.queue[idx];
-      int mv[8];
-      const int32_t g = eval_dispatch(T, a, E.oropt != 0, mv);
-      if (lane == 0) {
-        sh.gain[w] = g;
-        if (g > 0)
-          for (int t = 0; t < 8; ++t) sh.mv[w][t] = mv[t];
-      }
-    }
-    __syncthreads();
-    if (w == 0) {
-      const uint64_t t1 = global_ns();
-      S.t_eval += (int64_t)(t1 - t0);
-      const unsigned bal = __ballot_sync(kFull, lane < R && sh.gain[lane] > 0);
-      const int first = bal ? __ffs(bal) - 1 : R;
-      const int cnt = bal ? first + 1 : R;  // queue entries popped this round
-      int a = -1;
-      bool first_pop = false;
-      if (lane < cnt) {
-        int idx = qh + lane;
-        if (idx >= n) idx -= n;
-        a = E.queue[idx];
-        const uint8_t f = E.flags[a];
-        first_pop = !(f & 2);
-        E.flags[a] = (uint8_t)((f & ~1) | 2);
-      }
-      const unsigned fb = __ballot_sync(kFull, first_pop);
-      if (first_pop) E.logb[sh.nlog + __popc(fb & ((1u << lane) - 1u))] = a;
-      S.pops += cnt;
-      __syncwarp();
-      int qh2 = qh + cnt;
-      if (qh2 >= n) qh2 -= n;
-      int qn2 = qn - cnt;
-      const uint64_t t2 = global_ns();
-      S.t_confirm += (int64_t)(t2 - t1);
-      if (bal) {  // apply the first move found, queue its endpoints
-        int mv[8];
-        for (int t = 0; t < 8; ++t) mv[t] = sh.mv[first][t];
-        bool ok;
-        if (mv[7] == 0) {
-          ok = T.flip(mv[1], mv[2], S);
-          S.moves2++;
-        } else {
-          ok = apply_or_call(T, mv, S);
-          S.movesor++;
-        }
-        const uint64_t t3 = global_ns();
-        S.t_flip += (int64_t)(t3 - t2);
-        if (!ok) {
-          if (lane == 0) sh.fail = 1;
-        } else {
-          qn2 = ls_push_warp(E, mv, mv[7] == 0 ? 4 : 6, qh2, qn2);
-          if (lane == 0) {
-            sh.total += sh.gain[first];
-            sh.changes++;
-            sh.moves_round++;
-          }
-        }
-        __syncwarp();
-        S.t_push += (int64_t)(global_ns() - t3);
-      }
-      if (lane == 0) {
-        sh.nlog += __popc(fb);
-        sh.qh = qh2;
-        sh.qn = qn2;
-      }
-      __syncwarp();
-    }
-    __syncthreads();
-  }
-  __syncthreads();
-  const int qh = sh.qh, qn = sh.qn, nl = sh.nlog;
-  for (int t = tid; t < qn; t += blockDim.x) {
-    int i = qh + t;
-    if (i >= n) i -= n;
-    E.flags[E.queue[i]] = 0;
-  }
-  for (int i = tid; i < nl; i += blockDim.x) E.flags[E.logb[i]] = 0;
-  __syncthreads();
-  return sh.fail ? -1 : sh.total;
 }
 
 }  // namespace faco

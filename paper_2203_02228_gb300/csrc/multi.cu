@@ -274,7 +274,7 @@ void antset_layout(AntSet& a, const Group& g, int m, size_t smem_blk, int seg_mo
   for (int i = 0; i < C; ++i) {
     a.cap[i] = ant_cap(g.n[i], smem_blk, seg_mode);
     a.hA[i].seg_cap_ls = ants_seg_cap_ls(g.n[i], a.cap[i]);
-    a.hA[i].segs = B.take<int4>((size_t)m * (a.cap[i] > 0 ? a.hA[i].seg_cap_ls : 1));
+    a.hA[i].segs = B.take<int2>((size_t)m * (a.cap[i] > 0 ? a.hA[i].seg_cap_ls : 1));
   }
   for (int i = 0; i < C; ++i) {
     Ants& A = a.hA[i];

@@ -3,20 +3,26 @@
 // After focused construction (Alg 2) an ant's tour is a concatenation of a
 // few runs of the source solution; the local search (Alg 3) then changes
 // the tour by reversals.  Instead of materialising route[]/pos[] arrays of
-// n entries per ant, a warp keeps the tour as a table of segments in shared
-// memory: segment id covers source positions [lo, lo+len) and ant positions
-// [off, off+len), traversed upwards (rev = 0) or downwards (rev = 1) in the
-// source.  Nodes are named by their source position.  Two orders index the
-// table: A (ids by ant position, A[0] at position 0) and B (ids by lo).
-// Segments never straddle ant position 0 nor the source's end, so every
-// lookup is a binary search; the inverse orders (rankA, rankB: the rank of
-// each id) make every lookup by id direct.  A reversal of ant positions
-// i..j splits the segments at i and j+1, reverses that part of A and flips
-// each segment's direction -- exactly the array reversal, entry for entry,
-// in O(segments).
-// Neighbouring segments that continue each other are merged back.  When the
-// table is full the operation reports failure and the caller redoes the ant
-// with explicit arrays (same result, more memory traffic).
+// n entries per ant, a block keeps the tour as a table of segments in shared
+// memory.  Nodes are named by their source position; the segments tile
+// 0..n-1, so one sorted array of boundaries describes them all: boundary r
+// is the first node lo[r] of segment r, which ends before lo[r + 1]
+// (lo[S] = n).  Per boundary the table keeps
+//   - br: the segment's map from node to tour position, base + q (bit 31
+//     clear: the tour walks it upwards) or base - q (bit 31 set), modulo n;
+//   - nb: the tour neighbours across the boundary, x = that of lo[r] outside
+//     segment r, y = that of lo[r] - 1 outside segment r - 1.
+// A tour neighbour is one search by node, then q + 1, q - 1 or a stored
+// neighbour; no order by tour position is needed.  A reversal of positions
+// i..j maps base to i + j - base and flips bit 31 in every segment inside
+// the span, adds a boundary at each cut that falls inside a segment, drops
+// the boundaries between segments that now continue each other, and sets the
+// four neighbours of the two new edges -- exactly the array reversal.  Since
+// a split part keeps its map and a merge keeps either part's, one pass that
+// copies the table into its second buffer does all of it: segments may run
+// across tour position 0, so no span is a special case.
+// When the table is full the reversal reports failure and the ant is redone
+// on explicit arrays by the array kernel (same result, more memory traffic).
 #pragma once
 
 #include "common.cuh"
@@ -24,49 +30,28 @@
 
 namespace faco {
 
+// A run as construction emits it: source positions [lo, lo + len), tour
+// positions [off, off + len), walked downwards when rev.
 struct Seg {
   int32_t lo, len, off, rev;
 };
 
-// Shared-memory table of one warp.
+// Shared memory of a table of `cap` segments: two buffers of cap + 1
+// boundaries, 16 bytes each, then the count and the buffer in use.
+constexpr size_t kSegBytes = 2 * (sizeof(int2) + 2 * sizeof(int32_t));
+static_assert(kSegBytes == 2 * sizeof(Seg), "construction's list of runs takes one buffer's room");
+__host__ __device__ constexpr size_t segtab_bytes(int cap) { return (size_t)(cap + 1) * kSegBytes + 16; }
+
 struct SegTab {
-  Seg* sg;           // [cap] segments by id (ids 0..S-1)
-  uint16_t* A;       // [cap] ids in ant order
-  uint16_t* B;       // [cap] ids in source order
-  int32_t* offA;     // [cap] sg[A[r]].off
-  int32_t* loB;      // [cap] sg[B[r]].lo
-  uint16_t* tmp;     // [2 * cap + 2] scratch
-  uint16_t* rankA;   // [cap] rank in A of each id
-  uint16_t* rankB;   // [cap] rank in B of each id
-  int32_t* S;        // segment count (shared)
+  char* mem;         // buffers 0 and 1
+  int32_t* hdr;      // [0] segments, [1] buffer in use
   int cap;
 };
 
-// bytes of shared memory per segment, and per table of `cap` segments
-constexpr size_t kSegBytes = sizeof(Seg) + 6 * sizeof(uint16_t) + 2 * sizeof(int32_t);
-__host__ __device__ constexpr size_t segtab_bytes(int cap) {
-  return (size_t)cap * kSegBytes + 2 * sizeof(uint16_t) + 16;
-}
-
 __device__ __forceinline__ SegTab segtab_at(char* base, int cap) {
   SegTab T;
-  T.sg = reinterpret_cast<Seg*>(base);
-  char* p = base + (size_t)cap * sizeof(Seg);
-  T.offA = reinterpret_cast<int32_t*>(p);
-  p += (size_t)cap * sizeof(int32_t);
-  T.loB = reinterpret_cast<int32_t*>(p);
-  p += (size_t)cap * sizeof(int32_t);
-  T.A = reinterpret_cast<uint16_t*>(p);
-  p += (size_t)cap * sizeof(uint16_t);
-  T.B = reinterpret_cast<uint16_t*>(p);
-  p += (size_t)cap * sizeof(uint16_t);
-  T.tmp = reinterpret_cast<uint16_t*>(p);
-  p += (size_t)(2 * cap + 2) * sizeof(uint16_t);
-  T.rankA = reinterpret_cast<uint16_t*>(p);
-  p += (size_t)cap * sizeof(uint16_t);
-  T.rankB = reinterpret_cast<uint16_t*>(p);
-  p += (size_t)cap * sizeof(uint16_t);
-  T.S = reinterpret_cast<int32_t*>((reinterpret_cast<uintptr_t>(p) + 3) & ~uintptr_t(3));
+  T.mem = base;
+  T.hdr = reinterpret_cast<int32_t*>(base + (size_t)(cap + 1) * kSegBytes);
   T.cap = cap;
   return T;
 }
@@ -78,675 +63,446 @@ __host__ __device__ constexpr int segtab_cap_ls(size_t vis_bytes, int cap) {
   return cap + (int)((vis_bytes / kSegBytes) & ~(size_t)31);
 }
 
-// Moves the table `from` (placed after the visited bits) to `to` (placed at
-// the start of the same shared memory, larger capacity), with the whole
-// block.  Every array lies lower in `to` than in `from`, by at least the
-// room gained, so copying each array in increasing index order -- all of a
-// chunk's reads before its writes -- never overwrites an entry not yet
-// read.  The scratch array is not copied.
-__device__ __forceinline__ void seg_relayout(const SegTab& from, const SegTab& to) {
-  const int S = *from.S;
-  const int t = threadIdx.x, T = blockDim.x;
-  __syncthreads();
-  for (int c = 0; c < S; c += T) {
-    const int r = c + t;
-    Seg v{0, 0, 0, 0};
-    if (r < S) v = from.sg[r];
-    __syncthreads();
-    if (r < S) to.sg[r] = v;
-    __syncthreads();
-  }
-  for (int c = 0; c < S; c += T) {
-    const int r = c + t;
-    int32_t a = 0, b = 0;
-    if (r < S) {
-      a = from.offA[r];
-      b = from.loB[r];
-    }
-    __syncthreads();
-    if (r < S) {
-      to.offA[r] = a;
-      to.loB[r] = b;
-    }
-    __syncthreads();
-  }
-  for (int c = 0; c < S; c += T) {
-    const int r = c + t;
-    uint16_t a = 0, b = 0, k = 0, kb = 0;
-    if (r < S) {
-      a = from.A[r];
-      b = from.B[r];
-      k = from.rankA[r];
-      kb = from.rankB[r];
-    }
-    __syncthreads();
-    if (r < S) {
-      to.A[r] = a;
-      to.B[r] = b;
-      to.rankA[r] = k;
-      to.rankB[r] = kb;
-    }
-    __syncthreads();
-  }
-  if (t == 0) *to.S = S;
-  __syncthreads();
+// Construction's list of runs: the last cap * 16 bytes of the shared memory
+// (`total` bytes) that holds the visited bits and a table of `cap` segments.
+// It lies behind the visited bits, and behind buffer 0 of the larger table
+// that the local search lays over both.
+__device__ __forceinline__ Seg* segtab_runs(char* smem, size_t vis_bytes, int cap) {
+  return reinterpret_cast<Seg*>(smem + vis_bytes + segtab_bytes(cap) - (size_t)cap * sizeof(Seg));
 }
 
-// Largest r in [0, S) with key[r] <= v (key ascending, key[0] <= v).
-__device__ __forceinline__ int bsearch_le(const int32_t* key, int S, int v) {
-  int lo = 0, hi = S - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (key[mid] <= v)
-      lo = mid;
-    else
-      hi = mid - 1;
+// One segment.
+struct SegRec {
+  int lo, hi, base, nlo, nhi;  // nlo, nhi: tour neighbours of lo and hi outside the segment
+  bool rev;
+  // the next node towards higher (else lower) source positions, or across
+  // the segment's end
+  __device__ __forceinline__ int step(int q, bool up) const {
+    return up ? (q < hi ? q + 1 : nhi) : (q > lo ? q - 1 : nlo);
   }
-  return lo;
-}
+  __device__ __forceinline__ bool inside(int q, bool up) const { return up ? q < hi : q > lo; }
+  __device__ __forceinline__ int pos(int q, int n) const { return wrapn(rev ? base - q : base + q, n); }
+};
 
-// The same search by a whole warp for one (warp-uniform) value: each level
-// compares 32 keys spaced evenly over the remaining range and keeps the
-// last one <= v, so a table of up to 1,024 keys takes two shared-memory
-// round trips instead of ten dependent ones.  Every lane gets the rank.
-__device__ __forceinline__ int bsearch_le_warp(const int32_t* key, int S, int v) {
-  const int lane = lane_id();
-  int lo = 0, len = S;  // the answer lies in [lo, lo + len); key[lo] <= v
-  while (len > 1) {
-    const int st = (len + 31) >> 5;
-    const bool le = lane * st < len && key[lo + lane * st] <= v;
-    const unsigned b = __ballot_sync(kFull, le);
-    const int L = b ? 31 - __clz(b) : 0;
-    lo += L * st;
-    len = min(st, len - L * st);
-  }
-  return lo;
-}
-
-// Insert id (source start lo) at index r of B/loB, arrays of S entries;
-// rankB follows (warp-collective).
-__device__ __forceinline__ void ins_B(const SegTab& T, int S, int r, int id, int32_t lo) {
-  const int lane = lane_id();
-  for (int e = S - 1; e >= r; e -= 32) {
-    const int idx = e - lane;
-    uint16_t v = 0;
-    int32_t k = 0;
-    if (idx >= r) {
-      v = T.B[idx];
-      k = T.loB[idx];
-    }
-    __syncwarp();
-    if (idx >= r) {
-      T.B[idx + 1] = v;
-      T.loB[idx + 1] = k;
-      T.rankB[v] = (uint16_t)(idx + 1);
-    }
-    __syncwarp();
-  }
-  if (lane == 0) {
-    T.B[r] = (uint16_t)id;
-    T.loB[r] = lo;
-    T.rankB[id] = (uint16_t)r;
-  }
-  __syncwarp();
-}
-
-// Rebuild the search keys and the inverse orders from the orders
-// (warp-collective).
-__device__ __forceinline__ void segtab_keys(const SegTab& T) {
-  const int S = *T.S;
-  for (int r = lane_id(); r < S; r += 32) {
-    const int ida = T.A[r], idb = T.B[r];
-    T.offA[r] = T.sg[ida].off;
-    T.rankA[ida] = (uint16_t)r;
-    T.loB[r] = T.sg[idb].lo;
-    T.rankB[idb] = (uint16_t)r;
-  }
-  __syncwarp();
-}
-
-// The two inserts of a split in one pass: (idA, keyA) at index rA of
-// A/offA and (idB, keyB) at index rB of B/loB, both arrays of S entries;
-// rankA and rankB follow (warp-collective).
-__device__ __forceinline__ void ins2_both(const SegTab& T, int S, int rA, int idA, int32_t keyA, int rB, int idB,
-                                          int32_t keyB) {
-  const int lane = lane_id();
-  const int lo = rA < rB ? rA : rB;
-  for (int e = S - 1; e >= lo; e -= 32) {
-    const int idx = e - lane;
-    uint16_t va = 0, vb = 0;
-    int32_t ka = 0, kb = 0;
-    if (idx >= rA) {
-      va = T.A[idx];
-      ka = T.offA[idx];
-    }
-    if (idx >= rB) {
-      vb = T.B[idx];
-      kb = T.loB[idx];
-    }
-    __syncwarp();
-    if (idx >= rA) {
-      T.A[idx + 1] = va;
-      T.offA[idx + 1] = ka;
-      T.rankA[va] = (uint16_t)(idx + 1);
-    }
-    if (idx >= rB) {
-      T.B[idx + 1] = vb;
-      T.loB[idx + 1] = kb;
-      T.rankB[vb] = (uint16_t)(idx + 1);
-    }
-    __syncwarp();
-  }
-  if (lane == 0) {
-    T.A[rA] = (uint16_t)idA;
-    T.offA[rA] = keyA;
-    T.rankA[idA] = (uint16_t)rA;
-    T.B[rB] = (uint16_t)idB;
-    T.loB[rB] = keyB;
-    T.rankB[idB] = (uint16_t)rB;
-  }
-  __syncwarp();
-}
-
-// The two removals of a merge in one pass: index rA of A/offA and index rB
-// of B/loB, arrays of S entries; rankA and rankB follow (warp-collective).
-__device__ __forceinline__ void del_both(const SegTab& T, int S, int rA, int rB) {
-  const int lane = lane_id();
-  for (int e = (rA < rB ? rA : rB) + 1; e < S; e += 32) {
-    const int idx = e + lane;
-    const bool da = idx > rA && idx < S, db = idx > rB && idx < S;
-    uint16_t va = 0, vb = 0;
-    int32_t ka = 0, kb = 0;
-    if (da) {
-      va = T.A[idx];
-      ka = T.offA[idx];
-    }
-    if (db) {
-      vb = T.B[idx];
-      kb = T.loB[idx];
-    }
-    __syncwarp();
-    if (da) {
-      T.A[idx - 1] = va;
-      T.offA[idx - 1] = ka;
-      T.rankA[va] = (uint16_t)(idx - 1);
-    }
-    if (db) {
-      T.B[idx - 1] = vb;
-      T.loB[idx - 1] = kb;
-      T.rankB[vb] = (uint16_t)(idx - 1);
-    }
-    __syncwarp();
-  }
-}
-
-// Ensure a segment starts at ant position t (0 < t < n), given the id of
-// the segment that holds t.  Keys and ranks are current on entry and on
-// exit.  Returns the id of the segment that starts at t (id itself when t
-// is already its first position, else the new id, which takes the part
-// from t on), or -1 when the table is full.
-static __device__ __noinline__ int seg_split(const SegTab& T, int t, int id) {
-  const int S = *T.S;
-  const Seg s = T.sg[id];
-  if (s.off == t) return id;
-  if (S >= T.cap) return -1;
-  const int d = t - s.off;
-  const int nid = S;
-  const int r = T.rankA[id], rb = T.rankB[id];
-  __syncwarp();
-  if (lane_id() == 0) {
-    if (!s.rev) {
-      T.sg[nid] = Seg{s.lo + d, s.len - d, t, 0};
-      T.sg[id].len = d;
-    } else {
-      T.sg[nid] = Seg{s.lo, s.len - d, t, 1};
-      T.sg[id].lo = s.lo + s.len - d;
-      T.sg[id].len = d;
-    }
-  }
-  __syncwarp();
-  if (!s.rev) {
-    ins2_both(T, S, r + 1, nid, t, rb + 1, nid, s.lo + d);
-  } else {  // nid keeps the low end: it goes before id, whose lo moved up
-    ins2_both(T, S, r + 1, nid, t, rb, nid, s.lo);
-    if (lane_id() == 0) T.loB[rb + 1] = s.lo + s.len - d;
-  }
-  if (lane_id() == 0) *T.S = S + 1;
-  __syncwarp();
-  return nid;
-}
-
-// Merge ant ranks r and r+1 if the second continues the first in the
-// source (r + 1 > 0, so never across ant position 0).  Keys and ranks stay
-// current.
-static __device__ __noinline__ void seg_merge_at(const SegTab& T, int r) {
-  const int S = *T.S;
-  if (r < 0 || r + 1 >= S) return;
-  const int ia = T.A[r], ib = T.A[r + 1];
-  const Seg a = T.sg[ia], b = T.sg[ib];
-  if (!(a.rev == b.rev && (a.rev ? (b.lo + b.len == a.lo) : (a.lo + a.len == b.lo)))) return;
-  const int rbb = T.rankB[ib];
-  __syncwarp();
-  if (lane_id() == 0) {
-    T.sg[ia].len = a.len + b.len;
-    if (a.rev) T.sg[ia].lo = b.lo;
-  }
-  __syncwarp();
-  del_both(T, S, r + 1, rbb);
-  if (a.rev && lane_id() == 0) T.loB[rbb] = b.lo;  // a slid down to b's rank and took its lo
-  __syncwarp();
-  // free id ib: move the last id into its slot
-  const int last = S - 1;
-  if (ib != last) {
-    const Seg sl = T.sg[last];
-    const int ra = T.rankA[last], rl = T.rankB[last];
-    __syncwarp();
-    if (lane_id() == 0) {
-      T.sg[ib] = sl;
-      T.A[ra] = (uint16_t)ib;
-      T.rankA[ib] = (uint16_t)ra;
-      T.B[rl] = (uint16_t)ib;
-      T.rankB[ib] = (uint16_t)rl;
-    }
-  }
-  if (lane_id() == 0) *T.S = S - 1;
-  __syncwarp();
-}
-
-// Tour over the segment table (nodes = source positions).
-struct SegTour {
-  int n, k, kw;
-  SegTab T;
+// The table's current buffer, and the tour over it (nodes = source
+// positions).  Taken anew after every reversal.
+struct SegView {
+  int n, k, kw, S;
+  const int2* nb;
+  const int32_t* lo;
+  const int32_t* br;
   const int2* xy;       // coordinates by source position
   const int32_t* cn;    // candidate source positions by source position [n][kw]
   const int32_t* cd;    // their EUC_2D costs, same layout
 
-  // Lookups stay in [0, n) even if the table were inconsistent (which would
-  // be a library bug: it is flagged and shows up as a wrong tour, not as an
-  // out-of-range access).
-  __device__ __forceinline__ int pos_of(int q) const {
-    const int r = bsearch_le(T.loB, *T.S, q);
-    const Seg s = T.sg[T.B[r]];
-    const int t = s.off + (s.rev ? s.lo + s.len - 1 - q : q - s.lo);
-    return (unsigned)t < (unsigned)n ? t : 0;
-  }
-  // pos_of and succ for a warp-uniform argument (warp-collective)
-  __device__ __forceinline__ int pos_of_w(int q) const {
-    const int r = bsearch_le_warp(T.loB, *T.S, q);
-    const Seg s = T.sg[T.B[r]];
-    const int t = s.off + (s.rev ? s.lo + s.len - 1 - q : q - s.lo);
-    return (unsigned)t < (unsigned)n ? t : 0;
-  }
-  __device__ __forceinline__ int succ_w(int q) const {
-    int id = T.B[bsearch_le_warp(T.loB, *T.S, q)];
-    return step_up(q, id);
-  }
-  // pos_of for two warp-uniform nodes, with the segments that hold them
-  // (warp-collective): the two searches of B go level by level together,
-  // so that their shared-memory round trips overlap.
-  __device__ __forceinline__ void pos_id2_w(int q1, int q2, int& t1, int& id1, int& t2, int& id2) const {
-    const int lane = lane_id(), S = *T.S;
-    int lo1 = 0, len1 = S, lo2 = 0, len2 = S;
-    while (len1 > 1 || len2 > 1) {
-      const int st1 = (len1 + 31) >> 5, st2 = (len2 + 31) >> 5;
-      const bool le1 = len1 > 1 && lane * st1 < len1 && T.loB[lo1 + lane * st1] <= q1;
-      const bool le2 = len2 > 1 && lane * st2 < len2 && T.loB[lo2 + lane * st2] <= q2;
-      const unsigned b1 = __ballot_sync(kFull, le1), b2 = __ballot_sync(kFull, le2);
-      if (len1 > 1) {
-        const int L = b1 ? 31 - __clz(b1) : 0;
-        lo1 += L * st1;
-        len1 = min(st1, len1 - L * st1);
-      }
-      if (len2 > 1) {
-        const int L = b2 ? 31 - __clz(b2) : 0;
-        lo2 += L * st2;
-        len2 = min(st2, len2 - L * st2);
-      }
-    }
-    id1 = T.B[lo1];
-    id2 = T.B[lo2];
-    const Seg s1 = T.sg[id1], s2 = T.sg[id2];
-    t1 = s1.off + (s1.rev ? s1.lo + s1.len - 1 - q1 : q1 - s1.lo);
-    t2 = s2.off + (s2.rev ? s2.lo + s2.len - 1 - q2 : q2 - s2.lo);
-    if ((unsigned)t1 >= (unsigned)n) t1 = 0;
-    if ((unsigned)t2 >= (unsigned)n) t2 = 0;
-  }
-  __device__ __forceinline__ int at(int t) const {
-    const int r = bsearch_le(T.offA, *T.S, t);
-    const Seg s = T.sg[T.A[r]];
-    const int d = t - s.off;
-    const int q = s.rev ? s.lo + s.len - 1 - d : s.lo + d;
-    return (unsigned)q < (unsigned)n ? q : 0;
-  }
   __device__ __forceinline__ int2 coord(int q) const { return xy[q]; }
   __device__ __forceinline__ int cand(int q, int s) const { return cn[(size_t)q * kw + s]; }
   __device__ __forceinline__ int cdist(int q, int s) const { return cd[(size_t)q * kw + s]; }
 
-  // Segment id holding source position q.
-  __device__ __forceinline__ int locate(int q) const { return T.B[bsearch_le(T.loB, *T.S, q)]; }
-  // Next / previous node in ant order from q (in segment id); id follows.
-  __device__ __forceinline__ int step_up(int q, int& id) const {
-    const Seg s = T.sg[id];
-    const int d = s.rev ? s.lo + s.len - 1 - q : q - s.lo;
-    if (d < s.len - 1) return s.rev ? q - 1 : q + 1;
-    int r = T.rankA[id] + 1;
-    if (r == *T.S) r = 0;
-    id = T.A[r];
-    const Seg t = T.sg[id];
-    return t.rev ? t.lo + t.len - 1 : t.lo;
+  // Segment of node q: the largest r with lo[r] <= q.
+  __device__ __forceinline__ int locate(int q) const {
+    int r = 0;
+    for (int st = 1 << (31 - __clz(S)); st > 0; st >>= 1) {
+      const int m = r + st;
+      if (m < S && lo[m] <= q) r = m;
+    }
+    return r;
   }
-  __device__ __forceinline__ int step_dn(int q, int& id) const {
-    const Seg s = T.sg[id];
-    const int d = s.rev ? s.lo + s.len - 1 - q : q - s.lo;
-    if (d > 0) return s.rev ? q + 1 : q - 1;
-    int r = T.rankA[id] - 1;
-    if (r < 0) r = *T.S - 1;
-    id = T.A[r];
-    const Seg t = T.sg[id];
-    return t.rev ? t.lo : t.lo + t.len - 1;
+  // The same by a whole warp for one (warp-uniform) node: each level
+  // compares 32 boundaries spaced evenly over the remaining range, so a
+  // table of up to 1,024 segments takes two shared-memory round trips
+  // instead of ten dependent ones.
+  __device__ __forceinline__ int locate_w(int q) const {
+    const int lane = lane_id();
+    int at = 0, len = S;  // the answer lies in [at, at + len); lo[at] <= q
+    while (len > 1) {
+      const int st = (len + 31) >> 5;
+      const bool le = lane * st < len && lo[at + lane * st] <= q;
+      const unsigned b = __ballot_sync(kFull, le);
+      const int L = b ? 31 - __clz(b) : 0;
+      at += L * st;
+      len = min(st, len - L * st);
+    }
+    return at;
   }
-  __device__ __forceinline__ int succ(int q) const {
-    int id = locate(q);
-    return step_up(q, id);
+  // Two of them level by level, so that their round trips overlap.
+  __device__ __forceinline__ void locate2_w(int q1, int q2, int& r1, int& r2) const {
+    const int lane = lane_id();
+    int at1 = 0, at2 = 0, len = S;  // both ranges shrink alike, up to a shorter last part
+    int len1 = S, len2 = S;
+    while (len > 1) {
+      const int st = (len + 31) >> 5, o = lane * st;
+      const bool le1 = o < len1 && lo[at1 + o] <= q1, le2 = o < len2 && lo[at2 + o] <= q2;
+      const unsigned b1 = __ballot_sync(kFull, le1), b2 = __ballot_sync(kFull, le2);
+      const int L1 = b1 ? (31 - __clz(b1)) * st : 0, L2 = b2 ? (31 - __clz(b2)) * st : 0;
+      at1 += L1;
+      at2 += L2;
+      len1 = min(st, len1 - L1);
+      len2 = min(st, len2 - L2);
+      len = st;
+    }
+    r1 = at1;
+    r2 = at2;
   }
-  __device__ __forceinline__ int pred(int q) const {
-    int id = locate(q);
-    return step_dn(q, id);
+  __device__ __forceinline__ SegRec rec(int r) const {
+    const int b = br[r];
+    SegRec s;
+    s.lo = lo[r];
+    s.hi = lo[r + 1] - 1;
+    s.nlo = nb[r].x;
+    s.nhi = nb[r + 1].y;
+    s.base = b & 0x7fffffff;
+    s.rev = b < 0;
+    return s;
   }
   // succ(q) when up, else pred(q): one lookup whatever the direction
   __device__ __forceinline__ int adj(int q, bool up) const {
-    const int id = locate(q);
-    const Seg s = T.sg[id];
-    const int d = s.rev ? s.lo + s.len - 1 - q : q - s.lo;  // q's offset in ant order
-    if (up ? d < s.len - 1 : d > 0) return (up != (bool)s.rev) ? q + 1 : q - 1;
-    int r = T.rankA[id] + (up ? 1 : -1);
-    if (r == *T.S) r = 0;
-    if (r < 0) r = *T.S - 1;
-    const Seg t = T.sg[T.A[r]];
-    // first node in ant order of the next segment, or last of the previous
-    return (up == (bool)t.rev) ? t.lo + t.len - 1 : t.lo;
+    const SegRec s = rec(locate(q));
+    return s.step(q, up != s.rev);
   }
   __device__ __forceinline__ void nbrs(int q, int& p, int& s) const {
-    const int id = locate(q);
-    int i1 = id, i2 = id;
-    p = step_dn(q, i1);
-    s = step_up(q, i2);
+    const SegRec g = rec(locate(q));
+    p = g.step(q, g.rev);
+    s = g.step(q, !g.rev);
   }
+  // the predecessor and three successors of a warp-uniform node
+  // (warp-collective); most often all in one segment
   __device__ __forceinline__ void walk(int a, int& p, int& s1, int& s2, int& s3) const {
-    const int id = locate(a);
-    int i1 = id, i2 = id;
-    p = step_dn(a, i1);
-    s1 = step_up(a, i2);
-    s2 = step_up(s1, i2);
-    s3 = step_up(s2, i2);
+    SegRec g = rec(locate_w(a));
+    p = g.step(a, g.rev);
+    int q = a;
+    int s[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const bool in = g.inside(q, !g.rev);
+      q = g.step(q, !g.rev);
+      s[t] = q;
+      if (t < 2 && !in) g = rec(locate_w(q));
+    }
+    s1 = s[0];
+    s2 = s[1];
+    s3 = s[2];
+  }
+};
+
+// Tour over the segment table: what changes it.
+struct SegTour {
+  int n, k, kw;
+  SegTab T;
+  const int2* xy;
+  const int32_t* cn;
+  const int32_t* cd;
+
+  __device__ __forceinline__ char* buffer(int which) const {
+    return T.mem + (which ? (size_t)(T.cap + 1) * (kSegBytes / 2) : 0);
+  }
+  __device__ __forceinline__ SegView view() const {
+    const int m = T.cap + 1;
+    char* b = buffer(T.hdr[1]);
+    SegView v;
+    v.n = n;
+    v.k = k;
+    v.kw = kw;
+    v.S = T.hdr[0];
+    v.nb = reinterpret_cast<const int2*>(b);
+    v.lo = reinterpret_cast<const int32_t*>(b + (size_t)m * sizeof(int2));
+    v.br = v.lo + m;
+    v.xy = xy;
+    v.cn = cn;
+    v.cd = cd;
+    return v;
+  }
+  // The table of construction's `S` runs (in tour order), with the whole
+  // block: a thread per run finds its rank by counting.
+  __device__ __forceinline__ void build(const Seg* runs, int S) const {
+    const int m = T.cap + 1;
+    char* b = buffer(0);
+    int2* nb = reinterpret_cast<int2*>(b);
+    int32_t* lo = reinterpret_cast<int32_t*>(b + (size_t)m * sizeof(int2));
+    int32_t* br = lo + m;
+    for (int id = threadIdx.x; id < S; id += blockDim.x) {
+      const Seg s = runs[id];
+      int r = 0;
+      for (int o = 0; o < S; ++o) r += runs[o].lo < s.lo;
+      const Seg pr = runs[id == 0 ? S - 1 : id - 1], nx = runs[id + 1 == S ? 0 : id + 1];
+      const int hi = s.lo + s.len - 1;
+      const int before = pr.rev ? pr.lo : pr.lo + pr.len - 1;   // last node of the run before
+      const int after = nx.rev ? nx.lo + nx.len - 1 : nx.lo;    // first node of the run after
+      lo[r] = s.lo;
+      br[r] = s.rev ? (wrapn(s.off + hi, n) | (int)0x80000000) : wrapn(s.off - s.lo, n);
+      nb[r].x = s.rev ? after : before;
+      nb[r + 1].y = s.rev ? before : after;
+    }
+    if (threadIdx.x == 0) {
+      nb[0].y = 0;  // no node before 0: never read
+      nb[S].x = 0;
+      lo[S] = n;
+      br[S] = 0;
+    }
+    __syncthreads();  // the count and buffer number may lie in the runs' room
+    if (threadIdx.x == 0) {
+      T.hdr[0] = S;
+      T.hdr[1] = 0;
+    }
+    __syncthreads();
   }
 
   // Reverse the forward span x..y, or its complement when longer than n/2
-  // (the array rule, entry for entry).  false: the table is full.
-  __device__ __noinline__ bool flip(int x, int y, LsStats& St) {
+  // (the array rule, entry for entry).  Returns the nodes reversed, or -1
+  // when the table is full.  One warp; V: the current view.
+  //
+  // Bound by the latency of one warp's dependent steps: the search for x and
+  // y, the one for the nodes before and after them (only where a cut falls
+  // on a boundary), and the copying pass, S / 32 independent steps.  (The
+  // table it replaced kept an order by tour position beside the one by
+  // source position, shifted both for every cut and merge, and cut segments
+  // at position 0: with it the iteration of 1,024 ants at n = 100k took
+  // 6.3 ms and 2,048 ants at n = 200k 8.6 ms, with this one 4.8 and 6.0 ms.)
+  // Inlined, like everything else in the block kernel: it makes no calls.
+  __device__ __forceinline__ int flip(const SegView& V, int x, int y) const {
     const int lane = lane_id();
-    int px, hx, py, hy;
-    pos_id2_w(x, y, px, hx, py, hy);
-    // the position after y and the segment that holds it: y's own, unless
-    // y ends it (then the next one in ant order)
-    const int cy = (py + 1 == n) ? 0 : py + 1;
-    int hcy = hy;
-    if (cy != 0) {
-      const Seg sy = T.sg[hy];
-      if (cy >= sy.off + sy.len) hcy = T.A[T.rankA[hy] + 1];
-    }
-    __syncwarp();  // every lane has read the table before any lane rewrites a segment
-    // the span i..j and the segments holding its cuts i and j1 = j + 1
-    // (positions 0 and n need no cut): x..y, or y+1..x-1
-    int i = px, j = py, hi = hx, j1 = cy, hj = hcy;
+    const int S = V.S;
+    int rx, ry;
+    V.locate2_w(x, y, rx, ry);
+    const SegRec X = V.rec(rx), Y = V.rec(ry);
+    const int px = X.step(x, X.rev), sy = Y.step(y, !Y.rev);  // pred x, succ y
+    const bool inx = X.inside(x, X.rev), iny = Y.inside(y, !Y.rev);
+    int i = X.pos(x, n);
+    const int j = Y.pos(y, n);
     int L = j - i;
     if (L < 0) L += n;
     L += 1;
+    int sum = i + j;  // a position t of the span goes to sum - t, whichever part is reversed
+    if (sum >= n) sum -= n;
     if (2 * L > n) {
-      i = cy;
-      hi = hcy;
-      j = (px == 0) ? n - 1 : px - 1;
-      j1 = px;
-      hj = hx;
+      i = (j + 1 == n) ? 0 : j + 1;
       L = n - L;
     }
-    if (L <= 1) {
-      St.flip += L;
-      return true;
+    if (L <= 1) return L;
+    // at most two boundaries more: refuse before touching the table, which
+    // then still holds the tour
+    if (S + 2 > T.cap) return -1;
+    int rp = rx, rs = ry;  // segments of px and sy
+    bool revp = X.rev, revs = Y.rev;
+    if (!inx || !iny) {
+      V.locate2_w(px, sy, rp, rs);
+      revp = V.br[rp] < 0;
+      revs = V.br[rs] < 0;
     }
-    // a reversal adds at most three segments (two cuts, one at position 0):
-    // refuse before touching the table, which then still holds the tour
-    if (*T.S + 3 > T.cap) return false;
-    St.flip += L;
-    int si = -1, sj = -1;  // the segments that start at i and at j1
-    if (i != 0) {
-      si = seg_split(T, i, hi);
-      if (si < 0) return false;
-      // both cuts in one segment: the part from i on now holds j1
-      if (hj == hi && si != hi && j1 >= i) hj = si;
-    }
-    if (j1 != 0) {
-      sj = seg_split(T, j1, hj);
-      if (sj < 0) return false;
-    }
-    const int S = *T.S;
-    const int ri = (i == 0) ? 0 : T.rankA[si];
-    const int rj = (j1 == 0) ? S - 1 : T.rankA[sj] - 1;
-    if (i <= j) {
-      // contiguous ranks ri..rj: new off = i + j + 1 - off - len, direction
-      // flips, and the ranks reverse.  Lane m takes the pair of ranks
-      // (ri + m, rj - m) in one pass: the pairs, their ids and their
-      // segments are disjoint, so no lane reads what another writes.
-      const int c = rj - ri + 1, h = (c + 1) >> 1;
-      for (int m = lane; m < h; m += 32) {
-        const int ra = ri + m, rb = rj - m;
-        const int ida = T.A[ra], idb = T.A[rb];
-        const Seg sa = T.sg[ida], sb = T.sg[idb];
-        const int offa = i + j + 1 - sa.off - sa.len, offb = i + j + 1 - sb.off - sb.len;
-        T.sg[ida].off = offa;
-        T.sg[ida].rev = sa.rev ^ 1;
-        T.A[rb] = (uint16_t)ida;
-        T.offA[rb] = offa;
-        T.rankA[ida] = (uint16_t)rb;
-        if (rb != ra) {
-          T.sg[idb].off = offb;
-          T.sg[idb].rev = sb.rev ^ 1;
-          T.A[ra] = (uint16_t)idb;
-          T.offA[ra] = offb;
-          T.rankA[idb] = (uint16_t)ra;
-        }
+    // new boundaries where a cut edge lies inside a segment; boundaries that
+    // go: the new edge {px, y} or {x, sy} joins source neighbours, each at the
+    // end of its segment that faces the other
+    constexpr int kNone = INT_MAX;
+    const int c1 = inx ? max(px, x) : kNone, c2 = iny ? max(y, sy) : kNone;
+    const int m1 = (revp != Y.rev && y - px == (revp ? -1 : 1)) ? max(px, y) : kNone;
+    const int m2 = (X.rev != revs && sy - x == (X.rev ? 1 : -1)) ? max(x, sy) : kNone;
+    // (boundaries of the new table) - (of the old one) below node v
+    auto shift = [&](int v) { return (c1 < v) + (c2 < v) - (m1 < v) - (m2 < v); };
+    // the map of a segment that contains node v, after the reversal
+    auto turned = [&](int b, int v) {
+      const int base = b & 0x7fffffff;
+      int d = wrapn(b < 0 ? base - v : base + v, n) - i;
+      if (d < 0) d += n;
+      if (d >= L) return b;
+      int nbase = sum - base;
+      if (nbase < 0) nbase += n;
+      return nbase | (~b & (int)0x80000000);
+    };
+    const int m = T.cap + 1, cur = T.hdr[1];
+    char* out = buffer(cur ^ 1);
+    int2* nb2 = reinterpret_cast<int2*>(out);
+    int32_t* lo2 = reinterpret_cast<int32_t*>(out + (size_t)m * sizeof(int2));
+    int32_t* br2 = lo2 + m;
+#pragma unroll 2
+    for (int r = lane; r <= S; r += 32) {
+      const int v = V.lo[r];
+      const int b = V.br[r];
+      const int2 e = V.nb[r];
+      if (v != m1 && v != m2) {
+        const int w = r + shift(v);
+        lo2[w] = v;
+        br2[w] = turned(b, v);
+        nb2[w] = e;
       }
-      __syncwarp();
-      seg_merge_at(T, rj);      // the span's right end and its old right neighbour
-      seg_merge_at(T, ri - 1);  // its left neighbour and the span's new left end
-      return true;
-    } else {
-      // the span wraps: ranks ri..S-1 then 0..rj; lay the reversed list
-      // out from position i, cutting the segment that crosses position 0
-      const int clo = rj + 1, chi = S - ri, c = clo + chi;
-      // R[m] = A[rj - m] (m < clo), A[S - 1 - (m - clo)] (m >= clo)
-      for (int m = lane; m < c; m += 32) T.tmp[m] = m < clo ? T.A[rj - m] : T.A[S - 1 - (m - clo)];
-      __syncwarp();
-      // new offsets: R laid out from position i (a prefix sum of the lengths,
-      // 32 segments at a time), wrapped below n; the segment that crosses
-      // position n (straddle) and how many start below n (nhi)
-      int straddle = -1, cut = 0, nhi = 0, carry = 0;
-      for (int m0 = 0; m0 < c; m0 += 32) {
-        const int m = m0 + lane;
-        int len = 0;
-        if (m < c) len = T.sg[T.tmp[m]].len;
-        int incl = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const int at = i + carry + incl - len;  // first position of segment m
-        if (m < c) {
-          Seg& s = T.sg[T.tmp[m]];
-          s.rev ^= 1;
-          s.off = at >= n ? at - n : at;
-        }
-        const unsigned bs = __ballot_sync(kFull, m < c && at < n && at + len > n);
-        if (bs) {
-          const int l = __ffs(bs) - 1;
-          straddle = m0 + l;
-          cut = n - __shfl_sync(kFull, at, l);
-        }
-        nhi += __popc(__ballot_sync(kFull, m < c && at < n));
-        carry += __shfl_sync(kFull, incl, 31);
+    }
+    __syncwarp();  // the neighbours below overwrite copied ones
+    // lanes 0..3: the ends px, x, y, sy of the two cut edges get their new
+    // neighbours y, sy, px, x, in the slot of the side that faced the cut
+    if (lane < 4) {
+      const bool first = lane < 2;  // an end of the cut {px, x}
+      const int o = lane == 0 ? px : (lane == 1 ? x : (lane == 2 ? y : sy));
+      const int to = lane == 0 ? y : (lane == 1 ? sy : (lane == 2 ? px : x));
+      const bool hiside = lane == 0 ? !revp : (lane == 1 ? X.rev : (lane == 2 ? !Y.rev : revs));
+      const int ro = lane == 0 ? rp : (lane == 1 ? rx : (lane == 2 ? ry : rs));
+      const bool in = first ? inx : iny;
+      const int v = hiside ? o + 1 : o;  // the boundary
+      const int w = ro + ((in || hiside) ? 1 : 0) + shift(v);
+      const bool gone = ((lane == 0 || lane == 2) ? m1 : m2) != kNone;
+      if (!gone) {
+        if (hiside)
+          nb2[w].y = to;
+        else
+          nb2[w].x = to;
       }
+      // lanes 1 and 2 also write the new boundary of their cut
+      if (in && (lane == 1 || lane == 2)) {
+        lo2[w] = v;
+        br2[w] = turned((first ? X.base | (X.rev ? (int)0x80000000 : 0) : Y.base | (Y.rev ? (int)0x80000000 : 0)), v);
+      }
+    }
+    if (lane == 0) {
+      T.hdr[0] = S + (inx ? 1 : 0) + (iny ? 1 : 0) - (m1 != kNone) - (m2 != kNone);
+      T.hdr[1] = cur ^ 1;
+    }
+    __syncwarp();
+    return L;
+  }
+};
+
+// Shared scratch of the block search.
+struct LsShared {
+  int32_t gain[32];
+  int mv[32][8];
+  int qh, qn, nlog, changes, moves_round, fail;
+  int64_t total;
+};
+
+// The search of ls_run by a block of W warps on one tour: each round, warp w
+// evaluates the w-th queued node; entries are popped in queue order up to
+// and including the first one whose evaluation found a move, which warp 0
+// applies.  Nothing changes the tour between the confirmed evaluations, so
+// the result equals popping one node at a time.  Must be called by every
+// thread of the block.  Returns the gain, or -1 when the table filled up
+// (flags are left clean either way; the caller has the ant redone on arrays).
+__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, const int32_t* init, int ninit,
+                                                LsStats& S, LsShared& sh) {
+  const int n = E.n, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int W = blockDim.x >> 5;
+  for (int i = tid; i < ninit; i += blockDim.x) {
+    const int x = init[i];
+    E.queue[i] = x;
+    E.flags[x] = 1;
+  }
+  if (tid == 0) {
+    sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.fail = 0;
+    sh.total = 0;
+  }
+  __syncthreads();
+  for (;;) {
+    const int qh = sh.qh, qn = sh.qn;
+    if (qn == 0 || sh.changes >= n || sh.fail) {
+      if (sh.fail || sh.changes >= n || !E.verify || sh.moves_round == 0) break;
+      const int nl = sh.nlog;  // verify round: queue again the nodes popped
+      for (int i = tid; i < nl; i += blockDim.x) {
+        const int x = E.logb[i];
+        E.queue[i] = x;
+        E.flags[x] = 1;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        sh.qh = 0; sh.qn = nl; sh.nlog = 0; sh.moves_round = 0;
+      }
+      if (w == 0) S.verify++;
+      __syncthreads();
+      continue;
+    }
+    const int R = qn < W ? qn : W;
+    const uint64_t t0 = (w == 0) ? global_ns() : 0;
+    if (w < R) {
+      int idx = qh + w;
+      if (idx >= n) idx -= n;
+      const int a = E.queue[idx];
+      int mv[8];
+      const int32_t g = eval_both(T.view(), a, E.oropt != 0, mv);
+      if (lane == 0) {
+        sh.gain[w] = g;
+        if (g > 0)
+          for (int t = 0; t < 8; ++t) sh.mv[w][t] = mv[t];
+      }
+    }
+    __syncthreads();
+    if (w == 0) {
+      const uint64_t t1 = global_ns();
+      S.t_eval += (int64_t)(t1 - t0);
+      const unsigned bal = __ballot_sync(kFull, lane < R && sh.gain[lane] > 0);
+      const int first = bal ? __ffs(bal) - 1 : R;
+      const int cnt = bal ? first + 1 : R;  // queue entries popped this round
+      int a = -1;
+      bool first_pop = false;
+      if (lane < cnt) {
+        int idx = qh + lane;
+        if (idx >= n) idx -= n;
+        a = E.queue[idx];
+        const uint8_t f = E.flags[a];
+        first_pop = !(f & 2);
+        E.flags[a] = (uint8_t)((f & ~1) | 2);
+      }
+      const unsigned fb = __ballot_sync(kFull, first_pop);
+      if (first_pop) E.logb[sh.nlog + __popc(fb & ((1u << lane) - 1u))] = a;
+      S.pops += cnt;
       __syncwarp();
-      int S2 = S;
-      int nid = -1;
-      if (straddle >= 0) {
-        if (S >= T.cap) return false;
-        const int id = T.tmp[straddle];
-        const Seg s = T.sg[id];
-        nid = S;
-        const int rb = T.rankB[id];
-        __syncwarp();
-        if (lane == 0) {
-          // id keeps ant positions [s.off, n); nid takes [0, s.len - cut)
-          if (!s.rev) {
-            T.sg[nid] = Seg{s.lo + cut, s.len - cut, 0, 0};
-            T.sg[id].len = cut;
-          } else {
-            T.sg[nid] = Seg{s.lo, s.len - cut, 0, 1};
-            T.sg[id].lo = s.lo + s.len - cut;
-            T.sg[id].len = cut;
+      int qh2 = qh + cnt;
+      if (qh2 >= n) qh2 -= n;
+      int qn2 = qn - cnt;
+      const uint64_t t2 = global_ns();
+      S.t_confirm += (int64_t)(t2 - t1);
+      if (bal) {  // apply the first move found, queue its endpoints
+        const int* mv = sh.mv[first];
+        const bool two = mv[7] == 0;
+        // a 2-opt move is one edge exchange, its first edge (mv[0], mv[1])
+        // forward; an Or-opt move is two or three
+        const int steps = two ? 1 : (mv[6] ? 3 : 2);
+        for (int st = 0; st < steps; ++st) {
+          const int n1 = st == 2 ? mv[4] : mv[0];
+          const int n2 = st == 0 ? mv[1] : (st == 1 ? mv[4] : mv[2]);
+          const int n3 = st == 0 ? (two ? mv[2] : mv[4]) : (st == 1 ? mv[3] : mv[1]);
+          const int n4 = st == 0 ? (two ? mv[3] : mv[5]) : (st == 1 ? mv[2] : mv[5]);
+          const SegView V = T.view();
+          bool fwd = two;
+          if (!two) {
+            const SegRec g = V.rec(V.locate_w(n1));
+            fwd = g.step(n1, !g.rev) == n2;
           }
+          const int L = T.flip(V, fwd ? n2 : n1, fwd ? n3 : n4);
+          if (L < 0) {  // the table is full
+            if (lane == 0) sh.fail = 1;
+            break;
+          }
+          S.flip += L;
         }
-        __syncwarp();
-        if (!s.rev) {
-          ins_B(T, S, rb + 1, nid, s.lo + cut);
-        } else {  // nid keeps the low end: it goes before id, whose lo moved up
-          ins_B(T, S, rb, nid, s.lo);
-          if (lane == 0) T.loB[rb + 1] = s.lo + s.len - cut;
-          __syncwarp();
+        if (two)
+          S.moves2++;
+        else
+          S.movesor++;
+        const uint64_t t3 = global_ns();
+        S.t_flip += (int64_t)(t3 - t2);
+        qn2 = ls_push_warp(E, mv, two ? 4 : 6, qh2, qn2);
+        if (lane == 0) {
+          sh.total += sh.gain[first];
+          sh.changes++;
+          sh.moves_round++;
         }
-        S2 = S + 1;
+        S.t_push += (int64_t)(global_ns() - t3);
       }
-      // new A: [nid] + wrapped part of R + middle A[clo..ri) + unwrapped part of R
-      // R is ordered by new position: the unwrapped part (offsets >= i) comes
-      // first in R, the wrapped part after it.
-      // nhi: R entries placed in [i, n), up to and including the straddler
-      // assemble into the tail of tmp: tmp[c..c+S2)
-      uint16_t* out = T.tmp + c;
-      const int mid = ri - clo;
-      const int head = (nid >= 0) ? 1 : 0;
-      const int nlo = c - nhi;
-      if (lane == 0 && nid >= 0) out[0] = (uint16_t)nid;
-      for (int m = lane; m < nlo; m += 32) out[head + m] = T.tmp[nhi + m];
-      for (int m = lane; m < mid; m += 32) out[head + nlo + m] = T.A[clo + m];
-      for (int m = lane; m < nhi; m += 32) out[head + nlo + mid + m] = T.tmp[m];
-      __syncwarp();
-      for (int m = lane; m < S2; m += 32) {
-        const int id = out[m];
-        T.A[m] = (uint16_t)id;
-        T.offA[m] = T.sg[id].off;
-        T.rankA[id] = (uint16_t)m;
+      if (lane == 0) {
+        sh.nlog += __popc(fb);
+        sh.qh = qh2;
+        sh.qn = qn2;
       }
       __syncwarp();
-      if (lane == 0) *T.S = S2;
-      __syncwarp();
-      // Merges: reversing a run of segments keeps every pair inside it as
-      // (un)mergeable as it was, and the table held no mergeable pair except
-      // across position 0.  New pairs: the span's right end with the middle
-      // (r1), the middle with the span's left end (r2), and the pair that
-      // crossed position 0 (R[clo-1], R[clo]), now inside the span (r3; none
-      // when the new cut at position 0 falls between them).  Highest rank
-      // first, so that no merge moves a rank still to be merged.
-      const int r1 = head + nlo - 1, r2 = r1 + mid;
-      int r3 = -1;
-      if (clo < nhi)
-        r3 = r2 + clo;  // both in the part placed from position i
-      else if (clo - 1 >= nhi)
-        r3 = head + clo - 1 - nhi;  // both in the part wrapped below position i
-      else if (head)
-        r3 = 0;  // the cut split R[clo-1]: its tail (nid) precedes R[clo]
-      if (r3 > r2) seg_merge_at(T, r3);
-      seg_merge_at(T, r2);
-      seg_merge_at(T, r1);
-      if (r3 >= 0 && r3 < r1) seg_merge_at(T, r3);
-      return true;
     }
+    __syncthreads();
   }
-};
-
-// A segment tour that moves to explicit arrays the first time its table is
-// full: the table (which still holds the tour) is written out as
-// route[t] = source position, pos = inverse, and the search goes on there
-// with the same node names, queue and counters.
-struct HybTour {
-  int n, k;
-  SegTour sg;
-  ArrTour ar;       // over source positions (XYsrc, Csrc), used once *mode != 0
-  int32_t* mode;    // shared flag: 0 = table, 1 = arrays
-
-  __device__ __forceinline__ bool arrays() const { return *mode != 0; }
-  __device__ __forceinline__ int pos_of(int x) const { return arrays() ? ar.pos_of(x) : sg.pos_of(x); }
-  __device__ __forceinline__ int succ(int x) const { return arrays() ? ar.succ(x) : sg.succ(x); }
-  __device__ __forceinline__ int succ_w(int x) const { return arrays() ? ar.succ(x) : sg.succ_w(x); }
-  __device__ __forceinline__ int pred(int x) const { return arrays() ? ar.pred(x) : sg.pred(x); }
-  __device__ __forceinline__ int adj(int x, bool up) const { return arrays() ? ar.adj(x, up) : sg.adj(x, up); }
-  __device__ __forceinline__ void nbrs(int x, int& p, int& s) const {
-    if (arrays())
-      ar.nbrs(x, p, s);
-    else
-      sg.nbrs(x, p, s);
+  __syncthreads();
+  const int qh = sh.qh, qn = sh.qn, nl = sh.nlog;
+  for (int t = tid; t < qn; t += blockDim.x) {
+    int i = qh + t;
+    if (i >= n) i -= n;
+    E.flags[E.queue[i]] = 0;
   }
-  __device__ __forceinline__ void walk(int a, int& p, int& s1, int& s2, int& s3) const {
-    if (arrays())
-      ar.walk(a, p, s1, s2, s3);
-    else
-      sg.walk(a, p, s1, s2, s3);
-  }
-  __device__ __forceinline__ int2 coord(int x) const { return sg.coord(x); }
-  __device__ __forceinline__ int cand(int x, int s) const { return sg.cand(x, s); }
-  __device__ __forceinline__ int cdist(int x, int s) const { return sg.cdist(x, s); }
-
-  __device__ __noinline__ void to_arrays() {
-    const int S = *sg.T.S;
-    for (int r = 0; r < S; ++r) {
-      const Seg s = sg.T.sg[sg.T.A[r]];
-      for (int d = lane_id(); d < s.len; d += 32) {
-        const int q = s.rev ? s.lo + s.len - 1 - d : s.lo + d;
-        ar.route[s.off + d] = q;
-        ar.pos[q] = s.off + d;
-      }
-    }
-    __syncwarp();
-    if (lane_id() == 0) *mode = 1;
-    __syncwarp();
-  }
-
-  static __device__ __noinline__ bool flip_arrays(ArrTour& A, int x, int y, LsStats& S) { return A.flip(x, y, S); }
-  // warp-collective; never fails
-  __device__ __forceinline__ bool flip(int x, int y, LsStats& S) {
-    if (!arrays()) {
-      if (sg.flip(x, y, S)) return true;
-      to_arrays();
-    }
-    return flip_arrays(ar, x, y, S);
-  }
-};
-
-// Evaluation on the representation the hybrid tour holds now (uniform
-// across the block): the table path and the array path stay separate
-// code, instead of a branch in every lookup.
-// The array representation serves only ants whose table filled up: its
-// evaluation and reversal stay out of line, so that the table's hot loop
-// keeps its registers and a smaller code footprint (spill stores of the
-// per-ant kernel 620 -> 220 bytes, the kernel 3-4 % faster).
-static __device__ __noinline__ int32_t eval_arrays(const ArrTour& T, int a, bool do_or, int* mv) {
-  int m[8];
-  const int32_t g = eval_both(T, a, do_or, m);
-  for (int t = 0; t < 8; ++t) mv[t] = m[t];
-  return g;
-}
-__device__ __forceinline__ int32_t eval_dispatch(const HybTour& T, int a, bool do_or, int (&mv)[8]) {
-  return T.arrays() ? eval_arrays(T.ar, a, do_or, mv) : eval_both(T.sg, a, do_or, mv);
+  for (int i = tid; i < nl; i += blockDim.x) E.flags[E.logb[i]] = 0;
+  __syncthreads();
+  return sh.fail ? -1 : sh.total;
 }
 
 }  // namespace faco

@@ -59,3 +59,12 @@ def test_euc2d_at_the_limit_of_the_estimate():
     device_selftest(1, inp, out, len(d))
     want = [oracle.euc2d(np.array([[a, b], [c, e]], np.int32), 0, 1) for a, b, c, e in inp]
     np.testing.assert_array_equal(out, np.array(want, np.int32))
+
+
+@pytest.mark.parametrize("seg_cap", [8, 33, 64, 256, -1])
+@pytest.mark.parametrize("n", [31, 65, 1023, 2500])
+def test_segment_table_capacities(n, seg_cap):
+    """Tables that fill up in construction, in the search, or never: an ant
+    that outgrows its table is redone on arrays with the same result."""
+    xy = inputs.stippled(n, seed=n, blobs=6, ridges=1, side=50_000) if n > 1000 else inputs.uniform(n, seed=n)
+    assert_run_equals_oracle(xy, 16, 12, 5, seg_cap=seg_cap, min_new_edges=24)
