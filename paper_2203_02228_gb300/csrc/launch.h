@@ -62,6 +62,7 @@ cudaError_t launch_tour_length(const int2* xy, const int32_t* route, int n, int6
                                cudaStream_t s);
 
 // knn.cu
+constexpr int kKnnBatchNodes = 32;  // nodes per block of the batch list builder (its block map)
 cudaError_t launch_bbox_check(const int2* xy, int n, int32_t* out5, cudaStream_t s);
 cudaError_t build_lists(const int2* xy, int n, int k, int bl, const Grid& g, int32_t* cell_count,
                         int32_t* cell_start, int32_t* cell_pts, int4* cell_src, int32_t* cand, int32_t* backup,
@@ -70,7 +71,7 @@ cudaError_t build_lists(const int2* xy, int n, int k, int bl, const Grid& g, int
 cudaError_t launch_grid_batch(Colony* cols, const ColonySetup* sets, int count, const int2* map256, int nmap256,
                               cudaStream_t s);
 cudaError_t build_lists_batch(const Colony* cols, const ColonySetup* sets, int count, const int2* map256,
-                              int nmap256, const int2* map128, int nmap128, cudaStream_t s);
+                              int nmap256, const int2* map_knn, int nmap_knn, cudaStream_t s);
 
 // tour.cu
 cudaError_t launch_nn_tour(const int2* xy, int n, const int32_t* cand, int k, const int32_t* backup,

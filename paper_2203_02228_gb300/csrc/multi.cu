@@ -118,17 +118,17 @@ void group_layout(Group& g, char* base) {
   for (int i = 0; i < C; ++i) g.hS[i].flags = B.take<uint8_t>(g.n[i]);
   g.zero_bytes = (B.size + 255) & ~(size_t)255;
   // tables
-  std::vector<int2> m256, m128;
+  std::vector<int2> m256, mknn;
   for (int i = 0; i < C; ++i) {
     add_blocks(m256, i, g.n[i], 256);
-    add_blocks(m128, i, g.n[i], 128);
+    add_blocks(mknn, i, g.n[i], kKnnBatchNodes);
   }
   g.nmap256 = (int)m256.size();
-  g.nmap128 = (int)m128.size();
+  g.nmap_knn = (int)mknn.size();
   g.dC = B.take<Colony>(C);
   g.dS = B.take<ColonySetup>(C);
   g.map256 = B.take<int2>(m256.size());
-  g.map128 = B.take<int2>(m128.size());
+  g.map_knn = B.take<int2>(mknn.size());
   g.d_node_off = B.take<int64_t>(C + 1);
   for (int i = 0; i < C; ++i) g.hS[i].bb = B.take<int32_t>(5);
   // per-colony arrays, type by type
@@ -221,19 +221,19 @@ int group_setup(Group& g, const int32_t* const* coords, cudaStream_t s) {
   for (int i = 0; i < g.count; ++i)
     CK(cudaMemcpyAsync(const_cast<int2*>(g.hC[i].xy), coords[i], sizeof(int2) * (size_t)g.n[i],
                        cudaMemcpyHostToDevice, s));
-  std::vector<int2> m256, m128;
+  std::vector<int2> m256, mknn;
   for (int i = 0; i < g.count; ++i) {
     add_blocks(m256, i, g.n[i], 256);
-    add_blocks(m128, i, g.n[i], 128);
+    add_blocks(mknn, i, g.n[i], kKnnBatchNodes);
   }
   // pageable sources: each copy has been staged when the call returns
   CK(cudaMemcpyAsync(g.dC, g.hC.data(), sizeof(Colony) * g.count, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(g.dS, g.hS.data(), sizeof(ColonySetup) * g.count, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(g.map256, m256.data(), sizeof(int2) * m256.size(), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g.map128, m128.data(), sizeof(int2) * m128.size(), cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(g.map_knn, mknn.data(), sizeof(int2) * mknn.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(g.d_node_off, g.node_off.data(), sizeof(int64_t) * (g.count + 1), cudaMemcpyHostToDevice, s));
   CK(launch_grid_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, s));
-  CK(build_lists_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, g.map128, g.nmap128, s));
+  CK(build_lists_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, g.map_knn, g.nmap_knn, s));
   CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, 0, s));       // nearest-neighbour tours
   CK(launch_colony_init_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, 0, s));
   CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, 1, s));       // their local search

@@ -43,8 +43,8 @@ struct Group {
   Colony* dC = nullptr;
   ColonySetup* dS = nullptr;
   int2* map256 = nullptr;
-  int2* map128 = nullptr;
-  int nmap256 = 0, nmap128 = 0;
+  int2* map_knn = nullptr;
+  int nmap256 = 0, nmap_knn = 0;
   int64_t* d_node_off = nullptr;  // node_off on the device
 };
 

@@ -68,3 +68,38 @@ def test_segment_table_capacities(n, seg_cap):
     that outgrows its table is redone on arrays with the same result."""
     xy = inputs.stippled(n, seed=n, blobs=6, ridges=1, side=50_000) if n > 1000 else inputs.uniform(n, seed=n)
     assert_run_equals_oracle(xy, 16, 12, 5, seg_cap=seg_cap, min_new_edges=24)
+
+
+def _list_points(kind):
+    rng = np.random.default_rng(17)
+    if kind == "heap":       # one grid cell holds far more than a warp's buffer
+        a = rng.integers(0, 60, size=(1500, 2))
+        return np.concatenate([a, rng.integers(0, 1_000_000, size=(300, 2))])
+    if kind == "same":       # most points coincide
+        return np.concatenate([np.full((900, 2), 777), rng.integers(0, 5_000, size=(40, 2))])
+    if kind == "outlier":    # one point far from the rest
+        return np.concatenate([rng.integers(0, 2_000, size=(700, 2)), [[(1 << 24) - 1, (1 << 24) - 1]]])
+    if kind == "line":
+        return np.stack([np.arange(900) * 13, np.zeros(900)], 1)
+    return rng.integers(0, 100_000, size=(int(kind), 2))
+
+
+@pytest.mark.parametrize("kind", ["heap", "same", "outlier", "line", "4", "81", "82", "161", "162", "385"])
+@pytest.mark.parametrize("k,bl", [(16, 64), (32, 128), (2, 0)])
+def test_lists_of_uneven_points(kind, k, bl):
+    xy = np.ascontiguousarray(_list_points(kind), dtype=np.int32)
+    n = len(xy)
+    g = Colony(xy, k, bl_size=bl)
+    cand, backup, eta = g.lists()
+    x = xy.astype(np.int64)
+    d2 = (x[:, None, 0] - x[None, :, 0]) ** 2 + (x[:, None, 1] - x[None, :, 1]) ** 2
+    d2[np.arange(n), np.arange(n)] = np.iinfo(np.int64).max
+    order = np.argsort(d2, axis=1, kind="stable")  # ties by node id
+    ke = min(k, n - 1)
+    ble = min(bl, n - 1 - ke)
+    np.testing.assert_array_equal(cand, order[:, :ke])
+    np.testing.assert_array_equal(backup, order[:, ke:ke + ble])
+    near = np.take_along_axis(d2, order[:, :ke], 1)
+    d = np.floor(np.sqrt(near.astype(np.float64)) + 0.5)
+    want = np.where(d > 0, np.float32(1) / np.maximum(d, 1).astype(np.float32), np.float32(1)).astype(np.float32)
+    np.testing.assert_array_equal(eta, want)
