@@ -101,13 +101,6 @@ __global__ void __launch_bounds__(32) k_nn_tour_b(const Colony* cols, const Colo
   nn_tour_body(C.xy, C.n, S.cand, C.k, S.backup, C.bl, S.init_route, sv, C.grid, S.cell_start, S.cell_src);
 }
 
-// Positions reversed by one move (at most three flips): first position and
-// length of each reversed span, appended by thread 0.
-struct SpanLog {
-  int2 span[3];
-  int count;
-};
-
 // The initial search's tour with its positions in shared memory (n up to
 // about 106k nodes fits): the low 16 bits of each position in lo[n], bit 16
 // in the bitmap hi.  Otherwise the same lookups as ArrTour.
@@ -185,28 +178,32 @@ __device__ __forceinline__ void smem_pos_load(SmemPosTour& T) {
   __syncthreads();
 }
 
-// Reverse the forward span x..y (or its complement) with the whole block;
-// the span actually reversed goes to the log.  Every caller reaches it
-// after a block barrier that follows the last write to the tour.
-template <class TT>
-__device__ void cta_flip(TT& T, int x, int y, SpanLog& log) {
-  const int n = T.n;
-  int i = T.pos_of(x), j = T.pos_of(y);
-  __syncthreads();  // every thread has read i, j before any position moves
+// A reversed span of tour positions: i, i + 1, ..., i + L - 1 (cyclic).
+struct Span {
+  int i, L;
+};
+
+// The span that reversing the forward span i..j turns over: itself, or its
+// complement when longer than n / 2.
+__device__ __forceinline__ Span flip_span(int i, int j, int n) {
   int L = j - i;
   if (L < 0) L += n;
   L += 1;
-  if (2 * L > n) {
-    const int i2 = (j + 1 == n) ? 0 : j + 1;
-    const int j2 = (i == 0) ? n - 1 : i - 1;
-    i = i2;
-    j = j2;
-    L = n - L;
-  }
-  if (threadIdx.x == 0 && log.count < 3) log.span[log.count++] = make_int2(i, L);
-  const int half = L >> 1;
+  if (2 * L > n) return Span{j + 1 == n ? 0 : j + 1, n - L};
+  return Span{i, L};
+}
+
+// Reverses a span with the whole block.  Every caller reaches it after a
+// block barrier that follows the last write to the tour, and the next reader
+// waits at one.
+template <class TT>
+__device__ __forceinline__ void cta_reverse(TT& T, Span sp) {
+  const int n = T.n;
+  int j = sp.i + sp.L - 1;
+  if (j >= n) j -= n;
+  const int half = sp.L >> 1;
   for (int t = threadIdx.x; t < half; t += blockDim.x) {
-    int ia = i + t;
+    int ia = sp.i + t;
     if (ia >= n) ia -= n;
     int ib = j - t;
     if (ib < 0) ib += n;
@@ -216,68 +213,114 @@ __device__ void cta_flip(TT& T, int x, int y, SpanLog& log) {
     T.move_pos(vb, ib, ia);
     T.move_pos(va, ia, ib);
   }
-  __syncthreads();
-}
-
-template <class TT>
-__device__ void cta_move2(TT& T, int n1, int n2, int n3, int n4, SpanLog& log) {
-  const bool fwd = T.succ(n1) == n2;
-  if (fwd)
-    cta_flip(T, n2, n3, log);
-  else
-    cta_flip(T, n1, n4, log);
-}
-
-// true when position p lies in the cyclic span (first position i, length L).
-__device__ __forceinline__ bool in_span(int p, int2 sp, int n) {
-  int d = p - sp.x;
-  if (d < 0) d += n;
-  return d < sp.y;
 }
 
 // The local search with every node queued (the initial tour), run by one
-// block of 32 warps over a window of the next 32 queued nodes.  Each window
-// entry keeps its evaluation -- the best 2-opt / Or-opt move from its node
-// on the tour as it was -- together with the tour positions that evaluation
-// read (the node's, the next three and the previous one; each candidate's
-// and its two neighbours').  A move reverses spans of positions; an entry
-// whose positions meet none of them would evaluate to the same result, so
-// it is kept, the others are dropped.  Each round pops entries in queue
-// order up to and including the first one whose evaluation found a move,
-// which is applied.  An evaluation runs only when an entry without one
-// comes before the first improving entry (all entries without one are then
-// evaluated, a warp each).  The pops, moves and queue are exactly those of
-// popping one node at a time.
-constexpr int kWin = 32;
+// block of 32 warps over a window of the next kWin queued nodes.  Each
+// window entry keeps its evaluation -- the best move from its node on the
+// tour as it was -- together with the tour positions that evaluation read
+// (the node's, the next three and the previous one; each candidate's and its
+// two neighbours').  A move reverses spans of positions; an entry whose
+// positions meet none of them would evaluate to the same result, so it is
+// kept, the others are dropped.  Each round pops entries in queue order up
+// to and including the first one whose evaluation found a move, which is
+// applied.  An evaluation runs only when an entry without one comes before
+// the first improving entry (all entries without one are then evaluated, a
+// warp each).  The pops, moves and queue are exactly those of popping one
+// node at a time.
+//
+// Bound by the latency of a round, one move long: evaluation, decision,
+// reversal.  So every warp takes the same decisions from the same shared
+// values, in registers, with two block barriers per round (after the
+// evaluations, after the reversal); a 2-opt move brings the positions of its
+// ends along; entries to drop are found while the span is being reversed;
+// and the queue's own work -- flags, log, pushes, reading nodes ahead into
+// shared memory -- is left to the last warp, during the next round's
+// evaluations.  Only with less than kAhead nodes queued does a round wait
+// for it (sync_queue).  Set-up 14.1 -> 12.1 ms at n = 5,003 and 322 -> 302 ms at
+// n = 100,000 against the form with six barriers per round and the queue's
+// work between them.  Evaluating only the first 8 / 16 / 24 entries of the
+// window without an evaluation: 408 / 330 / 316 ms against 318 (n = 100,000).
+constexpr int kWin = 31;     // entries, a warp each; the last warp keeps the queue
+constexpr int kAhead = 96;   // queued nodes read ahead (a ring of 128)
 
 template <class TT>
 __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int init3, int32_t* queue, uint8_t* flags,
                                              int32_t* logb) {
-  __shared__ int64_t s_gain[kWin];
-  __shared__ int s_mv[kWin][8];
-  __shared__ int s_any[kWin];             // 1: the evaluation read beyond s_dep (3-opt scan): any move drops it
-  __shared__ int s_node[kWin];            // node whose evaluation the slot holds, -1: none
-  __shared__ int s_dep[kWin][kMaxK + 1];  // [0]: its position, [1 + s]: candidate s's position
-  __shared__ SpanLog s_log;
-  __shared__ int s_qh, s_qn, s_nlog, s_changes, s_moves_round, s_win, s_base;
+  __shared__ int32_t s_gain[32];
+  __shared__ int s_mv[32][8];
+  __shared__ int2 s_ij[32];               // 2-opt: positions of the span's ends
+  __shared__ int s_any[32];               // 1: the evaluation read beyond s_dep (3-opt scan): any move drops it
+  __shared__ int s_dep[32][kMaxK + 1];    // [0]: its position, [1 + s]: candidate s's position
+  __shared__ int s_inv[2][32];            // 1: the round's move drops the entry
+  __shared__ int s_q[128];                // nodes of the queue by position modulo 128, from the head on
+  __shared__ int s_pmv[8];                // the last warp's copy of that round's move
+  __shared__ int s_qn, s_nlog;
   const int n = T.n, k = T.k;
   int32_t* route = T.route;
   LsEnv E{n, oropt, verify, queue, flags, logb};
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const bool keeper = w == kWin;
   for (int i = tid; i < n; i += blockDim.x) {
     const int x = route[i];
     queue[i] = x;
     flags[x] = 1;
   }
-  if (tid < kWin) s_node[tid] = -1;
-  if (tid == 0) {
-    s_qh = 0; s_qn = n; s_nlog = 0; s_changes = 0; s_moves_round = 0; s_base = 0;
-  }
   __syncthreads();
+  // the same on every thread: queue position of the head (counted from the
+  // start, and modulo n), nodes queued (not counting pushes since the last
+  // sync_queue), moves applied, entries of the window with an evaluation
+  unsigned qa = 0;
+  int qh = 0, qn = n, changes = 0, moves_round = 0, par = 0;
+  unsigned have = 0;
+  // the last warp: nodes queued, nodes logged, nodes read ahead, and the
+  // round whose pops and pushes it has not done yet
+  int kq = n, klog = 0, kld = 0, p_cnt = 0, p_np = 0, p_node = -1, p_qh = 0;
+  auto keep_pending = [&]() {  // (last warp)
+    if (p_cnt == 0) return;
+    bool first_pop = false;
+    if (lane < p_cnt) {
+      const uint8_t f = flags[p_node];
+      first_pop = !(f & 2);
+      flags[p_node] = (uint8_t)((f & ~1) | 2);
+    }
+    const unsigned fb = __ballot_sync(kFull, first_pop);
+    if (first_pop) logb[klog + __popc(fb & ((1u << lane) - 1u))] = p_node;
+    klog += __popc(fb);
+    kq -= p_cnt;
+    __syncwarp();
+    if (p_np > 0) kq = ls_push_warp(E, s_pmv, p_np, p_qh, kq);
+    p_cnt = 0;
+  };
+  auto read_ahead = [&]() {  // (last warp) up to kAhead nodes from the head on
+    const int upto = min(kAhead, kq);
+    for (int o = kld; o < upto; o += 32) {
+      if (o + lane < upto) {
+        int idx = qh + o + lane;
+        if (idx >= n) idx -= n;
+        s_q[(qa + o + lane) & 127] = queue[idx];
+      }
+    }
+    kld = max(kld, upto);
+  };
+  // every thread: the exact queue length, and the nodes ahead of it
+  auto sync_queue = [&]() {
+    if (keeper) {
+      keep_pending();
+      kld = 0;
+      read_ahead();
+      if (lane == 0) {
+        s_qn = kq;
+        s_nlog = klog;
+      }
+    }
+    __syncthreads();
+    qn = s_qn;
+  };
+  sync_queue();
   for (;;) {
-    const int qh = s_qh, qn = s_qn, base = s_base;
-    if (qn == 0 || s_changes >= n) {
-      if (s_changes >= n || !verify || s_moves_round == 0) break;
+    if (qn == 0 || changes >= n) {
+      if (changes >= n || !verify || moves_round == 0) break;
       const int nl = s_nlog;  // verify round: queue again the nodes popped
       for (int i = tid; i < nl; i += blockDim.x) {
         const int x = logb[i];
@@ -285,149 +328,155 @@ __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int i
         flags[x] = 1;
       }
       __syncthreads();
-      if (tid < kWin) s_node[tid] = -1;  // the queue changed: no evaluation carries over
-      if (tid == 0) {
-        s_qh = 0; s_qn = nl; s_nlog = 0; s_moves_round = 0; s_base = 0;
-      }
-      __syncthreads();
+      qh = 0;
+      moves_round = 0;
+      have = 0;  // the queue changed: no evaluation carries over
+      kq = nl;
+      klog = 0;
+      sync_queue();
       continue;
     }
-    // window offset `lane` of every warp: its node, slot, and whether its
-    // evaluation is there and improves
+    // window offset `lane` of every warp: its node and slot
     const int R = qn < kWin ? qn : kWin;
-    const int slot = (base + lane) & (kWin - 1);
-    int node = -1;
-    bool have = false, impr = false;
-    if (lane < R) {
-      int idx = qh + lane;
-      if (idx >= n) idx -= n;
-      node = queue[idx];
-      have = s_node[slot] == node;
-      impr = have && s_gain[slot] > 0;
-    }
-    const unsigned bimp = __ballot_sync(kFull, impr);
-    const unsigned bmiss = __ballot_sync(kFull, lane < R && !have);
+    const unsigned live = R == 32 ? kFull : ((1u << R) - 1u);
+    const int slot = (qa + lane) & 31;
+    const int node = lane < R ? s_q[(qa + lane) & 127] : -1;
+    const unsigned bimp = __ballot_sync(kFull, ((have >> lane) & 1u) && s_gain[slot] > 0);
+    const unsigned bmiss = live & ~have;
     const int f = bimp ? __ffs(bimp) - 1 : R;
-    const unsigned before = f >= 32 ? kFull : ((1u << f) - 1u);
-    __syncthreads();  // every warp has decided (from the same slots) before any slot is written
-    if (bmiss & before) {  // an entry without an evaluation comes first: evaluate every such entry
-      const int my_node = __shfl_sync(kFull, node, w & 31);
-      const int my_slot = (base + w) & (kWin - 1);
-      if (w < R && ((bmiss >> w) & 1u)) {
-        int mv[8], mv3[6];
-        const int32_t g = eval_both(T, my_node, oropt != 0, mv);
-        int64_t g3 = 0;
-        // the 3-opt exchange only when neither 2-opt nor Or-opt improves
-        // (g is the warp's reduction: the branch is warp-uniform)
-        const bool try3 = init3 && g == 0;
-        if (try3) g3 = eval_or3(T, my_node, mv3);
-        if (lane < k) s_dep[my_slot][1 + lane] = T.pos_of(T.cand(my_node, lane));
-        if (lane == 0) {
-          s_dep[my_slot][0] = T.pos_of(my_node);
-          if (g3 > 0) {
-            s_gain[my_slot] = g3;
-            for (int t = 0; t < 6; ++t) s_mv[my_slot][t] = mv3[t];
-            s_mv[my_slot][7] = 2;
-          } else {
-            s_gain[my_slot] = g;
-            if (g > 0)
-              for (int t = 0; t < 8; ++t) s_mv[my_slot][t] = mv[t];
-          }
-          s_any[my_slot] = try3 ? 1 : 0;
-          s_node[my_slot] = my_node;
-        }
-      }
-      __syncthreads();
-    }
-    if (w == 0) {
-      const unsigned bal = __ballot_sync(kFull, lane < R && s_gain[slot] > 0);
-      const int first = bal ? __ffs(bal) - 1 : R;
-      const int cnt = bal ? first + 1 : R;  // queue entries popped this round
-      bool first_pop = false;
-      if (lane < cnt) {
-        const uint8_t fl = flags[node];
-        first_pop = !(fl & 2);
-        flags[node] = (uint8_t)((fl & ~1) | 2);
-      }
-      const unsigned fb = __ballot_sync(kFull, first_pop);
-      if (first_pop) logb[s_nlog + __popc(fb & ((1u << lane) - 1u))] = node;
-      const int win_slot = (base + first) & (kWin - 1);
-      __syncwarp();
-      if (lane < cnt && lane != first) s_node[slot] = -1;  // popped: the slots are free
+    const bool eval = (bmiss & ((1u << f) - 1u)) != 0;  // an entry without an evaluation comes first
+    if (keeper) {
+      keep_pending();
+      read_ahead();
+    } else if (eval && ((bmiss >> w) & 1u)) {
+      const int my_node = __shfl_sync(kFull, node, w);
+      const int my_slot = (qa + w) & 31;
+      int mv[8], mv3[6];
+      const int32_t g = eval_both(T, my_node, oropt != 0, mv);
+      int64_t g3 = 0;
+      // the 3-opt exchange only when neither 2-opt nor Or-opt improves
+      // (g is the warp's reduction: the branch is warp-uniform)
+      const bool try3 = init3 && g == 0;
+      if (try3) g3 = eval_or3(T, my_node, mv3);
+      if (lane < k) s_dep[my_slot][1 + lane] = T.pos_of(T.cand(my_node, lane));
       if (lane == 0) {
-        s_nlog += __popc(fb);
-        int h = qh + cnt;
-        if (h >= n) h -= n;
-        s_qh = h;
-        s_qn = qn - cnt;
-        s_base = (base + cnt) & (kWin - 1);
-        s_win = bal ? win_slot : -1;
-        s_log.count = 0;
+        s_dep[my_slot][0] = T.pos_of(my_node);
+        if (g3 > 0) {
+          s_gain[my_slot] = (int32_t)g3;
+          for (int t = 0; t < 6; ++t) s_mv[my_slot][t] = mv3[t];
+          s_mv[my_slot][7] = 2;
+        } else {
+          s_gain[my_slot] = g;
+          if (g > 0) {
+            for (int t = 0; t < 8; ++t) s_mv[my_slot][t] = mv[t];
+            s_ij[my_slot] = make_int2(T.pos_of(mv[1]), T.pos_of(mv[2]));
+          }
+        }
+        s_any[my_slot] = try3 ? 1 : 0;
       }
     }
-    __syncthreads();
-    const int win = s_win;
-    if (win >= 0) {
-      int mv[8];
-      for (int t = 0; t < 8; ++t) mv[t] = s_mv[win][t];
-      // the slot is free (its move is not overwritten before the next
-      // evaluation phase, several barriers on); the warp checking it below
-      // may still read the old node, which leaves the slot free either way
-      if (tid == 0) s_node[win] = -1;
-      if (mv[7] == 0) {
-        cta_flip(T, mv[1], mv[2], s_log);
-      } else if (mv[7] == 1) {
-        cta_move2(T, mv[0], mv[1], mv[4], mv[5], s_log);
-        cta_move2(T, mv[0], mv[4], mv[3], mv[2], s_log);
-        if (mv[6]) cta_move2(T, mv[4], mv[2], mv[1], mv[5], s_log);
-      } else {  // 3-opt exchange {a, t2, b, b', c, c'} as three edge exchanges
-        cta_move2(T, mv[0], mv[1], mv[2], mv[3], s_log);  // {a,t2},{b,b'} -> {a,b},{t2,b'}
-        cta_move2(T, mv[0], mv[2], mv[4], mv[5], s_log);  // {a,b},{c,c'} -> {a,c},{b,c'}
-        cta_move2(T, mv[0], mv[4], mv[3], mv[1], s_log);  // {a,c},{b',t2} -> {a,b'},{c,t2}
-      }
-      // drop the evaluations that read a reversed position (warp w checks slot w)
-      {
-        const int sn = s_node[w];
-        if (sn >= 0) {
-          const int ns = s_log.count;
-          bool hit = s_any[w] != 0;
-          if (lane < k) {
-            const int tb = s_dep[w][1 + lane];
-            for (int q = 0; q < ns && !hit; ++q) {
-              const int2 sp = s_log.span[q];
-              hit = in_span(tb, sp, n) || in_span(tb == 0 ? n - 1 : tb - 1, sp, n) ||
-                    in_span(tb + 1 == n ? 0 : tb + 1, sp, n);
-            }
-          }
-          if (lane == 31 && !hit) {
-            const int t0 = s_dep[w][0];
-            for (int q = 0; q < ns && !hit; ++q) {
-              const int2 sp = s_log.span[q];
-              for (int d = -1; d <= 3 && !hit; ++d) {
-                int p = t0 + d;
-                if (p < 0) p += n;
-                if (p >= n) p -= n;
-                hit = in_span(p, sp, n);
-              }
-            }
-          }
-          if (__any_sync(kFull, hit) && lane == 0) s_node[w] = -1;
-        }
-      }
-      if (w == 0) {
-        const int qn2 = ls_push_warp(E, mv, mv[7] == 0 ? 4 : 6, s_qh, s_qn);  // 2-opt: 4 ends, else 6
-        if (lane == 0) {
-          s_qn = qn2;
-          s_changes++;
-          s_moves_round++;
-        }
-      }
+    if (eval) {
       __syncthreads();
+      have |= bmiss;
+    }
+    const unsigned bal = __ballot_sync(kFull, ((have >> lane) & 1u) && s_gain[slot] > 0);
+    const int first = bal ? __ffs(bal) - 1 : R;
+    const int cnt = bal ? first + 1 : R;  // queue entries popped this round
+    if (keeper) {
+      p_cnt = cnt;
+      p_node = node;
+      p_np = 0;
+      p_qh = qh + cnt;
+      if (p_qh >= n) p_qh -= n;
+      kld -= cnt;
+    }
+    if (bal) {
+      const int win = (qa + first) & 31;
+      const int kind = s_mv[win][7];
+      if (keeper) {
+        p_np = kind == 0 ? 4 : 6;
+        if (lane < 8) s_pmv[lane] = s_mv[win][lane];
+        __syncwarp();
+      }
+      // the entry of window offset w: does a reversed position matter to it?
+      const int ws = (qa + w) & 31;
+      const bool mine = w > first && w < R && ((have >> w) & 1u);
+      bool hit = mine && s_any[ws] != 0;
+      const int dep = mine ? (lane < k ? s_dep[ws][1 + lane] : s_dep[ws][0]) : 0;
+      const int dn = mine ? s_dep[ws][0] : 0;
+      auto meets = [&](Span sp) {
+        // a candidate's position and its two neighbours: dep - 1 .. dep + 1
+        int d = dep + 1 - sp.i;
+        if (d < 0) d += n;
+        if (d >= n) d -= n;
+        if (lane < k && d < sp.L + 2) hit = true;
+        // the node's: dn - 1 .. dn + 3
+        d = dn + 3 - sp.i;
+        while (d < 0) d += n;
+        while (d >= n) d -= n;
+        if (d < sp.L + 4) hit = true;
+      };
+      if (kind == 0) {
+        const int2 ij = s_ij[win];
+        const Span sp = flip_span(ij.x, ij.y, n);
+        if (mine) meets(sp);
+        cta_reverse(T, sp);
+      } else {
+        // two or three edge exchanges {n1,n2},{n3,n4} -> {n1,n3},{n2,n4}
+        //   Or-opt {p,a,e,q,u,v,kept}; 3-opt {a,t2,b,b',c,c'}:
+        //   {a,t2},{b,b'} -> {a,b},{t2,b'}; {a,b},{c,c'} -> {a,c},{b,c'}; {a,c},{b',t2} -> {a,b'},{c,t2}
+        const int* mv = s_mv[win];
+        const int steps = kind == 1 ? (mv[6] ? 3 : 2) : 3;
+        for (int st = 0; st < steps; ++st) {
+          int n1, n2, n3, n4;
+          if (kind == 1) {
+            n1 = st == 2 ? mv[4] : mv[0];
+            n2 = st == 0 ? mv[1] : (st == 1 ? mv[4] : mv[2]);
+            n3 = st == 0 ? mv[4] : (st == 1 ? mv[3] : mv[1]);
+            n4 = st == 1 ? mv[2] : mv[5];
+          } else {
+            n1 = mv[0];
+            n2 = st == 0 ? mv[1] : (st == 1 ? mv[2] : mv[4]);
+            n3 = st == 0 ? mv[2] : (st == 1 ? mv[4] : mv[3]);
+            n4 = st == 0 ? mv[3] : (st == 1 ? mv[5] : mv[1]);
+          }
+          const bool fwd = T.succ(n1) == n2;
+          const int i = T.pos_of(fwd ? n2 : n1), j = T.pos_of(fwd ? n3 : n4);
+          __syncthreads();  // every thread has read the tour before a position moves
+          const Span sp = flip_span(i, j, n);
+          if (mine) meets(sp);
+          cta_reverse(T, sp);
+          if (st + 1 < steps) __syncthreads();
+        }
+      }
+      const bool any = __any_sync(kFull, hit);
+      if (lane == 0) s_inv[par][w] = any ? 1 : 0;
+      ++changes;
+      ++moves_round;
+    }
+    __syncthreads();  // the tour, s_inv and the nodes read ahead are there; s_gain and s_mv were read
+    if (bal) {
+      have &= ~__ballot_sync(kFull, s_inv[par][lane] != 0);
+      par ^= 1;
+    }
+    have = cnt >= 32 ? 0u : have >> cnt;
+    qa += cnt;
+    qh += cnt;
+    if (qh >= n) qh -= n;
+    qn -= cnt;
+    if (qn < kAhead) sync_queue();
+  }
+  __syncthreads();
+  if (keeper) {
+    keep_pending();
+    if (lane == 0) {
+      s_qn = kq;
+      s_nlog = klog;
     }
   }
   __syncthreads();
-  const int qh = s_qh, qn = s_qn, nl = s_nlog;
-  for (int t = tid; t < qn; t += blockDim.x) {
+  const int ql = s_qn, nl = s_nlog;
+  for (int t = tid; t < ql; t += blockDim.x) {
     int i = qh + t;
     if (i >= n) i -= n;
     flags[queue[i]] = 0;
