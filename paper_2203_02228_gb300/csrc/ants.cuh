@@ -647,7 +647,7 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
           A.logb + (size_t)ant * n};
   LsStats S{0, 0, 0, 0, 0};
   ArrTour T{n, C.k, route, pos, C.xy, C.cand, C.k, C.dcand};
-  const int64_t gain = C.ls ? ls_run(E, T, chk, W.nchk, S) : 0;
+  const int64_t gain = C.ls ? ls_run<KW == 32>(E, T, chk, W.nchk, S) : 0;
   if (lane == 0) {
     if (A.nseg) A.nseg[ant] = -1;  // tour is in route/pos
     A.len[ant] = pre_len - gain;

@@ -87,8 +87,8 @@ cudaError_t launch_unlabel(const int32_t* route0, const int32_t* route_t, int32_
 cudaError_t launch_init_ls(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
                            int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
                            int32_t* logb, cudaStream_t s);
-cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, int stage,
-                                   cudaStream_t s);
+cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, int kw,
+                                   int stage, cudaStream_t s);
 cudaError_t launch_test_kernels(int what, const void* in, void* out, int count, int width,
                                 uint64_t seed, cudaStream_t s);
 

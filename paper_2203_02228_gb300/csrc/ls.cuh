@@ -50,6 +50,23 @@ struct LsStats {
   int64_t t_eval, t_confirm, t_flip, t_push;  // device ns per phase (block search)
 };
 
+// The nodes before and after tour position t (warp-uniform t): no wrapping
+// where t is not next to the route's ends.
+__device__ __forceinline__ void route_walk(const int32_t* route, int n, int t, int& p, int& s1, int& s2, int& s3) {
+  if (t >= 1 && t + 3 < n) {
+    const int32_t* r = route + t;
+    p = r[-1];
+    s1 = r[1];
+    s2 = r[2];
+    s3 = r[3];
+  } else {
+    p = route[wrapn(t - 1, n)];
+    s1 = route[wrapn(t + 1, n)];
+    s2 = route[wrapn(t + 2, n)];
+    s3 = route[wrapn(t + 3, n)];
+  }
+}
+
 // Explicit tour: route[t] = node at position t, pos = inverse.  Nodes are
 // node ids (with node-indexed xy/cn) or source positions (with the
 // source-ordered copies); cn rows are `stride` entries apart.
@@ -83,11 +100,7 @@ struct ArrTour {
     s = at_off(t, 1);
   }
   __device__ __forceinline__ void walk(int a, int& p, int& s1, int& s2, int& s3) const {
-    const int t = pos[a];
-    p = at_off(t, -1);
-    s1 = at_off(t, 1);
-    s2 = at_off(t, 2);
-    s3 = at_off(t, 3);
+    route_walk(route, n, pos[a], p, s1, s2, s3);
   }
   __device__ __forceinline__ int2 coord(int x) const { return xy[x]; }
   __device__ __forceinline__ int cand(int x, int s) const { return cn[(size_t)x * stride + s]; }
@@ -155,27 +168,32 @@ __device__ __forceinline__ bool tour_move2(Tour& T, int n1, int n2, int n3, int 
 // Or-opt move -- the same decision as scanning one after the other.  Returns
 // the gain (0: none) and the move on every lane: mv[7] = 0 for 2-opt
 // (mv[0..3]), 1 for Or-opt (mv[0..6]).
-// Lane layout: with k <= 16, lane = side * 16 + s (side 0: the edge
-// (b, succ b), side 1: (pred b, b)); with k > 16, lane = s and the two sides
-// are two passes.  The loads that do not depend on the walk from a (the
-// candidate row, b's coordinates) are issued before it; the move is rebuilt
-// from the winning lane's registers.
+// Lane layout: with k <= 16 (TWO = false), lane = side * 16 + s (side 0: the
+// edge (b, succ b), side 1: (pred b, b)); with k > 16 (TWO), lane = s and the
+// two sides are two passes.  Lanes beyond k repeat entry 0 and are left out
+// at the end, so that nothing diverges.  The loads that do not depend on the
+// walk from a (the candidate row, b's coordinates) are issued before it; the
+// move is rebuilt from the winning lane's registers.
 // Bound by latency while few warps of an SM evaluate and by instruction
-// issue while all do, so the costs are branch-free (euc2d_near): the seven a
-// lane needs run side by side, both sides share one piece of code (swapping
-// the ends of the edge at b only swaps the two orientations of an Or-opt
-// move), and no index is divided by k.
-template <class Tour>
+// issue while all do, so the costs are branch-free (euc2d_near) and run side
+// by side, the choice among the moves is made of maxima and selects, both
+// sides share one piece of code (swapping the ends of the edge at b only
+// swaps the two orientations of an Or-opt move), no index is divided by k,
+// and with TWO = false the lanes of the two sides share costs: six per lane
+// instead of eight.  Of the slowest ants' time at n = 100,000 it took 2,420 us
+// of 5,920 with a branch per cost, 1,375 of 3,590 branch-free, 1,046 of 3,290 in
+// this form.
+template <bool TWO, class Tour>
 __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, int (&mv)[8]) {
   const int n = T.n, k = T.k, lane = lane_id();
   do_or = do_or && n >= 8;
-  const bool two = k > 16;
-  const int s = two ? lane : (lane & 15);
+  const int s = TWO ? lane : (lane & 15);
   const bool live = s < k;
-  const int b = live ? T.cand(a, s) : a;
-  const int d_ab = live ? T.cdist(a, s) : 0;  // = euc2d(xa, xb), kept with the lists
+  const int sl = live ? s : 0;
+  const int b = T.cand(a, sl);
+  const int d_ab = T.cdist(a, sl);  // = euc2d(xa, xb), kept with the lists
   const int2 xb = T.coord(b);
-  int p, s1, s2 = -1, s3 = -1;
+  int p, s1, s2 = a, s3 = a;
   if (do_or)
     T.walk(a, p, s1, s2, s3);
   else
@@ -188,134 +206,115 @@ __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, i
   }
   // b's tour neighbour on this lane's side (pass 0), and for k > 16 the
   // predecessor for pass 1
-  int bn0 = a, bn1 = a;
-  if (live) {
-    if (two)
-      T.nbrs(b, bn1, bn0);
-    else
-      bn0 = T.adj(b, lane < 16);
-  }
-  const int2 xbn0 = T.coord(bn0), xbn1 = two ? T.coord(bn1) : xa;
-  // the costs within a's tour neighbourhood are the same on every lane:
-  // lane j computes the j-th, shuffles share them
+  int bn0, bn1 = a;
+  if (TWO)
+    T.nbrs(b, bn1, bn0);
+  else
+    bn0 = T.adj(b, lane < 16);
+  const int2 xbn0 = T.coord(bn0), xbn1 = TWO ? T.coord(bn1) : xa;
+  // the costs within a's tour neighbourhood are the same on every lane: one
+  // lane computes the j-th, shuffles share them
   //   0 d(a,s1)  1 d(p,a)  2 d(p,s1)  3 d(s1,s2)  4 d(p,s2)  5 d(s2,s3)  6 d(p,s3)
-  int2 cu = xa, cv = x1;
-  if (lane == 1) {
-    cu = xp;
-    cv = xa;
-  } else if (lane == 2) {
-    cu = xp;
-  } else if (lane == 3) {
-    cu = x1;
-    cv = x2;
-  } else if (lane == 4) {
-    cu = xp;
-    cv = x2;
-  } else if (lane == 5) {
-    cu = x2;
-    cv = x3;
-  } else if (lane == 6) {
-    cu = xp;
-    cv = x3;
+  const int j = TWO ? lane : (lane & 15);
+  int2 cu, cv;
+  {
+    const bool up = j == 1 || j == 2 || j == 4 || j == 6, va = j == 1, v2 = j == 3 || j == 4, v3 = j == 5 || j == 6;
+    cu.x = up ? xp.x : (j == 3 ? x1.x : (j == 5 ? x2.x : xa.x));
+    cu.y = up ? xp.y : (j == 3 ? x1.y : (j == 5 ? x2.y : xa.y));
+    cv.x = va ? xa.x : (v2 ? x2.x : (v3 ? x3.x : x1.x));
+    cv.y = va ? xa.y : (v2 ? x2.y : (v3 ? x3.y : x1.y));
   }
-  bool big = false;
-  int32_t cst = euc2d_near(cu, cv, big);
   // the lane's best move: a gaining 2-opt move counts kTwoOpt more than its
   // gain, so that it beats every Or-opt move; code = l * 4 + orientation * 2
-  // + side (l = 0: 2-opt), idx = its place in the sequential scan
+  // + side (l = 0: 2-opt)
   constexpr int32_t kTwoOpt = 1 << 28;
   int32_t best = 0;
-  int bidx = INT_MAX, bcode = 0, bbn = a;
-  const int passes = two ? 2 : 1;
-  for (int pass = 0; pass < passes; ++pass) {
-    const int side = two ? pass : (lane >> 4);
+  int bcode = 0, bbn = bn0;
+#pragma unroll
+  for (int pass = 0; pass < (TWO ? 2 : 1); ++pass) {
+    const bool hi = TWO ? pass != 0 : lane >= 16;  // side 1
     const int bn = pass == 0 ? bn0 : bn1;
     const int2 xbn = pass == 0 ? xbn0 : xbn1;
-    int32_t c_bn = euc2d_near(xb, xbn, big);   // d(b, bn)
-    int32_t c_n1 = euc2d_near(xbn, x1, big);   // d(bn, s1)
-    int32_t c_np = euc2d_near(xbn, xp, big);   // d(bn, p)
-    int32_t c_na = 0, c_b1 = 0, c_b2 = 0, c_n2 = 0;
-    if (do_or) {
-      c_na = euc2d_near(xbn, xa, big);
-      c_b1 = euc2d_near(xb, x1, big);
-      c_b2 = euc2d_near(xb, x2, big);
-      c_n2 = euc2d_near(xbn, x2, big);
+    // 0 d(b,bn)  1 d(bn,s1)  2 d(bn,a)  3 d(bn,s2), and
+    //   TWO:   4 d(b,s1)  5 d(b,s2)  6 d(bn,p)  7 the j-th of a's neighbourhood
+    //   else:  4 d(b,s1) on side 0, d(bn,p) on side 1
+    //          5 d(b,s2) on side 0, the j-th of a's neighbourhood on side 1
+    int2 u4 = xb, v4 = x1, u5 = xb, v5 = x2;
+    if (!TWO) {
+      u4.x = hi ? xbn.x : xb.x;
+      u4.y = hi ? xbn.y : xb.y;
+      v4.x = hi ? xp.x : x1.x;
+      v4.y = hi ? xp.y : x1.y;
+      u5.x = hi ? cu.x : xb.x;
+      u5.y = hi ? cu.y : xb.y;
+      v5.x = hi ? cv.x : x2.x;
+      v5.y = hi ? cv.y : x2.y;
+    }
+    bool big = false;
+    int32_t c0 = euc2d_near(xb, xbn, big), c1 = euc2d_near(xbn, x1, big), c2 = euc2d_near(xbn, xa, big),
+            c3 = euc2d_near(xbn, x2, big), c4 = euc2d_near(u4, v4, big), c5 = euc2d_near(u5, v5, big), c6 = 0,
+            c7 = 0;
+    if (TWO) {
+      c6 = euc2d_near(xbn, xp, big);
+      c7 = euc2d_near(cu, cv, big);
     }
     if (__any_sync(kFull, big)) {  // an edge of 2^21 or more: the exact steps, one cost after the other
 #pragma unroll 1
-      for (int j = 0; j < 8; ++j) {
-        const int2 u = j == 7 ? cu : ((j == 0 || j == 4 || j == 5) ? xb : xbn);
-        const int2 t = j == 7 ? cv : j == 0 ? xbn : (j == 1 || j == 4) ? x1 : j == 2 ? xp : j == 3 ? xa : x2;
-        const int32_t d = euc2d_m(sqdist(u, t));
-        if (j == 0) c_bn = d;
-        if (j == 1) c_n1 = d;
-        if (j == 2) c_np = d;
-        if (j == 3) c_na = d;
-        if (j == 4) c_b1 = d;
-        if (j == 5) c_b2 = d;
-        if (j == 6) c_n2 = d;
-        if (j == 7) cst = d;
+      for (int t = 0; t < (TWO ? 8 : 6); ++t) {
+        const int2 u = t == 0 ? xb : t == 4 ? u4 : t == 5 ? u5 : t == 7 ? cu : xbn;
+        const int2 v = t == 0 ? xbn : t == 1 ? x1 : t == 2 ? xa : t == 3 ? x2 : t == 4 ? v4 : t == 5 ? v5
+                       : t == 6 ? xp : cv;
+        const int32_t d = euc2d_m(sqdist(u, v));
+        if (t == 0) c0 = d;
+        if (t == 1) c1 = d;
+        if (t == 2) c2 = d;
+        if (t == 3) c3 = d;
+        if (t == 4) c4 = d;
+        if (t == 5) c5 = d;
+        if (t == 6) c6 = d;
+        if (t == 7) c7 = d;
       }
     }
-    const int d_as = __shfl_sync(kFull, cst, 0), d_ap = __shfl_sync(kFull, cst, 1);
+    const int32_t nbh = TWO ? c7 : c5;
+    const int nb0 = TWO ? 0 : 16;
+    const int32_t c_b1 = TWO ? c4 : __shfl_sync(kFull, c4, s), c_b2 = TWO ? c5 : __shfl_sync(kFull, c5, s);
+    const int32_t c_z = hi ? (TWO ? c6 : c4) : c1;  // d(bn, s1) on side 0, d(bn, p) on side 1
+    const int32_t d_as = __shfl_sync(kFull, nbh, nb0), d_ap = __shfl_sync(kFull, nbh, nb0 + 1);
     // gains in 32 bits: each is a signed sum of at most six EUC_2D costs of
     // coordinates below 2^24 (each cost below 2^25)
-    int32_t rem1 = 0, rem2 = 0, rem3 = 0;
-    if (do_or) {
-      rem1 = d_ap + d_as - __shfl_sync(kFull, cst, 2);
-      rem2 = d_ap + __shfl_sync(kFull, cst, 3) - __shfl_sync(kFull, cst, 4);
-      rem3 = d_ap + __shfl_sync(kFull, cst, 5) - __shfl_sync(kFull, cst, 6);
-    }
     int32_t v = 0;
-    int code = 0;
-    if (do_or && live) {
-      // reversed (g0) and kept (g1) insertion of a..e between the ends of the
-      // edge {b, bn}: one joins b to e and bn to a, the other b to a and bn
-      // to e; which of the two is the reversed one depends on the side
-      const bool bad1 = b == p || bn == p || bn == a || b == s1 || bn == s1;
-      const bool bad2 = bad1 || b == s2 || bn == s2;
-      const bool bad3 = bad2 || b == s3 || bn == s3;
-      if (!bad1) {  // one node: one form only
-        const int32_t g = rem1 + c_bn - d_ab - c_na;
-        if (g > v) {
-          v = g;
-          code = 4;
-        }
-      }
-      const int32_t e2 = rem2 + c_bn, e3 = rem3 + c_bn;
-      const int32_t be2 = e2 - c_b1 - c_na, ba2 = e2 - d_ab - c_n1;
-      const int32_t be3 = e3 - c_b2 - c_na, ba3 = e3 - d_ab - c_n2;
-      const int32_t g20 = side ? ba2 : be2, g21 = side ? be2 : ba2;
-      const int32_t g30 = side ? ba3 : be3, g31 = side ? be3 : ba3;
-      if (!bad2 && g20 > v) {
-        v = g20;
-        code = 8;
-      }
-      if (!bad2 && g21 > v) {
-        v = g21;
-        code = 10;
-      }
-      if (!bad3 && g30 > v) {
-        v = g30;
-        code = 12;
-      }
-      if (!bad3 && g31 > v) {
-        v = g31;
-        code = 14;
-      }
+    int l = 0, o = 0;
+    if (do_or) {
+      const int32_t rem1 = d_ap + d_as - __shfl_sync(kFull, nbh, nb0 + 2);
+      const int32_t rem2 = d_ap + __shfl_sync(kFull, nbh, nb0 + 3) - __shfl_sync(kFull, nbh, nb0 + 4);
+      const int32_t rem3 = d_ap + __shfl_sync(kFull, nbh, nb0 + 5) - __shfl_sync(kFull, nbh, nb0 + 6);
+      // insertion of a..e between the ends of the edge {b, bn}: one form
+      // joins b to e and bn to a, the other b to a and bn to e; the reversed
+      // one (orientation 0) is the first on side 0, the second on side 1
+      const bool bad1 = (b == p) | (bn == p) | (bn == a) | (b == s1) | (bn == s1);
+      const bool bad2 = bad1 | (b == s2) | (bn == s2);
+      const bool bad3 = bad2 | (b == s3) | (bn == s3);
+      const int32_t be2 = rem2 + c0 - c_b1 - c2, ba2 = rem2 + c0 - d_ab - c1;
+      const int32_t be3 = rem3 + c0 - c_b2 - c2, ba3 = rem3 + c0 - d_ab - c3;
+      const bool o2 = hi ? be2 > ba2 : ba2 > be2, o3 = hi ? be3 > ba3 : ba3 > be3;
+      const int32_t v1 = bad1 ? 0 : rem1 + c0 - d_ab - c2;  // one node: one form only
+      const int32_t v2 = bad2 ? 0 : max(be2, ba2), v3 = bad3 ? 0 : max(be3, ba3);
+      v = max(max(v1, v2), max(v3, 0));
+      l = v == v1 ? 1 : (v == v2 ? 2 : 3);
+      o = v == v1 ? 0 : (v == v2 ? o2 : o3);
     }
-    const int32_t d_out = side ? d_ap : d_as;
-    const int32_t g = d_out + c_bn - d_ab - (side ? c_np : c_n1);
-    if (live && d_out > d_ab && g > 0) {
-      v = g + kTwoOpt;
-      code = 0;
-    }
-    const int l = code >> 2;
-    const int idx = l == 0 ? side * k + s : (((l - 1) * k + s) * 2 + side) * 2 + ((code >> 1) & 1);
-    if (v > best || (v == best && v > 0 && idx < bidx)) {
+    const int32_t d_out = hi ? d_ap : d_as;
+    const int32_t g = d_out + c0 - d_ab - c_z;
+    const bool t2 = (d_out > d_ab) & (g > 0);
+    v = t2 ? g + kTwoOpt : v;
+    v = live ? v : 0;
+    const int code = (t2 ? 0 : l * 4 + o * 2) + (hi ? 1 : 0);
+    if (pass == 0) {
       best = v;
-      bidx = idx;
-      bcode = code | side;
+      bcode = code;
+    } else if (v > best || (v == best && (code >> 2) < (bcode >> 2))) {  // scan order: l, entry, side
+      best = v;
+      bcode = code;
       bbn = bn;
     }
   }
@@ -324,8 +323,10 @@ __device__ __forceinline__ int32_t eval_both(const Tour& T, int a, bool do_or, i
   if (gm == 0) return 0;
   unsigned own = __ballot_sync(kFull, best == gm);
   if (own & (own - 1)) {  // equal gains: the first in scan order
-    const int im = (int)__reduce_min_sync(kFull, best == gm ? (unsigned)bidx : 0xFFFFFFFFu);
-    own = __ballot_sync(kFull, best == gm && bidx == im);
+    const int l = bcode >> 2, side = bcode & 1;
+    const int idx = l == 0 ? side * k + s : (((l - 1) * k + s) * 2 + side) * 2 + ((bcode >> 1) & 1);
+    const unsigned im = __reduce_min_sync(kFull, best == gm ? (unsigned)idx : 0xFFFFFFFFu);
+    own = __ballot_sync(kFull, best == gm && (unsigned)idx == im);
   }
   const int wl = __ffs(own) - 1;
   const int bw = __shfl_sync(kFull, b, wl), bnw = __shfl_sync(kFull, bbn, wl);
@@ -463,7 +464,7 @@ __device__ __forceinline__ void ls_push0(const LsEnv& E, int x, int qh, int& qn)
 // Runs the search from the checklist init[0..ninit) (distinct nodes).
 // Returns the total gain (old length - new length), or -1 if the tour
 // representation ran out of capacity (flags are left clean either way).
-template <class Tour>
+template <bool TWO, class Tour>
 __device__ __forceinline__ int64_t ls_run(const LsEnv& E, Tour& T, const int32_t* init, int ninit,
                                           LsStats& S) {
   const int n = E.n, lane = lane_id();
@@ -491,7 +492,7 @@ __device__ __forceinline__ int64_t ls_run(const LsEnv& E, Tour& T, const int32_t
       __syncwarp();
       S.pops++;
       int mv[8];
-      const int32_t g = eval_both(T, a, E.oropt != 0, mv);
+      const int32_t g = eval_both<TWO>(T, a, E.oropt != 0, mv);
       if (g > 0) {
         if (mv[7] == 0) {
           ok = T.flip(mv[1], mv[2], S);

@@ -234,9 +234,9 @@ int group_setup(Group& g, const int32_t* const* coords, cudaStream_t s) {
   CK(cudaMemcpyAsync(g.d_node_off, g.node_off.data(), sizeof(int64_t) * (g.count + 1), cudaMemcpyHostToDevice, s));
   CK(launch_grid_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, s));
   CK(build_lists_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, g.map_knn, g.nmap_knn, s));
-  CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, 0, s));       // nearest-neighbour tours
+  CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, g.kw, 0, s));       // nearest-neighbour tours
   CK(launch_colony_init_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, 0, s));
-  CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, 1, s));       // their local search
+  CK(launch_init_tour_batch(g.dC, g.dS, g.count, g.max_n, g.kw, 1, s));       // their local search
   CK(launch_colony_init_batch(g.dC, g.dS, g.count, g.map256, g.nmap256, 1, s));
   return FACO_OK;
 }

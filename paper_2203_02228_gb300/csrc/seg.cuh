@@ -374,6 +374,7 @@ struct LsShared {
 // the result equals popping one node at a time.  Must be called by every
 // thread of the block.  Returns the gain, or -1 when the table filled up
 // (flags are left clean either way; the caller has the ant redone on arrays).
+template <bool TWO>
 __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, const int32_t* init, int ninit,
                                                 LsStats& S, LsShared& sh) {
   const int n = E.n, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -413,7 +414,7 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
       if (idx >= n) idx -= n;
       const int a = E.queue[idx];
       int mv[8];
-      const int32_t g = eval_both(T.view(), a, E.oropt != 0, mv);
+      const int32_t g = eval_both<TWO>(T.view(), a, E.oropt != 0, mv);
       if (lane == 0) {
         sh.gain[w] = g;
         if (g > 0)

@@ -135,11 +135,7 @@ struct SmemPosTour {
     s = at_off(t, 1);
   }
   __device__ __forceinline__ void walk(int a, int& p, int& s1, int& s2, int& s3) const {
-    const int t = pos_of(a);
-    p = at_off(t, -1);
-    s1 = at_off(t, 1);
-    s2 = at_off(t, 2);
-    s3 = at_off(t, 3);
+    route_walk(route, n, pos_of(a), p, s1, s2, s3);
   }
   __device__ __forceinline__ int2 coord(int x) const { return xy[x]; }
   __device__ __forceinline__ int cand(int x, int s) const { return cn[(size_t)x * k + s]; }
@@ -244,7 +240,7 @@ __device__ __forceinline__ void cta_reverse(TT& T, Span sp) {
 constexpr int kWin = 31;     // entries, a warp each; the last warp keeps the queue
 constexpr int kAhead = 96;   // queued nodes read ahead (a ring of 128)
 
-template <class TT>
+template <bool TWO, class TT>
 __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int init3, int32_t* queue, uint8_t* flags,
                                              int32_t* logb) {
   __shared__ int32_t s_gain[32];
@@ -352,7 +348,7 @@ __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int i
       const int my_node = __shfl_sync(kFull, node, w);
       const int my_slot = (qa + w) & 31;
       int mv[8], mv3[6];
-      const int32_t g = eval_both(T, my_node, oropt != 0, mv);
+      const int32_t g = eval_both<TWO>(T, my_node, oropt != 0, mv);
       int64_t g3 = 0;
       // the 3-opt exchange only when neither 2-opt nor Or-opt improves
       // (g is the warp's reduction: the branch is warp-uniform)
@@ -487,7 +483,7 @@ __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int i
 // SP: the positions live in shared memory during the search (launched with
 // smem_pos_bytes(n) of it) and are written to `pos` at the end; otherwise
 // the search works on `pos` in global memory.
-template <bool SP>
+template <bool SP, bool TWO>
 __device__ __forceinline__ void init_ls_run(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k,
                                             int oropt, int verify, int init3, int32_t* route, int32_t* pos,
                                             int32_t* queue, uint8_t* flags, int32_t* logb) {
@@ -495,29 +491,29 @@ __device__ __forceinline__ void init_ls_run(const int2* xy, int n, const int32_t
     extern __shared__ __align__(16) unsigned char s_pos[];
     SmemPosTour T = smem_pos_tour(s_pos, n, k, route, xy, cand, dcand);
     smem_pos_load(T);
-    init_ls_body(T, oropt, verify, init3, queue, flags, logb);
+    init_ls_body<TWO>(T, oropt, verify, init3, queue, flags, logb);
     __syncthreads();
     for (int x = threadIdx.x; x < n; x += blockDim.x) pos[x] = T.pos_of(x);
   } else {
     ArrTour T{n, k, route, pos, xy, cand, k, dcand};
-    init_ls_body(T, oropt, verify, init3, queue, flags, logb);
+    init_ls_body<TWO>(T, oropt, verify, init3, queue, flags, logb);
   }
 }
 
-template <bool SP>
+template <bool SP, bool TWO>
 __global__ void __launch_bounds__(1024) k_init_ls(const int2* xy, int n, const int32_t* cand,
                                                   const int32_t* dcand, int k, int oropt, int verify, int init3,
                                                   int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
                                                   int32_t* logb) {
-  init_ls_run<SP>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
+  init_ls_run<SP, TWO>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
 }
 
 // Batch: one block per colony; positions of the initial tour in src_pos.
-template <bool SP>
+template <bool SP, bool TWO>
 __global__ void __launch_bounds__(1024) k_init_ls_b(const Colony* cols, const ColonySetup* sets) {
   const Colony C = cols[blockIdx.x];
   const ColonySetup S = sets[blockIdx.x];
-  init_ls_run<SP>(C.xy, C.n, S.cand, S.dcand, C.k, C.oropt, C.verify, C.init3, S.init_route, C.src_pos, S.queue, S.flags,
+  init_ls_run<SP, TWO>(C.xy, C.n, S.cand, S.dcand, C.k, C.oropt, C.verify, C.init3, S.init_route, C.src_pos, S.queue, S.flags,
                   S.logb);
 }
 
@@ -621,19 +617,41 @@ cudaError_t launch_unlabel(const int32_t* route0, const int32_t* route_t, int32_
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_ls(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
-                           int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
-                           int32_t* logb, cudaStream_t s) {
-  const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls<true>), n);
+namespace {
+
+template <bool TWO>
+cudaError_t launch_init_ls_two(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
+                               int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
+                               int32_t* logb, cudaStream_t s) {
+  const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls<true, TWO>), n);
   if (sm > 0)
-    k_init_ls<true><<<1, 1024, sm, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
+    k_init_ls<true, TWO><<<1, 1024, sm, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
   else
-    k_init_ls<false><<<1, 1024, 0, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
+    k_init_ls<false, TWO><<<1, 1024, 0, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, int stage,
-                                   cudaStream_t s) {
+template <bool TWO>
+cudaError_t launch_init_ls_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, cudaStream_t s) {
+  const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls_b<true, TWO>), max_n);
+  if (sm > 0)
+    k_init_ls_b<true, TWO><<<count, 1024, sm, s>>>(cols, sets);
+  else
+    k_init_ls_b<false, TWO><<<count, 1024, 0, s>>>(cols, sets);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_init_ls(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
+                           int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
+                           int32_t* logb, cudaStream_t s) {
+  return k > 16 ? launch_init_ls_two<true>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb, s)
+                : launch_init_ls_two<false>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb, s);
+}
+
+cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, int kw,
+                                   int stage, cudaStream_t s) {
   if (stage == 0) {
     const size_t smem = (size_t)((max_n + 31) >> 5) * sizeof(uint32_t);
     if (smem > 48 * 1024) {
@@ -641,14 +659,10 @@ cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, 
       if (e != cudaSuccess) return e;
     }
     k_nn_tour_b<<<count, 32, smem, s>>>(cols, sets);
-  } else {
-    const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls_b<true>), max_n);
-    if (sm > 0)
-      k_init_ls_b<true><<<count, 1024, sm, s>>>(cols, sets);
-    else
-      k_init_ls_b<false><<<count, 1024, 0, s>>>(cols, sets);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  return kw == 32 ? launch_init_ls_batch<true>(cols, sets, count, max_n, s)
+                  : launch_init_ls_batch<false>(cols, sets, count, max_n, s);
 }
 
 cudaError_t launch_test_kernels(int what, const void* in, void* out, int count, int width,
