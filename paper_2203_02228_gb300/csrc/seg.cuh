@@ -37,24 +37,10 @@ struct Seg {
 };
 
 // Shared memory of a table of `cap` segments: two buffers of cap + 1
-// boundaries, 16 bytes each, then the count and the buffer in use.
+// boundaries, 16 bytes each.
 constexpr size_t kSegBytes = 2 * (sizeof(int2) + 2 * sizeof(int32_t));
 static_assert(kSegBytes == 2 * sizeof(Seg), "construction's list of runs takes one buffer's room");
-__host__ __device__ constexpr size_t segtab_bytes(int cap) { return (size_t)(cap + 1) * kSegBytes + 16; }
-
-struct SegTab {
-  char* mem;         // buffers 0 and 1
-  int32_t* hdr;      // [0] segments, [1] buffer in use
-  int cap;
-};
-
-__device__ __forceinline__ SegTab segtab_at(char* base, int cap) {
-  SegTab T;
-  T.mem = base;
-  T.hdr = reinterpret_cast<int32_t*>(base + (size_t)(cap + 1) * kSegBytes);
-  T.cap = cap;
-  return T;
-}
+__host__ __device__ constexpr size_t segtab_bytes(int cap) { return (size_t)(cap + 1) * kSegBytes; }
 
 // Table capacity once the visited bits in front of a table of `cap`
 // segments are free (the local search does not need them): the same
@@ -185,25 +171,32 @@ struct SegView {
   }
 };
 
+// Segments in the table and the buffer they are in: the same on every thread
+// that changes the tour, kept in registers.
+struct SegState {
+  int S, cur;
+};
+
 // Tour over the segment table: what changes it.
 struct SegTour {
   int n, k, kw;
-  SegTab T;
+  char* mem;            // buffers 0 and 1
+  int cap;
   const int2* xy;
   const int32_t* cn;
   const int32_t* cd;
 
   __device__ __forceinline__ char* buffer(int which) const {
-    return T.mem + (which ? (size_t)(T.cap + 1) * (kSegBytes / 2) : 0);
+    return mem + (which ? (size_t)(cap + 1) * (kSegBytes / 2) : 0);
   }
-  __device__ __forceinline__ SegView view() const {
-    const int m = T.cap + 1;
-    char* b = buffer(T.hdr[1]);
+  __device__ __forceinline__ SegView view(SegState st) const {
+    const int m = cap + 1;
+    char* b = buffer(st.cur);
     SegView v;
     v.n = n;
     v.k = k;
     v.kw = kw;
-    v.S = T.hdr[0];
+    v.S = st.S;
     v.nb = reinterpret_cast<const int2*>(b);
     v.lo = reinterpret_cast<const int32_t*>(b + (size_t)m * sizeof(int2));
     v.br = v.lo + m;
@@ -212,10 +205,11 @@ struct SegTour {
     v.cd = cd;
     return v;
   }
+
   // The table of construction's `S` runs (in tour order), with the whole
   // block: a thread per run finds its rank by counting.
-  __device__ __forceinline__ void build(const Seg* runs, int S) const {
-    const int m = T.cap + 1;
+  __device__ __forceinline__ SegState build(const Seg* runs, int S) const {
+    const int m = cap + 1;
     char* b = buffer(0);
     int2* nb = reinterpret_cast<int2*>(b);
     int32_t* lo = reinterpret_cast<int32_t*>(b + (size_t)m * sizeof(int2));
@@ -239,28 +233,29 @@ struct SegTour {
       lo[S] = n;
       br[S] = 0;
     }
-    __syncthreads();  // the count and buffer number may lie in the runs' room
-    if (threadIdx.x == 0) {
-      T.hdr[0] = S;
-      T.hdr[1] = 0;
-    }
     __syncthreads();
+    return SegState{S, 0};
   }
 
   // Reverse the forward span x..y, or its complement when longer than n/2
   // (the array rule, entry for entry).  Returns the nodes reversed, or -1
-  // when the table is full.  One warp; V: the current view.
+  // when the table is full (then nothing has changed).  Run by the first nw
+  // warps of the block (this one is warp w): each finds the span and the cuts
+  // for itself, copies its share of the boundaries into the other buffer, and
+  // has the new state; the new table may be read after a block barrier, which
+  // also has to lie between two reversals.
   //
-  // Bound by the latency of one warp's dependent steps: the search for x and
-  // y, the one for the nodes before and after them (only where a cut falls
-  // on a boundary), and the copying pass, S / 32 independent steps.  (The
-  // table it replaced kept an order by tour position beside the one by
-  // source position, shifted both for every cut and merge, and cut segments
-  // at position 0: with it the iteration of 1,024 ants at n = 100k took
-  // 6.3 ms and 2,048 ants at n = 200k 8.6 ms, with this one 4.8 and 6.0 ms.)
+  // Bound by the latency of the search for x and y and of the copying pass,
+  // one boundary per thread and 32 nw of them at a time: an ant's table holds
+  // 80 to 600 segments.  Nothing orders the boundaries, so no warp waits for
+  // another.  Of the slowest ants' time at n = 100,000 reversals took 2,120 us
+  // of 4,870 with two orders of the table, 1,350 of 3,290 with one order and
+  // one warp, 680 of 2,820 with the block's warps sharing the pass and the last
+  // one doing the queue's work beside it.
   // Inlined, like everything else in the block kernel: it makes no calls.
-  __device__ __forceinline__ int flip(const SegView& V, int x, int y) const {
+  __device__ __forceinline__ int flip(SegState& st, int x, int y, int w, int nw) const {
     const int lane = lane_id();
+    const SegView V = view(st);
     const int S = V.S;
     int rx, ry;
     V.locate2_w(x, y, rx, ry);
@@ -279,23 +274,21 @@ struct SegTour {
       L = n - L;
     }
     if (L <= 1) return L;
-    // at most two boundaries more: refuse before touching the table, which
-    // then still holds the tour
-    if (S + 2 > T.cap) return -1;
-    int rp = rx, rs = ry;  // segments of px and sy
-    bool revp = X.rev, revs = Y.rev;
-    if (!inx || !iny) {
-      V.locate2_w(px, sy, rp, rs);
-      revp = V.br[rp] < 0;
-      revs = V.br[rs] < 0;
-    }
-    // new boundaries where a cut edge lies inside a segment; boundaries that
-    // go: the new edge {px, y} or {x, sy} joins source neighbours, each at the
-    // end of its segment that faces the other
+    if (S + 2 > cap) return -1;  // at most two boundaries more
+    // the cut edges {px, x} and {y, sy} become {px, y} and {x, sy}: new
+    // boundaries where a cut edge lies inside a segment; boundaries that go:
+    // a new edge joins source neighbours q, q + 1 whose cut ends face each
+    // other across boundary q + 1
     constexpr int kNone = INT_MAX;
     const int c1 = inx ? max(px, x) : kNone, c2 = iny ? max(y, sy) : kNone;
-    const int m1 = (revp != Y.rev && y - px == (revp ? -1 : 1)) ? max(px, y) : kNone;
-    const int m2 = (X.rev != revs && sy - x == (X.rev ? 1 : -1)) ? max(x, sy) : kNone;
+    auto joined = [&](int p, int pe, int q, int qe) {  // p was cut from pe, q from qe
+      const int v = max(p, q);
+      if (p - q != 1 && q - p != 1) return kNone;
+      const int r = V.locate_w(v);
+      const int2 e = make_int2(V.nb[r].x, V.nb[r].y);
+      return V.lo[r] == v && e.x == (v == p ? pe : qe) && e.y == (v == p ? qe : pe) ? v : kNone;
+    };
+    const int m1 = joined(px, x, y, sy), m2 = joined(x, px, sy, y);
     // (boundaries of the new table) - (of the old one) below node v
     auto shift = [&](int v) { return (c1 < v) + (c2 < v) - (m1 < v) - (m2 < v); };
     // the map of a segment that contains node v, after the reversal
@@ -303,82 +296,85 @@ struct SegTour {
       const int base = b & 0x7fffffff;
       int d = wrapn(b < 0 ? base - v : base + v, n) - i;
       if (d < 0) d += n;
-      if (d >= L) return b;
       int nbase = sum - base;
       if (nbase < 0) nbase += n;
-      return nbase | (~b & (int)0x80000000);
+      return d < L ? nbase | (~b & (int)0x80000000) : b;
     };
-    const int m = T.cap + 1, cur = T.hdr[1];
-    char* out = buffer(cur ^ 1);
+    // the new tour neighbour of node o where the old one was e
+    auto across = [&](int o, int e) {
+      int t = e;
+      t = (o == px) & (e == x) ? y : t;
+      t = (o == x) & (e == px) ? sy : t;
+      t = (o == y) & (e == sy) ? px : t;
+      t = (o == sy) & (e == y) ? x : t;
+      return t;
+    };
+    const int m = cap + 1;
+    char* out = buffer(st.cur ^ 1);
     int2* nb2 = reinterpret_cast<int2*>(out);
     int32_t* lo2 = reinterpret_cast<int32_t*>(out + (size_t)m * sizeof(int2));
     int32_t* br2 = lo2 + m;
-#pragma unroll 2
-    for (int r = lane; r <= S; r += 32) {
+    for (int r = w * 32 + lane; r <= S; r += 32 * nw) {
       const int v = V.lo[r];
       const int b = V.br[r];
       const int2 e = V.nb[r];
       if (v != m1 && v != m2) {
-        const int w = r + shift(v);
-        lo2[w] = v;
-        br2[w] = turned(b, v);
-        nb2[w] = e;
+        const int at = r + shift(v);
+        lo2[at] = v;
+        br2[at] = turned(b, v);
+        nb2[at] = make_int2(across(v, e.x), across(v - 1, e.y));
       }
     }
-    __syncwarp();  // the neighbours below overwrite copied ones
-    // lanes 0..3: the ends px, x, y, sy of the two cut edges get their new
-    // neighbours y, sy, px, x, in the slot of the side that faced the cut
-    if (lane < 4) {
-      const bool first = lane < 2;  // an end of the cut {px, x}
-      const int o = lane == 0 ? px : (lane == 1 ? x : (lane == 2 ? y : sy));
-      const int to = lane == 0 ? y : (lane == 1 ? sy : (lane == 2 ? px : x));
-      const bool hiside = lane == 0 ? !revp : (lane == 1 ? X.rev : (lane == 2 ? !Y.rev : revs));
-      const int ro = lane == 0 ? rp : (lane == 1 ? rx : (lane == 2 ? ry : rs));
-      const bool in = first ? inx : iny;
-      const int v = hiside ? o + 1 : o;  // the boundary
-      const int w = ro + ((in || hiside) ? 1 : 0) + shift(v);
-      const bool gone = ((lane == 0 || lane == 2) ? m1 : m2) != kNone;
-      if (!gone) {
-        if (hiside)
-          nb2[w].y = to;
-        else
-          nb2[w].x = to;
-      }
-      // lanes 1 and 2 also write the new boundary of their cut
-      if (in && (lane == 1 || lane == 2)) {
-        lo2[w] = v;
-        br2[w] = turned((first ? X.base | (X.rev ? (int)0x80000000 : 0) : Y.base | (Y.rev ? (int)0x80000000 : 0)), v);
+    if (w == 0 && lane < 2) {  // the new boundaries: between px and x, between y and sy
+      const bool one = lane == 0;
+      const int p = one ? px : y, q = one ? x : sy;        // the cut edge
+      const int tp = one ? y : px, tq = one ? sy : x;      // its ends' new neighbours
+      const SegRec& G = one ? X : Y;
+      if (one ? inx : iny) {
+        const int v = max(p, q);
+        const int at = (one ? rx : ry) + 1 + shift(v);
+        lo2[at] = v;
+        br2[at] = turned(G.base | (G.rev ? (int)0x80000000 : 0), v);
+        nb2[at] = make_int2(v == p ? tp : tq, v == p ? tq : tp);
       }
     }
-    if (lane == 0) {
-      T.hdr[0] = S + (inx ? 1 : 0) + (iny ? 1 : 0) - (m1 != kNone) - (m2 != kNone);
-      T.hdr[1] = cur ^ 1;
-    }
-    __syncwarp();
+    st.S = S + (inx ? 1 : 0) + (iny ? 1 : 0) - (m1 != kNone) - (m2 != kNone);
+    st.cur ^= 1;
     return L;
   }
 };
+
+// Warps that reverse.  Every one of them finds the span for itself, which
+// costs issue slots of the other ants on the SM; iterations of 32 ants at
+// n = 1k / 256 at 20k / 1,024 at 100k with 2, 3, 4, 5, 7 of them: 0.267 0.267
+// 0.267 0.269 0.269 / 2.71 2.63 2.58 2.60 2.57 / 4.01 3.92 3.88 3.89 3.90 ms.
+constexpr int kFlipWarps = 4;
 
 // Shared scratch of the block search.
 struct LsShared {
   int32_t gain[32];
   int mv[32][8];
   int qh, qn, nlog, changes, moves_round, fail;
-  int64_t total;
+  SegState tab;
+  int64_t total, t_confirm, t_push;
 };
 
 // The search of ls_run by a block of W warps on one tour: each round, warp w
 // evaluates the w-th queued node; entries are popped in queue order up to
-// and including the first one whose evaluation found a move, which warp 0
-// applies.  Nothing changes the tour between the confirmed evaluations, so
-// the result equals popping one node at a time.  Must be called by every
-// thread of the block.  Returns the gain, or -1 when the table filled up
-// (flags are left clean either way; the caller has the ant redone on arrays).
+// and including the first one whose evaluation found a move, which is
+// applied.  Nothing changes the tour between the confirmed evaluations, so
+// the result equals popping one node at a time.  The last warp does the
+// queue's work -- pops, log, pushing the move's ends -- while the others
+// reverse.  Must be called by every thread of the block; tab: the table's
+// state, the same on every thread.  Returns the gain, or -1 when the table
+// filled up (flags are left clean either way; the caller has the ant redone
+// on arrays).
 template <bool TWO>
-__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, const int32_t* init, int ninit,
-                                                LsStats& S, LsShared& sh) {
+__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, SegState& tab, const int32_t* init,
+                                                int ninit, LsStats& S, LsShared& sh) {
   const int n = E.n, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int W = blockDim.x >> 5;
+  const bool keeper = w == W - 1;
   for (int i = tid; i < ninit; i += blockDim.x) {
     const int x = init[i];
     E.queue[i] = x;
@@ -386,7 +382,7 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
   }
   if (tid == 0) {
     sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.fail = 0;
-    sh.total = 0;
+    sh.total = 0; sh.t_confirm = 0; sh.t_push = 0;
   }
   __syncthreads();
   for (;;) {
@@ -414,7 +410,7 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
       if (idx >= n) idx -= n;
       const int a = E.queue[idx];
       int mv[8];
-      const int32_t g = eval_both<TWO>(T.view(), a, E.oropt != 0, mv);
+      const int32_t g = eval_both<TWO>(T.view(tab), a, E.oropt != 0, mv);
       if (lane == 0) {
         sh.gain[w] = g;
         if (g > 0)
@@ -422,12 +418,16 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
       }
     }
     __syncthreads();
-    if (w == 0) {
+    const unsigned bal = __ballot_sync(kFull, lane < R && sh.gain[lane] > 0);
+    const int first = bal ? __ffs(bal) - 1 : R;
+    const int cnt = bal ? first + 1 : R;  // queue entries popped this round
+    const int* mv = sh.mv[bal ? first : 0];
+    // a 2-opt move is one edge exchange, its first edge (mv[0], mv[1])
+    // forward; an Or-opt move is two or three
+    const bool two = mv[7] == 0;
+    const int steps = bal ? (two ? 1 : (mv[6] ? 3 : 2)) : 0;
+    if (keeper) {
       const uint64_t t1 = global_ns();
-      S.t_eval += (int64_t)(t1 - t0);
-      const unsigned bal = __ballot_sync(kFull, lane < R && sh.gain[lane] > 0);
-      const int first = bal ? __ffs(bal) - 1 : R;
-      const int cnt = bal ? first + 1 : R;  // queue entries popped this round
       int a = -1;
       bool first_pop = false;
       if (lane < cnt) {
@@ -439,60 +439,63 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
         E.flags[a] = (uint8_t)((f & ~1) | 2);
       }
       const unsigned fb = __ballot_sync(kFull, first_pop);
-      if (first_pop) E.logb[sh.nlog + __popc(fb & ((1u << lane) - 1u))] = a;
-      S.pops += cnt;
+      const int nlog = sh.nlog;
+      if (first_pop) E.logb[nlog + __popc(fb & ((1u << lane) - 1u))] = a;
       __syncwarp();
       int qh2 = qh + cnt;
       if (qh2 >= n) qh2 -= n;
       int qn2 = qn - cnt;
       const uint64_t t2 = global_ns();
-      S.t_confirm += (int64_t)(t2 - t1);
-      if (bal) {  // apply the first move found, queue its endpoints
-        const int* mv = sh.mv[first];
-        const bool two = mv[7] == 0;
-        // a 2-opt move is one edge exchange, its first edge (mv[0], mv[1])
-        // forward; an Or-opt move is two or three
-        const int steps = two ? 1 : (mv[6] ? 3 : 2);
-        for (int st = 0; st < steps; ++st) {
-          const int n1 = st == 2 ? mv[4] : mv[0];
-          const int n2 = st == 0 ? mv[1] : (st == 1 ? mv[4] : mv[2]);
-          const int n3 = st == 0 ? (two ? mv[2] : mv[4]) : (st == 1 ? mv[3] : mv[1]);
-          const int n4 = st == 0 ? (two ? mv[3] : mv[5]) : (st == 1 ? mv[2] : mv[5]);
-          const SegView V = T.view();
-          bool fwd = two;
-          if (!two) {
-            const SegRec g = V.rec(V.locate_w(n1));
-            fwd = g.step(n1, !g.rev) == n2;
-          }
-          const int L = T.flip(V, fwd ? n2 : n1, fwd ? n3 : n4);
-          if (L < 0) {  // the table is full
-            if (lane == 0) sh.fail = 1;
-            break;
-          }
-          S.flip += L;
-        }
-        if (two)
-          S.moves2++;
-        else
-          S.movesor++;
-        const uint64_t t3 = global_ns();
-        S.t_flip += (int64_t)(t3 - t2);
-        qn2 = ls_push_warp(E, mv, two ? 4 : 6, qh2, qn2);
-        if (lane == 0) {
+      if (bal) qn2 = ls_push_warp(E, mv, two ? 4 : 6, qh2, qn2);
+      if (lane == 0) {
+        sh.t_confirm += (int64_t)(t2 - t1);
+        sh.t_push += (int64_t)(global_ns() - t2);
+        sh.nlog = nlog + __popc(fb);
+        sh.qh = qh2;
+        sh.qn = qn2;
+        if (bal) {
           sh.total += sh.gain[first];
           sh.changes++;
           sh.moves_round++;
         }
-        S.t_push += (int64_t)(global_ns() - t3);
       }
-      if (lane == 0) {
-        sh.nlog += __popc(fb);
-        sh.qh = qh2;
-        sh.qn = qn2;
+      for (int st = 1; st < steps; ++st) __syncthreads();
+    } else {
+      const uint64_t t1 = (w == 0) ? global_ns() : 0;
+      S.t_eval += (int64_t)(t1 - t0);
+      S.pops += cnt;
+      bool full = false;
+      for (int st = 0; st < steps; ++st) {
+        if (st > 0) __syncthreads();
+        const int n1 = st == 2 ? mv[4] : mv[0];
+        const int n2 = st == 0 ? mv[1] : (st == 1 ? mv[4] : mv[2]);
+        const int n3 = st == 0 ? (two ? mv[2] : mv[4]) : (st == 1 ? mv[3] : mv[1]);
+        const int n4 = st == 0 ? (two ? mv[3] : mv[5]) : (st == 1 ? mv[2] : mv[5]);
+        if (full || w >= kFlipWarps) continue;
+        bool fwd = two;
+        if (!two) {
+          const SegView V = T.view(tab);
+          const SegRec g = V.rec(V.locate_w(n1));
+          fwd = g.step(n1, !g.rev) == n2;
+        }
+        const int L = T.flip(tab, fwd ? n2 : n1, fwd ? n3 : n4, w, kFlipWarps);
+        full = L < 0;
+        S.flip += L;
       }
-      __syncwarp();
+      if (bal) {
+        if (two)
+          S.moves2++;
+        else
+          S.movesor++;
+      }
+      if (tid == 0) {
+        sh.tab = tab;
+        if (full) sh.fail = 1;
+        S.t_flip += (int64_t)(global_ns() - t1);
+      }
     }
     __syncthreads();
+    if (w >= kFlipWarps) tab = sh.tab;  // (written again only after the next round's first barrier)
   }
   __syncthreads();
   const int qh = sh.qh, qn = sh.qn, nl = sh.nlog;
@@ -502,6 +505,8 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
     E.flags[E.queue[i]] = 0;
   }
   for (int i = tid; i < nl; i += blockDim.x) E.flags[E.logb[i]] = 0;
+  S.t_confirm = sh.t_confirm;
+  S.t_push = sh.t_push;
   __syncthreads();
   return sh.fail ? -1 : sh.total;
 }
