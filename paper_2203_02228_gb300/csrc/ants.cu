@@ -40,14 +40,39 @@ size_t ants_smem_per_warp(int n, int seg_cap, bool segs) {
   return segs ? vis_bytes + segtab_bytes(seg_cap) : vis_bytes;
 }
 
+namespace {
+
+// Whether a launch of `blocks` ant blocks leaves at most two on an SM (it
+// then runs the kernel compiled for more registers).
+bool few_blocks(int blocks) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return blocks <= 2 * sms;
+}
+
+// The segment-table kernels by roulette width and registers.
+using BlkKernel = void (*)(Colony, Ants);
+using BlkKernelB = void (*)(const Colony*, const Ants*, const int2*, int2*, int32_t*);
+
+BlkKernel blk_kernel(int kw, bool few) {
+  if (kw == 16) return few ? k_ants_blk<16, kAntFewRegs> : k_ants_blk<16, kAntMaxRegs>;
+  return few ? k_ants_blk<32, kAntFewRegs> : k_ants_blk<32, kAntMaxRegs>;
+}
+
+BlkKernelB blk_kernel_b(int kw, bool few) {
+  if (kw == 16) return few ? k_ants_blk_b<16, kAntFewRegs> : k_ants_blk_b<16, kAntMaxRegs>;
+  return few ? k_ants_blk_b<32, kAntFewRegs> : k_ants_blk_b<32, kAntMaxRegs>;
+}
+
+}  // namespace
+
 cudaError_t launch_ants(const Colony& C, const Ants& A, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (A.segs) {  // one block per ant on segment tables, then arrays for the marked ants
     const size_t smem = ants_smem_per_warp(C.n, A.seg_cap, true);
-    if (C.kw == 16)
-      k_ants_blk<16><<<A.m, 32 * kAntWarps, smem, s>>>(C, A);
-    else
-      k_ants_blk<32><<<A.m, 32 * kAntWarps, smem, s>>>(C, A);
+    const BlkKernel k_blk = blk_kernel(C.kw, few_blocks(A.m));
+    k_blk<<<A.m, 32 * kAntWarps, smem, s>>>(C, A);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -64,18 +89,15 @@ cudaError_t launch_ants(const Colony& C, const Ants& A, cudaStream_t s) {
 cudaError_t launch_ants_blk_batch(int kw, const Colony* cols, const Ants* ants, const int2* map, int blocks,
                                   int2* redo_list, int32_t* redo_n, size_t smem, cudaStream_t s) {
   if (blocks <= 0) return cudaSuccess;
-  if (kw == 16)
-    k_ants_blk_b<16><<<blocks, 32 * kAntWarps, smem, s>>>(cols, ants, map, redo_list, redo_n);
-  else
-    k_ants_blk_b<32><<<blocks, 32 * kAntWarps, smem, s>>>(cols, ants, map, redo_list, redo_n);
+  const BlkKernelB k_blk = blk_kernel_b(kw, few_blocks(blocks));
+  k_blk<<<blocks, 32 * kAntWarps, smem, s>>>(cols, ants, map, redo_list, redo_n);
   return cudaGetLastError();
 }
 
 // Dynamic shared memory of the batch segment-table kernel that still lets
 // as many blocks reside per SM as its registers allow.
 size_t ants_blk_batch_smem(int kw) {
-  const void* f = kw == 16 ? reinterpret_cast<const void*>(k_ants_blk_b<16>)
-                           : reinterpret_cast<const void*>(k_ants_blk_b<32>);
+  const void* f = reinterpret_cast<const void*>(blk_kernel_b(kw, false));
   int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -121,8 +143,7 @@ cudaError_t launch_ants_arr_batch(int kw, int minb, const Colony* cols, const An
 
 int ants_batch_resident(int variant, int kw, size_t smem) {
   if (variant == 0) {
-    const void* f = kw == 16 ? reinterpret_cast<const void*>(k_ants_blk_b<16>)
-                             : reinterpret_cast<const void*>(k_ants_blk_b<32>);
+    const void* f = reinterpret_cast<const void*>(blk_kernel_b(kw, false));
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, 32 * kAntWarps, smem) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -140,9 +161,8 @@ int ants_batch_resident(int variant, int kw, size_t smem) {
 }
 
 cudaError_t prepare_ants_batch(int kw, size_t smem_blk, size_t smem_arr) {
-  const void* f = kw == 16 ? reinterpret_cast<const void*>(k_ants_blk_b<16>)
-                           : reinterpret_cast<const void*>(k_ants_blk_b<32>);
-  cudaError_t e = allow_dyn_smem(f, smem_blk);
+  cudaError_t e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel_b(kw, false)), smem_blk);
+  if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel_b(kw, true)), smem_blk);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_2(kw, smem_arr);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_4(kw, smem_arr);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_8(kw, smem_arr);
@@ -150,15 +170,11 @@ cudaError_t prepare_ants_batch(int kw, size_t smem_blk, size_t smem_arr) {
 }
 
 cudaError_t prepare_ants_kernel(int kw, size_t smem_seg, size_t smem_arr) {
-  cudaError_t e;
-  if (kw == 16) {
-    e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants_blk<16>), smem_seg);
-    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<16>), smem_arr);
-  } else {
-    e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants_blk<32>), smem_seg);
-    if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(k_ants<32>), smem_arr);
-  }
-  return e;
+  cudaError_t e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel(kw, false)), smem_seg);
+  if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel(kw, true)), smem_seg);
+  if (e != cudaSuccess) return e;
+  return allow_dyn_smem(kw == 16 ? reinterpret_cast<const void*>(k_ants<16>)
+                                 : reinterpret_cast<const void*>(k_ants<32>), smem_arr);
 }
 
 }  // namespace faco

@@ -671,11 +671,24 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 // speculative in-order pops (ls_run_block).  An ant whose table fills up is
 // marked and redone by the array kernel.  A launch lasts as long as its
 // slowest ant; wider blocks speculate deeper, so the slowest ants finish
-// sooner, while fewer blocks fit an SM (with 64 registers, four blocks of
-// eight warps: 608 of 1,024 ants start at once, the rest as the quick ones
-// finish).  Measured best of 4..12 warps and 40..72 registers.
+// sooner, while fewer blocks fit an SM.  Registers per thread: with
+// kAntMaxRegs three blocks fit an SM and nothing of the evaluation spills;
+// when the launch has no more than two blocks per SM, kAntFewRegs lets them
+// have the rest of the register file.  Measured, ms per iteration (32 ants
+// at n = 1k, 256 at 20k, 256 at 30k with 32-wide lists, 1,024 at 100k, 2,048
+// at 200k):
+//   warps x registers    1k     20k    30k    100k   200k
+//   8 x 64              0.267  2.58   3.42   3.88   5.40
+//   8 x 80              0.232  2.10   2.76   3.43   5.10
+//   8 x 96              0.223  2.01   2.65   3.76   5.90
+//   8 x 128             0.220  1.97   2.63   3.69   5.82
+//   6 x 80              0.247  2.33   3.07   3.48   5.10
+//   6 x 96              0.235  2.20   2.92   3.54   5.27
+//   10 x 80             0.233  2.04   2.72   3.83   6.00
+//   12 x 128            0.219  1.90   2.63   4.88   8.35
 constexpr int kAntWarps = 8;
-constexpr int kAntMaxRegs = 64;
+constexpr int kAntMaxRegs = 80;
+constexpr int kAntFewRegs = 128;
 
 // ---------------------------------------------------------------------
 // Kernels.  One colony: the Colony and Ants descriptors are kernel
@@ -692,8 +705,8 @@ __global__ void __launch_bounds__(128, 1) k_ants(Colony C, Ants A) {
   ants_arr_body<KW>(C, A, ant, smem + (A.smem_vis ? (size_t)wib * vis_bytes : 0));
 }
 
-template <int KW>
-__global__ void __maxnreg__(kAntMaxRegs) k_ants_blk(Colony C, Ants A) {
+template <int KW, int REGS>
+__global__ void __maxnreg__(REGS) k_ants_blk(Colony C, Ants A) {
   const int ant = blockIdx.x;
   if (ant >= A.m) return;
 #define ANTS_BLK_OVERFLOW (void)0
@@ -710,8 +723,8 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, size_t by
 
 // Batch: block b runs ant map[b].y of colony map[b].x; an ant whose table
 // filled up is appended to the redo list.
-template <int KW>
-__global__ void __maxnreg__(kAntMaxRegs)
+template <int KW, int REGS>
+__global__ void __maxnreg__(REGS)
     k_ants_blk_b(const Colony* cols, const Ants* ants, const int2* map, int2* redo_list, int32_t* redo_n) {
   __shared__ Colony sC;
   __shared__ Ants sA;
