@@ -101,78 +101,14 @@ __global__ void __launch_bounds__(32) k_nn_tour_b(const Colony* cols, const Colo
   nn_tour_body(C.xy, C.n, S.cand, C.k, S.backup, C.bl, S.init_route, sv, C.grid, S.cell_start, S.cell_src);
 }
 
-// The initial search's tour with its positions in shared memory (n up to
-// about 106k nodes fits): the low 16 bits of each position in lo[n], bit 16
-// in the bitmap hi.  Otherwise the same lookups as ArrTour.
-struct SmemPosTour {
-  int n, k;
-  int32_t* route;
-  uint16_t* lo;
-  uint32_t* hi;
-  const int2* xy;
-  const int32_t* cn;
-  const int32_t* cd;
-  __device__ __forceinline__ int pos_of(int x) const {
-    return (int)lo[x] | (int)(((hi[x >> 5] >> (x & 31)) & 1u) << 16);
-  }
-  // x moves from position `from` to `to`; each node moves by one thread at a
-  // time, but the 32 nodes of a bitmap word may move together
-  __device__ __forceinline__ void move_pos(int x, int from, int to) {
-    lo[x] = (uint16_t)to;
-    if ((from ^ to) >> 16) atomicXor(&hi[x >> 5], 1u << (x & 31));
-  }
-  __device__ __forceinline__ int at_off(int p, int d) const {
-    p += d;
-    if (p >= n) p -= n;
-    if (p < 0) p += n;
-    return route[p];
-  }
-  __device__ __forceinline__ int succ(int x) const { return at_off(pos_of(x), 1); }
-  __device__ __forceinline__ int adj(int x, bool up) const { return at_off(pos_of(x), up ? 1 : -1); }
-  __device__ __forceinline__ void nbrs(int x, int& p, int& s) const {
-    const int t = pos_of(x);
-    p = at_off(t, -1);
-    s = at_off(t, 1);
-  }
-  __device__ __forceinline__ void walk(int a, int& p, int& s1, int& s2, int& s3) const {
-    route_walk(route, n, pos_of(a), p, s1, s2, s3);
-  }
-  __device__ __forceinline__ int2 coord(int x) const { return xy[x]; }
-  __device__ __forceinline__ int cand(int x, int s) const { return cn[(size_t)x * k + s]; }
-  __device__ __forceinline__ int cdist(int x, int s) const { return cd[(size_t)x * k + s]; }
-};
-
-// Shared-memory bytes of an n-node SmemPosTour.
-__host__ __device__ __forceinline__ size_t smem_pos_bytes(int n) {
-  return (((size_t)n * 2 + 15) & ~(size_t)15) + (size_t)((n + 31) >> 5) * 4;
-}
-
-__device__ __forceinline__ SmemPosTour smem_pos_tour(unsigned char* sm, int n, int k, int32_t* route,
-                                                     const int2* xy, const int32_t* cand, const int32_t* dcand) {
-  SmemPosTour T;
-  T.n = n;
-  T.k = k;
-  T.route = route;
-  T.lo = reinterpret_cast<uint16_t*>(sm);
-  T.hi = reinterpret_cast<uint32_t*>(sm + (((size_t)n * 2 + 15) & ~(size_t)15));
-  T.xy = xy;
-  T.cn = cand;
-  T.cd = dcand;
-  return T;
-}
-
-// Positions of the tour `route` into T (block).
-__device__ __forceinline__ void smem_pos_load(SmemPosTour& T) {
-  const int n = T.n;
-  for (int w = threadIdx.x; w < ((n + 31) >> 5); w += blockDim.x) T.hi[w] = 0;
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int x = T.route[i];
-    T.lo[x] = (uint16_t)i;
-    if (i >> 16) atomicOr(&T.hi[x >> 5], 1u << (x & 31));
-  }
-  __syncthreads();
-}
+// Window and block size (entries + 1 warps), set-up in ms at n = 5k / 20k /
+// 100k / 200k: 11: 9.7 / 38.8 / 242 / 621; 15: 8.8 / 35.2 / 212 / 531; 19: 9.0 /
+// 35.8 / 208 / 505; 23: 9.4 / 37.2 / 211 / 499; 31 (64 registers, spills): 10.3 /
+// 41.2 / 229 / 526.  The tour positions stay in global memory: in shared memory
+// (17 bits a node, up to 106k nodes) they took the L1 cache from everything
+// else, 272 against 229 ms at n = 100k with 31 entries.
+constexpr int kWin = 19;                       // entries, a warp each; the last warp keeps the queue
+constexpr int kInitThreads = 32 * (kWin + 1);
 
 // A reversed span of tour positions: i, i + 1, ..., i + L - 1 (cyclic).
 struct Span {
@@ -192,22 +128,49 @@ __device__ __forceinline__ Span flip_span(int i, int j, int n) {
 // Reverses a span with the whole block.  Every caller reaches it after a
 // block barrier that follows the last write to the tour, and the next reader
 // waits at one.
-template <class TT>
-__device__ __forceinline__ void cta_reverse(TT& T, Span sp) {
+// Most spans are shorter than the block; on the long ones, bound by the
+// latency of their loads, each thread keeps U swaps in flight (set-up at
+// n = 200,000 505 -> 491 ms).
+__device__ __forceinline__ void cta_reverse(ArrTour& T, Span sp) {
+  constexpr int U = 4;
   const int n = T.n;
   int j = sp.i + sp.L - 1;
   if (j >= n) j -= n;
   const int half = sp.L >> 1;
-  for (int t = threadIdx.x; t < half; t += blockDim.x) {
-    int ia = sp.i + t;
-    if (ia >= n) ia -= n;
-    int ib = j - t;
-    if (ib < 0) ib += n;
-    const int va = T.route[ia], vb = T.route[ib];
-    T.route[ia] = vb;
-    T.route[ib] = va;
-    T.move_pos(vb, ib, ia);
-    T.move_pos(va, ia, ib);
+  if (half <= kInitThreads) {
+    const int t = threadIdx.x;
+    if (t < half) {
+      const int ia = wrapn(sp.i + t, n), ib = wrapn(j - t, n);
+      const int va = T.route[ia], vb = T.route[ib];
+      T.route[ia] = vb;
+      T.route[ib] = va;
+      T.pos[vb] = ia;
+      T.pos[va] = ib;
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int t0 = threadIdx.x; t0 < half; t0 += U * kInitThreads) {
+    int va[U], vb[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = t0 + u * kInitThreads;
+      if (t < half) {
+        va[u] = T.route[wrapn(sp.i + t, n)];
+        vb[u] = T.route[wrapn(j - t, n)];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = t0 + u * kInitThreads;
+      if (t < half) {
+        const int ia = wrapn(sp.i + t, n), ib = wrapn(j - t, n);
+        T.route[ia] = vb[u];
+        T.route[ib] = va[u];
+        T.pos[vb[u]] = ia;
+        T.pos[va[u]] = ib;
+      }
+    }
   }
 }
 
@@ -237,11 +200,10 @@ __device__ __forceinline__ void cta_reverse(TT& T, Span sp) {
 // n = 100,000 against the form with six barriers per round and the queue's
 // work between them.  Evaluating only the first 8 / 16 / 24 entries of the
 // window without an evaluation: 408 / 330 / 316 ms against 318 (n = 100,000).
-constexpr int kWin = 31;     // entries, a warp each; the last warp keeps the queue
 constexpr int kAhead = 96;   // queued nodes read ahead (a ring of 128)
 
-template <bool TWO, class TT>
-__device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int init3, int32_t* queue, uint8_t* flags,
+template <bool TWO>
+__device__ __forceinline__ void init_ls_body(ArrTour& T, int oropt, int verify, int init3, int32_t* queue, uint8_t* flags,
                                              int32_t* logb) {
   __shared__ int32_t s_gain[32];
   __shared__ int s_mv[32][8];
@@ -480,52 +442,22 @@ __device__ __forceinline__ void init_ls_body(TT& T, int oropt, int verify, int i
   for (int i = tid; i < nl; i += blockDim.x) flags[logb[i]] = 0;
 }
 
-// SP: the positions live in shared memory during the search (launched with
-// smem_pos_bytes(n) of it) and are written to `pos` at the end; otherwise
-// the search works on `pos` in global memory.
-template <bool SP, bool TWO>
-__device__ __forceinline__ void init_ls_run(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k,
-                                            int oropt, int verify, int init3, int32_t* route, int32_t* pos,
-                                            int32_t* queue, uint8_t* flags, int32_t* logb) {
-  if constexpr (SP) {
-    extern __shared__ __align__(16) unsigned char s_pos[];
-    SmemPosTour T = smem_pos_tour(s_pos, n, k, route, xy, cand, dcand);
-    smem_pos_load(T);
-    init_ls_body<TWO>(T, oropt, verify, init3, queue, flags, logb);
-    __syncthreads();
-    for (int x = threadIdx.x; x < n; x += blockDim.x) pos[x] = T.pos_of(x);
-  } else {
-    ArrTour T{n, k, route, pos, xy, cand, k, dcand};
-    init_ls_body<TWO>(T, oropt, verify, init3, queue, flags, logb);
-  }
-}
-
-template <bool SP, bool TWO>
-__global__ void __launch_bounds__(1024) k_init_ls(const int2* xy, int n, const int32_t* cand,
-                                                  const int32_t* dcand, int k, int oropt, int verify, int init3,
-                                                  int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
-                                                  int32_t* logb) {
-  init_ls_run<SP, TWO>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
+template <bool TWO>
+__global__ void __launch_bounds__(kInitThreads) k_init_ls(const int2* xy, int n, const int32_t* cand,
+                                                          const int32_t* dcand, int k, int oropt, int verify,
+                                                          int init3, int32_t* route, int32_t* pos, int32_t* queue,
+                                                          uint8_t* flags, int32_t* logb) {
+  ArrTour T{n, k, route, pos, xy, cand, k, dcand};
+  init_ls_body<TWO>(T, oropt, verify, init3, queue, flags, logb);
 }
 
 // Batch: one block per colony; positions of the initial tour in src_pos.
-template <bool SP, bool TWO>
-__global__ void __launch_bounds__(1024) k_init_ls_b(const Colony* cols, const ColonySetup* sets) {
+template <bool TWO>
+__global__ void __launch_bounds__(kInitThreads) k_init_ls_b(const Colony* cols, const ColonySetup* sets) {
   const Colony C = cols[blockIdx.x];
   const ColonySetup S = sets[blockIdx.x];
-  init_ls_run<SP, TWO>(C.xy, C.n, S.cand, S.dcand, C.k, C.oropt, C.verify, C.init3, S.init_route, C.src_pos, S.queue, S.flags,
-                  S.logb);
-}
-
-// Shared memory for positions of up to n nodes if kernel f can take it,
-// else 0 (the positions then stay in global memory).
-size_t init_ls_pos_smem(const void* f, int n) {
-  const size_t b = smem_pos_bytes(n);
-  if (allow_dyn_smem(f, b) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
-  return b;
+  ArrTour T{C.n, C.k, S.init_route, C.src_pos, C.xy, S.cand, C.k, S.dcand};
+  init_ls_body<TWO>(T, C.oropt, C.verify, C.init3, S.queue, S.flags, S.logb);
 }
 
 // what = 0: Philox draws   in: uint32 [count][4] = (idx, ant, iter, tag) -> out uint32
@@ -617,37 +549,16 @@ cudaError_t launch_unlabel(const int32_t* route0, const int32_t* route_t, int32_
   return cudaGetLastError();
 }
 
-namespace {
-
-template <bool TWO>
-cudaError_t launch_init_ls_two(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
-                               int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
-                               int32_t* logb, cudaStream_t s) {
-  const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls<true, TWO>), n);
-  if (sm > 0)
-    k_init_ls<true, TWO><<<1, 1024, sm, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
-  else
-    k_init_ls<false, TWO><<<1, 1024, 0, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb);
-  return cudaGetLastError();
-}
-
-template <bool TWO>
-cudaError_t launch_init_ls_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, cudaStream_t s) {
-  const size_t sm = init_ls_pos_smem(reinterpret_cast<const void*>(k_init_ls_b<true, TWO>), max_n);
-  if (sm > 0)
-    k_init_ls_b<true, TWO><<<count, 1024, sm, s>>>(cols, sets);
-  else
-    k_init_ls_b<false, TWO><<<count, 1024, 0, s>>>(cols, sets);
-  return cudaGetLastError();
-}
-
-}  // namespace
-
 cudaError_t launch_init_ls(const int2* xy, int n, const int32_t* cand, const int32_t* dcand, int k, int oropt,
                            int verify, int init3, int32_t* route, int32_t* pos, int32_t* queue, uint8_t* flags,
                            int32_t* logb, cudaStream_t s) {
-  return k > 16 ? launch_init_ls_two<true>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb, s)
-                : launch_init_ls_two<false>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags, logb, s);
+  if (k > 16)
+    k_init_ls<true><<<1, kInitThreads, 0, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags,
+                                               logb);
+  else
+    k_init_ls<false><<<1, kInitThreads, 0, s>>>(xy, n, cand, dcand, k, oropt, verify, init3, route, pos, queue, flags,
+                                                logb);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, int count, int max_n, int kw,
@@ -659,10 +570,12 @@ cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, 
       if (e != cudaSuccess) return e;
     }
     k_nn_tour_b<<<count, 32, smem, s>>>(cols, sets);
-    return cudaGetLastError();
+  } else if (kw == 32) {
+    k_init_ls_b<true><<<count, kInitThreads, 0, s>>>(cols, sets);
+  } else {
+    k_init_ls_b<false><<<count, kInitThreads, 0, s>>>(cols, sets);
   }
-  return kw == 32 ? launch_init_ls_batch<true>(cols, sets, count, max_n, s)
-                  : launch_init_ls_batch<false>(cols, sets, count, max_n, s);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_test_kernels(int what, const void* in, void* out, int count, int width,
