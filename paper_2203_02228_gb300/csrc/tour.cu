@@ -2,7 +2,7 @@
 // tour from node 0 -- first unvisited candidate, else first unvisited backup
 // entry, else the globally nearest unvisited node by (squared distance, id)
 // -- improved by the local search with every node queued in tour order.
-// Both steps are sequential by definition; each runs on one warp.
+// Both steps are sequential by definition; each runs on one block.
 //
 // Also: small device self-test kernels (Philox, EUC_2D, roulette) that the
 // tests call through the library to compare with their own expectations.
@@ -17,9 +17,42 @@ namespace faco {
 
 namespace {
 
+// The walk is one warp's chain of dependent steps: the row of the current
+// node, the visited bits of its candidates, the first free one.  A row costs
+// an L2 round trip unless it is in L1 by then, and a prefetch of the
+// candidates' rows, one step ahead, comes too late for half of them (L1 hit
+// rate 48 %, 837 cycles a step).  So kNnHelpers more warps follow the walk
+// and bring the rows two steps out into L1: they read the current node from
+// shared memory and touch the rows of its candidates' candidates.  They only
+// load: the walk never waits for them.  Set-up in ms at n = 5k / 20k / 100k /
+// 200k with 0, 1, 3, 7 helpers: 9.2 / 36.8 / 208 / 485; 8.5 / 34.2 / 197 / 461; 8.5 /
+// 34.1 / 196 / 460; 8.5 / 34.0 / 195 / 457.
+constexpr int kNnHelpers = 3;
+
+__device__ __forceinline__ void nn_helper(int n, const int32_t* cand, int k, const volatile int* cur) {
+  const int lane = lane_id();
+  const int part = ((threadIdx.x >> 5) - 1) * 2 + (lane >> 4);  // of a row's entries
+  const int limit = n < (1 << 18) ? n * 4096 : 1 << 30;  // never reached: the walk ends first
+  int last = -1;
+  for (int spin = 0; spin < limit; ++spin) {
+    const int u = *cur;
+    if (u < 0) break;  // the walk is done
+    if (u == last) {
+      __nanosleep(40);
+      continue;
+    }
+    last = u;
+    for (int j = lane & 15; j < k; j += 16) {
+      const int c = cand[(size_t)u * k + j];
+      for (int e = part; e < k; e += 2 * kNnHelpers) prefetch_l1(cand + (size_t)cand[(size_t)c * k + e] * k);
+    }
+  }
+}
+
 __device__ __forceinline__ void nn_tour_body(const int2* xy, int n, const int32_t* cand, int k,
                                              const int32_t* backup, int bl, int32_t* route, uint32_t* vis,
-                                             const Grid& g, const int32_t* cstart, const int4* recs) {
+                                             const Grid& g, const int32_t* cstart, const int4* recs,
+                                             volatile int* cur) {
   const int lane = lane_id();
   const int words = (n + 31) >> 5;
   for (int i = lane; i < words; i += 32) vis[i] = 0;
@@ -27,16 +60,14 @@ __device__ __forceinline__ void nn_tour_body(const int2* xy, int n, const int32_
   if (lane == 0) {
     route[0] = 0;
     vis[0] = 1u;
+    *cur = 0;
   }
   __syncwarp();
   int u = 0;
+  int c = lane < k ? cand[lane] : -1;  // the row of u
   for (int i = 1; i < n; ++i) {
     int v = -1;
     {
-      const int c = lane < k ? cand[(size_t)u * k + lane] : -1;
-      // the next node is most often one of these: their own lists start on
-      // their way to L1 now, off the chain of dependent steps
-      if (c >= 0) prefetch_l1(cand + (size_t)c * k);
       const bool ok = c >= 0 && !((vis[c >> 5] >> (c & 31)) & 1u);
       const unsigned bal = __ballot_sync(kFull, ok);
       if (bal) v = __shfl_sync(kFull, c, __ffs(bal) - 1);
@@ -76,29 +107,46 @@ __device__ __forceinline__ void nn_tour_body(const int2* xy, int n, const int32_
       warp_min_key(bk, bi);
       v = (bi >= 0 && bi < n) ? bi : 0;  // bi is valid while a node is unvisited
     }
+    u = v;
+    c = lane < k ? cand[(size_t)u * k + lane] : -1;  // on its way while the step is written down
     if (lane == 0) {
       route[i] = v;
       vis[v >> 5] |= 1u << (v & 31);
+      *cur = v;
     }
     __syncwarp();
-    u = v;
   }
+  if (lane == 0) *cur = -1;
 }
 
-__global__ void __launch_bounds__(32) k_nn_tour(const int2* xy, int n, const int32_t* cand, int k,
-                                                const int32_t* backup, int bl, int32_t* route,
-                                                uint32_t* vis_g, Grid g, const int32_t* cstart,
-                                                const int4* recs) {
+constexpr int kNnThreads = 32 * (1 + kNnHelpers);
+
+__global__ void __launch_bounds__(kNnThreads) k_nn_tour(const int2* xy, int n, const int32_t* cand, int k,
+                                                        const int32_t* backup, int bl, int32_t* route,
+                                                        uint32_t* vis_g, Grid g, const int32_t* cstart,
+                                                        const int4* recs) {
   extern __shared__ uint32_t sv[];
-  nn_tour_body(xy, n, cand, k, backup, bl, route, vis_g ? vis_g : sv, g, cstart, recs);
+  __shared__ int s_cur;
+  if (threadIdx.x == 0) s_cur = 0;
+  __syncthreads();
+  if (threadIdx.x >= 32)
+    nn_helper(n, cand, k, &s_cur);
+  else
+    nn_tour_body(xy, n, cand, k, backup, bl, route, vis_g ? vis_g : sv, g, cstart, recs, &s_cur);
 }
 
-// Batch: one warp per colony, visited bits in shared memory.
-__global__ void __launch_bounds__(32) k_nn_tour_b(const Colony* cols, const ColonySetup* sets) {
+// Batch: one block per colony, visited bits in shared memory.
+__global__ void __launch_bounds__(kNnThreads) k_nn_tour_b(const Colony* cols, const ColonySetup* sets) {
   extern __shared__ uint32_t sv[];
   const Colony C = cols[blockIdx.x];
   const ColonySetup S = sets[blockIdx.x];
-  nn_tour_body(C.xy, C.n, S.cand, C.k, S.backup, C.bl, S.init_route, sv, C.grid, S.cell_start, S.cell_src);
+  __shared__ int s_cur;
+  if (threadIdx.x == 0) s_cur = 0;
+  __syncthreads();
+  if (threadIdx.x >= 32)
+    nn_helper(C.n, S.cand, C.k, &s_cur);
+  else
+    nn_tour_body(C.xy, C.n, S.cand, C.k, S.backup, C.bl, S.init_route, sv, C.grid, S.cell_start, S.cell_src, &s_cur);
 }
 
 // Window and block size (entries + 1 warps), set-up in ms at n = 5k / 20k /
@@ -531,7 +579,7 @@ cudaError_t launch_nn_tour(const int2* xy, int n, const int32_t* cand, int k, co
     cudaError_t e = allow_dyn_smem(reinterpret_cast<const void*>(k_nn_tour), smem);
     if (e != cudaSuccess) return e;
   }
-  k_nn_tour<<<1, 32, smem, s>>>(xy, n, cand, k, backup, bl, route, vis_g, g, cstart, recs);
+  k_nn_tour<<<1, kNnThreads, smem, s>>>(xy, n, cand, k, backup, bl, route, vis_g, g, cstart, recs);
   return cudaGetLastError();
 }
 
@@ -569,7 +617,7 @@ cudaError_t launch_init_tour_batch(const Colony* cols, const ColonySetup* sets, 
       cudaError_t e = allow_dyn_smem(reinterpret_cast<const void*>(k_nn_tour_b), smem);
       if (e != cudaSuccess) return e;
     }
-    k_nn_tour_b<<<count, 32, smem, s>>>(cols, sets);
+    k_nn_tour_b<<<count, kNnThreads, smem, s>>>(cols, sets);
   } else if (kw == 32) {
     k_init_ls_b<true><<<count, kInitThreads, 0, s>>>(cols, sets);
   } else {
