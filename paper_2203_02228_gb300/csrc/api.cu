@@ -33,6 +33,7 @@ struct faco_ctx {
   int2* XYsrc = nullptr;
   int32_t* Dsrc = nullptr;
   int64_t* Psrc = nullptr;
+  int32_t* Dpart = nullptr;
   DevState* st = nullptr;
   int64_t* hist = nullptr;
   int64_t hist_cap = 0;
@@ -108,7 +109,7 @@ Colony colony_view(const faco_ctx* c) {
   C.c_min = c->c_min; C.p_src_gb = c->prm.p_source_gb;
   C.xy = c->xy; C.cand = c->cand; C.backup = c->backup; C.eta = c->eta; C.tau = c->tau;
   C.src_route = c->src_route; C.src_pos = c->src_pos; C.gb_route = c->gb_route; C.gb_pos = c->gb_pos;
-  C.Wsrc = c->Wsrc; C.Csrc = c->Csrc; C.XYsrc = c->XYsrc; C.Dsrc = c->Dsrc; C.Psrc = c->Psrc;
+  C.Wsrc = c->Wsrc; C.Csrc = c->Csrc; C.XYsrc = c->XYsrc; C.Dsrc = c->Dsrc; C.Psrc = c->Psrc; C.Dpart = c->Dpart;
   C.Dcsrc = c->Dcsrc; C.dcand = c->dcand;
   C.st = c->st;
   C.grid = c->grid;
@@ -222,6 +223,7 @@ int create_common(const int32_t* coords, int32_t n, int32_t k, const faco_params
     DA(L, c->XYsrc, n);
     DA(L, c->Dsrc, n);
     DA(L, c->Psrc, (size_t)n + 1);
+    DA(L, c->Dpart, ((size_t)n * c->kw + 255) / 256);
     DA(L, c->st, 1);
     DA(L, c->init_route, n);
     DA(L, c->len_tmp, 1);

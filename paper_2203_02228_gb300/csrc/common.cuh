@@ -87,6 +87,7 @@ struct Colony {
   int2* XYsrc;           // [n] coordinates in source order
   int32_t* Dsrc;         // [n] length of source edge (p, p+1)
   int64_t* Psrc;         // [n+1] exclusive prefix sums of Dsrc
+  int32_t* Dpart;        // sums of Dsrc by block of k_rows (one colony only)
   DevState* st;
   Grid grid;             // point grid of the candidate-list build
   const int32_t* cell_start;  // [cells+1]

@@ -103,3 +103,10 @@ def test_lists_of_uneven_points(kind, k, bl):
     d = np.floor(np.sqrt(near.astype(np.float64)) + 0.5)
     want = np.where(d > 0, np.float32(1) / np.maximum(d, 1).astype(np.float32), np.float32(1)).astype(np.float32)
     np.testing.assert_array_equal(eta, want)
+
+
+@pytest.mark.parametrize("n,k", [(4095, 16), (4096, 16), (4097, 20), (8193, 16)])
+def test_prefix_sums_at_tile_edges(n, k):
+    """Tour lengths come from the prefix sums of the source edges, a block per
+    4,096 of them."""
+    assert_run_equals_oracle(inputs.uniform(n, seed=n), k, 6, 2)
