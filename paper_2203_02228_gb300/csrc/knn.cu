@@ -117,12 +117,13 @@ __global__ void k_cell_fill(const int2* xy, int n, Grid g, int32_t* cursor, int3
 // thirty on uniform points).  The order is found by counting: lane i's key
 // against every key of the buffer, read as a broadcast.
 //
-// Bound by instruction issue (a key comparison is four instructions, about
-// 100 x 4 of them per lane and query).  The form it replaced, a thread per
+// Bound by instruction issue (a key comparison is three instructions while
+// squared distances stay below 2^32, about 100 x 4 of them per lane and query).  The form it replaced, a thread per
 // node with an insertion sort of K entries in local memory, was bound by
-// that local memory.  Lists of 16 + 64 per node: this kernel 8.76 -> 1.05 ms at
-// n = 100,000 (clustered points; 3.58 ms without the thinning), the list call
-// at n = 2,000 0.84 -> 0.07 ms.
+// that local memory.  Lists of 16 + 64 per node, the whole list call: 8.16 ->
+// 0.85 ms at n = 100,003 (clustered points; 3.9 ms without the thinning, 1.15
+// with 96-bit comparisons only), 0.84 -> 0.07 ms at n = 2,000.  Three blocks of
+// 80 registers per SM.
 constexpr int kKnnWarps = 8;     // warps per block, a node each at a time
 constexpr int kKnnBuf = 384;     // candidates a warp holds (> kMaxKnn + 32)
 
@@ -146,13 +147,32 @@ __device__ __forceinline__ int knn_order(KnnBuf& B, int cnt, int K) {
     rank[c] = 0;
   }
   const int per = (cnt + 31) >> 5;
-  for (int j = 0; j < cnt; ++j) {
-    const uint64_t mj = B.m[j];
-    const int32_t ij = B.id[j];
+  unsigned high = 0;
 #pragma unroll
-    for (int c = 0; c < kPer; ++c) {
-      if (c >= per) break;  // (uniform)
-      rank[c] += (mj < m[c] || (mj == m[c] && ij < id[c])) ? 1 : 0;
+  for (int c = 0; c < kPer; ++c) high |= c * 32 + lane < cnt ? (unsigned)(m[c] >> 32) : 0u;
+  if (!__any_sync(kFull, high != 0)) {
+    // squared distances below 2^32 (the usual case): distance and id as one
+    // 64-bit key, half the instructions per comparison
+    uint64_t key[kPer];
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) key[c] = (m[c] << 32) | (unsigned)id[c];
+    for (int j = 0; j < cnt; ++j) {
+      const uint64_t kj = (B.m[j] << 32) | (unsigned)B.id[j];
+#pragma unroll
+      for (int c = 0; c < kPer; ++c) {
+        if (c >= per) break;  // (uniform)
+        rank[c] += kj < key[c] ? 1 : 0;
+      }
+    }
+  } else {
+    for (int j = 0; j < cnt; ++j) {
+      const uint64_t mj = B.m[j];
+      const int32_t ij = B.id[j];
+#pragma unroll
+      for (int c = 0; c < kPer; ++c) {
+        if (c >= per) break;  // (uniform)
+        rank[c] += (mj < m[c] || (mj == m[c] && ij < id[c])) ? 1 : 0;
+      }
     }
   }
   __syncwarp();
@@ -307,7 +327,7 @@ __device__ __forceinline__ void knn_node(const int2* xy, int n, const Grid& g, c
   __syncwarp();  // the next node overwrites the buffer
 }
 
-__global__ void __launch_bounds__(32 * kKnnWarps) k_knn(const int2* xy, int n, Grid g, const int32_t* start,
+__global__ void __launch_bounds__(32 * kKnnWarps, 3) k_knn(const int2* xy, int n, Grid g, const int32_t* start,
                                                         const int32_t* pts, int k, int bl, int32_t* cand,
                                                         int32_t* backup, float* eta, int32_t* dcand) {
   __shared__ KnnBuf s_buf[kKnnWarps];
@@ -383,7 +403,7 @@ __global__ void k_cell_fill_b(const Colony* cols, const ColonySetup* sets, const
 }
 
 // Block e.y of colony e.x: kKnnBatchNodes nodes, in turn over the warps.
-__global__ void __launch_bounds__(32 * kKnnWarps) k_knn_b(const Colony* cols, const ColonySetup* sets,
+__global__ void __launch_bounds__(32 * kKnnWarps, 3) k_knn_b(const Colony* cols, const ColonySetup* sets,
                                                           const int2* map) {
   __shared__ KnnBuf s_buf[kKnnWarps];
   const int2 e = map[blockIdx.x];
