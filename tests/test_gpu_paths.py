@@ -110,3 +110,18 @@ def test_prefix_sums_at_tile_edges(n, k):
     """Tour lengths come from the prefix sums of the source edges, a block per
     4,096 of them."""
     assert_run_equals_oracle(inputs.uniform(n, seed=n), k, 6, 2)
+
+
+@pytest.mark.parametrize("n", [8100, 8192, 8300, 40_000])
+def test_lists_over_several_tiles_of_cells(n):
+    """More than 4,096 grid cells: the cell starts come from several blocks."""
+    xy = inputs.uniform(n, seed=n)
+    g = Colony(xy, 4, bl_size=2)
+    cand, backup, _ = g.lists()
+    x = xy.astype(np.int64)
+    for u in np.random.default_rng(n).integers(0, n, 300):
+        d2 = ((x - x[u]) ** 2).sum(1)
+        d2[u] = np.iinfo(np.int64).max
+        near = np.argpartition(d2, 12)[:12]
+        near = near[np.lexsort((near, d2[near]))][:6]
+        np.testing.assert_array_equal(np.concatenate([cand[u], backup[u]]), near)
