@@ -267,7 +267,8 @@ __device__ __forceinline__ int knn_thin(KnnBuf& B, int cnt, int K, uint64_t& tm,
     const uint64_t m = i < cnt ? B.m[i] : ~0ull;
     const int32_t id = i < cnt ? B.id[i] : 0;
     const bool take = i < cnt && m < hi;
-    const unsigned b = __ballot_sync(kFull, take);  // (also: every lane has read its entry)
+    const unsigned b = __ballot_sync(kFull, take);
+    __syncwarp();  // every lane has read its entry before one is overwritten (a vote orders no memory)
     if (take) {
       const int at = out + __popc(b & ((1u << lane) - 1u));
       B.m[at] = m;
@@ -347,6 +348,7 @@ __device__ __forceinline__ void knn_node(const int2* xy, int n, const Grid& g, c
     }
     if (found >= K || all) break;
     ++r;
+    __syncwarp();  // the buffer is filled again, by other lanes
   }
   __syncwarp();
   if (cnt > K + 32) {

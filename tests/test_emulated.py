@@ -1,0 +1,60 @@
+"""The kernels' own code on the CPU (tests/emu), with the order of a block's
+threads shuffled and shared memory watched: results against plain numpy or the
+oracle, and no access that CUDA would not order."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+EMU = os.path.join(os.path.dirname(os.path.abspath(__file__)), "emu")
+
+
+@pytest.fixture(scope="module")
+def emulated():
+    """Runs Python code against the emulated library in a process of its own."""
+    out = subprocess.run([sys.executable, "-c", "import build; print(build.build())"], cwd=EMU, capture_output=True,
+                         text=True)
+    assert out.returncode == 0, out.stderr
+    lib = out.stdout.strip()
+
+    def run(code, seed=1):
+        r = subprocess.run([sys.executable, os.path.join(EMU, "run.py")], input=code, capture_output=True, text=True,
+                           env=dict(os.environ, FACO_EMU=lib, EMU_SEED=str(seed)), timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+
+    return run
+
+
+LISTS = """
+import ctypes
+import numpy as np
+from paper_2203_02228_gb300 import load
+
+rng = np.random.default_rng(3)
+kind = "{kind}"
+if kind == "heap":       # a cell with more points than a warp's buffer
+    xy = np.concatenate([rng.integers(0, 60, size=(500, 2)), rng.integers(0, 1_000_000, size=(60, 2))])
+elif kind == "same":     # no distance cuts the buffer down
+    xy = np.concatenate([np.full((420, 2), 777), rng.integers(0, 5_000, size=(30, 2))])
+elif kind == "outlier":  # a block of cells with enough points, none of them close enough
+    xy = np.concatenate([rng.integers(0, 2_000, size=(250, 2)), [[(1 << 24) - 1, (1 << 24) - 1]]])
+else:
+    xy = rng.integers(0, 100_000, size=(300, 2))
+xy = np.ascontiguousarray(xy, np.int32)
+n, k, bl = len(xy), 16, 64
+cand, backup = np.zeros((n, k), np.int32), np.zeros((n, bl), np.int32)
+eta = np.zeros((n, k), np.float32)
+p = lambda a: ctypes.c_void_p(a.ctypes.data)
+assert load().faco_lists_noalloc(p(xy), n, k, bl, p(cand), p(backup), p(eta), None) == 0
+x = xy.astype(np.int64)
+d2 = ((x[:, None] - x[None]) ** 2).sum(2)
+d2[np.arange(n), np.arange(n)] = np.iinfo(np.int64).max
+order = np.argsort(d2, axis=1, kind="stable")  # ties by node id
+np.testing.assert_array_equal(np.concatenate([cand, backup], 1), order[:, :k + bl])
+"""
+
+
+@pytest.mark.parametrize("kind", ["heap", "same", "outlier", "even"])
+def test_lists(emulated, kind):
+    emulated(LISTS.format(kind=kind))
