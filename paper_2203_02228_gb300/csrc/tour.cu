@@ -462,7 +462,7 @@ __device__ __forceinline__ void init_ls_body(ArrTour& T, int oropt, int verify, 
     }
     __syncthreads();  // the tour, s_inv and the nodes read ahead are there; s_gain and s_mv were read
     if (bal) {
-      have &= ~__ballot_sync(kFull, s_inv[par][lane] != 0);
+      have &= ~__ballot_sync(kFull, lane < R && s_inv[par][lane] != 0);  // a warp each: entries below R
       par ^= 1;
     }
     have = cnt >= 32 ? 0u : have >> cnt;

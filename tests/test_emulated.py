@@ -58,3 +58,22 @@ np.testing.assert_array_equal(np.concatenate([cand, backup], 1), order[:, :k + b
 @pytest.mark.parametrize("kind", ["heap", "same", "outlier", "even"])
 def test_lists(emulated, kind):
     emulated(LISTS.format(kind=kind))
+
+
+SETUP = """
+import numpy as np
+import oracle
+from paper_2203_02228_gb300 import Colony, inputs
+
+xy = inputs.uniform({n}, seed={n})
+g, o = Colony(xy, {k}, init_3opt={three_opt}), oracle.Colony(xy, {k}, threads=2, init_3opt={three_opt})
+np.testing.assert_array_equal(g.initial()[0], o.initial()[0])
+assert g.initial()[1] == o.initial()[1]
+"""
+
+
+@pytest.mark.parametrize("n,k,three_opt", [(7, 3, 0), (90, 16, 0), (260, 16, 0), (120, 24, 1)])
+def test_initial_search(emulated, n, k, three_opt):
+    """Fewer and more nodes than the window, than the nodes read ahead, and
+    than the ring they are kept in."""
+    emulated(SETUP.format(n=n, k=k, three_opt=three_opt))
