@@ -66,8 +66,8 @@ typedef struct {
   int32_t seg_cap;        /* per-ant tour table in shared memory, in segments:   */
                           /* -1 = sized from shared memory (default), 0 = every  */
                           /* ant on explicit n-entry arrays, 8..4096 = that size */
-                          /* (an ant whose table fills up is redone on arrays;   */
-                          /* results are identical in every case)                */
+                          /* (an ant whose table fills up goes on, or is redone, */
+                          /* on arrays; results are identical in every case)     */
   int32_t local_search;   /* 1: every new tour gets the local search (FACO+LS,   */
                           /* default); 0: base FACO, tours kept as constructed   */
                           /* (the min_new_edges study, Figs. 1 and 3, uses it    */
@@ -100,7 +100,7 @@ typedef struct {
   int64_t flip_elems;      /* elements moved by reversals (sum)            */
   int64_t kernel_launches; /* kernels this context has launched so far     */
   int64_t redone_ants;     /* ants whose segment table filled up and that  */
-                           /* were rebuilt on explicit arrays (sum)        */
+                           /* went on, or were redone, on arrays (sum)     */
   int32_t seg_cap;         /* segments per ant table (0: arrays only)      */
   int32_t pad;
 } faco_stats;

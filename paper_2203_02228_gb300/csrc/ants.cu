@@ -1,6 +1,6 @@
 // ants.cu -- host launchers of the per-ant kernels of ants.cuh: the
 // one-colony kernels (segment-table block per ant, then arrays for the ants
-// whose table filled up) and the batch segment-table kernel.  The batch
+// whose table filled up in construction) and the batch segment-table kernel.  The batch
 // array kernel is instantiated in ants_arr_b.cu.
 #include <mutex>
 #include <set>

@@ -17,8 +17,9 @@
 // The tour is a sequence of runs of the source.  The main kernel keeps it
 // that way -- a segment table in shared memory (seg.cuh) on which the local
 // search runs -- so an ant never writes n-entry arrays.  If an ant's table
-// fills up, the ant is marked and redone by the array kernel, which writes
-// route[]/pos[] explicitly; both give the same tour.
+// fills up in the search, the search goes on over explicit route[]/pos[]
+// (seg.cuh); if it fills up in construction, the ant is marked and redone by
+// the array kernel.  All give the same tour.
 //
 // Readings (shared with the oracle, decided there independently):
 //   start node   floor(x * n / 2^32) of draw 0;
@@ -668,8 +669,8 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 
 // One block of kAntWarps warps per ant, tour as a segment table in shared
 // memory: warp 0 constructs, then all warps run the local search with
-// speculative in-order pops (ls_run_block).  An ant whose table fills up is
-// marked and redone by the array kernel.  A launch lasts as long as its
+// speculative in-order pops (ls_run_block).  An ant whose table fills up in
+// construction is marked and redone by the array kernel.  A launch lasts as long as its
 // slowest ant; wider blocks speculate deeper, so the slowest ants finish
 // sooner, while fewer blocks fit an SM.  Registers per thread: with
 // kAntMaxRegs three blocks fit an SM and nothing of the evaluation spills;
@@ -722,7 +723,7 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, size_t by
 }
 
 // Batch: block b runs ant map[b].y of colony map[b].x; an ant whose table
-// filled up is appended to the redo list.
+// filled up in construction is appended to the redo list.
 template <int KW, int REGS>
 __global__ void __maxnreg__(REGS)
     k_ants_blk_b(const Colony* cols, const Ants* ants, const int2* map, int2* redo_list, int32_t* redo_n) {

@@ -206,8 +206,9 @@ __device__ __forceinline__ void best_tour_body(const Colony& C, const Ants& A, i
   const int a = st->it_best_ant;
   int node, at = t;  // the node at tour position `at`
   const int S = A.nseg ? A.nseg[a] : -1;
-  if (S < 0) {  // arrays, as node ids
+  if (S < 0) {  // arrays, as source positions (-2) or node ids
     node = A.route[(size_t)a * n + t];
+    if (S == -2) node = C.src_route[node];
   } else {  // t is a source position: its segment's map gives its tour position
     const int2* sg = A.segs + (size_t)a * A.seg_cap_ls;
     int lo = 0, hi = S - 1;

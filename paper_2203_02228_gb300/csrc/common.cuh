@@ -135,8 +135,8 @@ struct Ants {
                          // the stride of segs
   int2* segs;            // [m][seg_cap_ls] final tours as segments in source order: first node and
                          // map to tour positions (seg.cuh), or null
-  int32_t* nseg;         // [m] segment count, -1 when the tour is in route/pos
-  int32_t* redo;         // [m] 1: the table overflowed, the array kernel redoes the ant
+  int32_t* nseg;         // [m] segment count; tour in route: -1 as node ids, -2 as source positions
+  int32_t* redo;         // [m] 1: the table overflowed in construction, the array kernel redoes the ant
   int32_t keep_tours;    // 1: also write every tour to route[] (inspection)
   int32_t* pre_route;    // [m][n] optional: tours before local search
   int64_t* pre_len;      // [m]

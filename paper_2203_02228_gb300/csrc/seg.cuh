@@ -21,8 +21,8 @@
 // a split part keeps its map and a merge keeps either part's, one pass that
 // copies the table into its second buffer does all of it: segments may run
 // across tour position 0, so no span is a special case.
-// When the table is full the reversal reports failure and the ant is redone
-// on explicit arrays by the array kernel (same result, more memory traffic).
+// When the table is full the reversal reports failure and the search goes on
+// on explicit arrays (same result, more memory traffic).
 #pragma once
 
 #include "common.cuh"
@@ -354,41 +354,68 @@ constexpr int kFlipWarps = 4;
 struct LsShared {
   int32_t gain[32];
   int mv[32][8];
-  int qh, qn, nlog, changes, moves_round, fail;
+  int qh, qn, nlog, changes, moves_round;
+  int full;  // the table filled up: 1 + exchanges of the move that were done
+  int full_mv;  // the move
   SegState tab;
   int64_t total, t_confirm, t_push;
 };
 
-// The search of ls_run by a block of W warps on one tour: each round, warp w
-// evaluates the w-th queued node; entries are popped in queue order up to
-// and including the first one whose evaluation found a move, which is
-// applied.  Nothing changes the tour between the confirmed evaluations, so
-// the result equals popping one node at a time.  The last warp does the
-// queue's work -- pops, log, pushing the move's ends -- while the others
-// reverse.  Must be called by every thread of the block; tab: the table's
-// state, the same on every thread.  Returns the gain, or -1 when the table
-// filled up (flags are left clean either way; the caller has the ant redone
-// on arrays).
-template <bool TWO>
-__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, SegState& tab, const int32_t* init,
-                                                int ninit, LsStats& S, LsShared& sh) {
+// The block search's tour: a segment table ...
+struct TableRep {
+  static constexpr int kWarps = kFlipWarps;  // that apply a move, from warp 0 on
+  const SegTour& T;
+  SegState tab;  // the same on every thread
+
+  __device__ __forceinline__ SegView view() const { return T.view(tab); }
+  // {n1,n2},{n3,n4} -> {n1,n3},{n2,n4}; fwd: n2 is known to follow n1.  Below 0:
+  // the table is full (nothing has changed)
+  __device__ __forceinline__ int exchange(int n1, int n2, int n3, int n4, bool fwd, int w, LsStats& S) {
+    if (!fwd) {
+      const SegView V = T.view(tab);
+      const SegRec g = V.rec(V.locate_w(n1));
+      fwd = g.step(n1, !g.rev) == n2;
+    }
+    const int L = T.flip(tab, fwd ? n2 : n1, fwd ? n3 : n4, w, kWarps);
+    S.flip += max(L, 0);
+    return L;
+  }
+  __device__ __forceinline__ void post(LsShared& sh) const { sh.tab = tab; }
+  __device__ __forceinline__ void fetch(const LsShared& sh, int w) {
+    if (w >= kWarps) tab = sh.tab;  // (written again only after the next round's first barrier)
+  }
+};
+
+// ... or, once that is full, arrays over source positions.
+struct ArrayRep {
+  static constexpr int kWarps = 1;
+  ArrTour T;
+
+  __device__ __forceinline__ const ArrTour& view() const { return T; }
+  __device__ __forceinline__ int exchange(int n1, int n2, int n3, int n4, bool, int, LsStats& S) {
+    (void)tour_move2(T, n1, n2, n3, n4, S);
+    return 0;
+  }
+  __device__ __forceinline__ void post(LsShared&) const {}
+  __device__ __forceinline__ void fetch(const LsShared&, int) {}
+};
+
+// The rounds of ls_run_block, until the search ends or the table is full
+// (sh.full).  In each, warp w evaluates the w-th queued node; entries are
+// popped in queue order up to and including the first one whose evaluation
+// found a move, which is applied.  Nothing changes the tour between the
+// confirmed evaluations, so the result equals popping one node at a time.  The
+// last warp does the queue's work -- pops, log, pushing the move's ends --
+// while the others reverse.
+template <bool TWO, class Rep>
+__device__ __forceinline__ void ls_rounds(const LsEnv& E, Rep& rep, LsStats& S, LsShared& sh) {
   const int n = E.n, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int W = blockDim.x >> 5;
   const bool keeper = w == W - 1;
-  for (int i = tid; i < ninit; i += blockDim.x) {
-    const int x = init[i];
-    E.queue[i] = x;
-    E.flags[x] = 1;
-  }
-  if (tid == 0) {
-    sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.fail = 0;
-    sh.total = 0; sh.t_confirm = 0; sh.t_push = 0;
-  }
-  __syncthreads();
   for (;;) {
     const int qh = sh.qh, qn = sh.qn;
-    if (qn == 0 || sh.changes >= n || sh.fail) {
-      if (sh.fail || sh.changes >= n || !E.verify || sh.moves_round == 0) break;
+    if (qn == 0 || sh.changes >= n || sh.full) {
+      if (sh.full || sh.changes >= n || !E.verify || sh.moves_round == 0) break;
       const int nl = sh.nlog;  // verify round: queue again the nodes popped
       for (int i = tid; i < nl; i += blockDim.x) {
         const int x = E.logb[i];
@@ -410,7 +437,7 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
       if (idx >= n) idx -= n;
       const int a = E.queue[idx];
       int mv[8];
-      const int32_t g = eval_both<TWO>(T.view(tab), a, E.oropt != 0, mv);
+      const int32_t g = eval_both<TWO>(rep.view(), a, E.oropt != 0, mv);
       if (lane == 0) {
         sh.gain[w] = g;
         if (g > 0)
@@ -464,23 +491,16 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
       const uint64_t t1 = (w == 0) ? global_ns() : 0;
       S.t_eval += (int64_t)(t1 - t0);
       S.pops += cnt;
-      bool full = false;
+      int full = 0;
       for (int st = 0; st < steps; ++st) {
         if (st > 0) __syncthreads();
         const int n1 = st == 2 ? mv[4] : mv[0];
         const int n2 = st == 0 ? mv[1] : (st == 1 ? mv[4] : mv[2]);
         const int n3 = st == 0 ? (two ? mv[2] : mv[4]) : (st == 1 ? mv[3] : mv[1]);
         const int n4 = st == 0 ? (two ? mv[3] : mv[5]) : (st == 1 ? mv[2] : mv[5]);
-        if (full || w >= kFlipWarps) continue;
-        bool fwd = two;
-        if (!two) {
-          const SegView V = T.view(tab);
-          const SegRec g = V.rec(V.locate_w(n1));
-          fwd = g.step(n1, !g.rev) == n2;
-        }
-        const int L = T.flip(tab, fwd ? n2 : n1, fwd ? n3 : n4, w, kFlipWarps);
-        full = L < 0;
-        S.flip += L;
+        if (full || w >= Rep::kWarps) continue;
+        const int L = rep.exchange(n1, n2, n3, n4, two, w, S);
+        if (L < 0) full = 1 + st;
       }
       if (bal) {
         if (two)
@@ -489,15 +509,84 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
           S.movesor++;
       }
       if (tid == 0) {
-        sh.tab = tab;
-        if (full) sh.fail = 1;
+        rep.post(sh);
+        if (full) {
+          sh.full = full;
+          sh.full_mv = first;
+        }
         S.t_flip += (int64_t)(global_ns() - t1);
       }
     }
     __syncthreads();
-    if (w >= kFlipWarps) tab = sh.tab;  // (written again only after the next round's first barrier)
+    rep.fetch(sh, w);
   }
   __syncthreads();
+}
+
+// The search of ls_run by a block on one tour.  A table that fills up (rare:
+// the tables are sized for it not to) is written out to arrays_of(), a tour over
+// source positions, the rest of the move that did not fit is applied there,
+// and the rounds go on with the same queue.  Must be called by every thread of
+// the block; tab: the table's state, the same on every thread.  Returns the
+// gain, and whether the tour is in the arrays.
+//
+// (A launch lasts as long as its slowest ant, and an ant that one warp builds
+// and searches again from the start takes several times as long as it had.
+// Left to the array kernel instead, an iteration of 1,024 ants at n = 100,000
+// took 36.6 ms with min_new_edges = 64 (53 ants' tables fill up) and 197 ms with
+// 256 (963); going on takes 16.4 and 66.5 ms.  256 ants at n = 20,000 with
+// 64-segment tables: 4.0 against 1.16 ms.)
+template <bool TWO, class Arrays>
+__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, SegState& tab, Arrays arrays_of,
+                                                const int32_t* init, int ninit, LsStats& S, LsShared& sh,
+                                                bool& arrays) {
+  const int n = E.n, tid = threadIdx.x;
+  for (int i = tid; i < ninit; i += blockDim.x) {
+    const int x = init[i];
+    E.queue[i] = x;
+    E.flags[x] = 1;
+  }
+  if (tid == 0) {
+    sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.full = 0;
+    sh.total = 0; sh.t_confirm = 0; sh.t_push = 0;
+  }
+  __syncthreads();
+  TableRep rep{T, tab};
+  ls_rounds<TWO>(E, rep, S, sh);
+  tab = rep.tab;
+  const int full = sh.full;
+  arrays = full != 0;
+  if (arrays) {
+    const uint64_t t0 = tid == 0 ? global_ns() : 0;
+    const SegView V = T.view(tab);
+    ArrayRep arr{arrays_of()};
+    for (int r = 0; r < V.S; ++r) {
+      const SegRec g = V.rec(r);
+      for (int q = g.lo + tid; q <= g.hi; q += blockDim.x) {
+        const int t = g.pos(q, n);
+        arr.T.route[t] = q;
+        arr.T.pos[q] = t;
+      }
+    }
+    __syncthreads();
+    if (tid < 32) {
+      // an Or-opt move's exchanges from the one that did not fit on (ls.cuh: apply_or)
+      const int* mv = sh.mv[sh.full_mv];
+      if (mv[7] == 0) {
+        (void)tour_move2(arr.T, mv[0], mv[1], mv[2], mv[3], S);
+      } else {
+        if (full == 1) (void)tour_move2(arr.T, mv[0], mv[1], mv[4], mv[5], S);
+        if (full <= 2) (void)tour_move2(arr.T, mv[0], mv[4], mv[3], mv[2], S);
+        if (mv[6]) (void)tour_move2(arr.T, mv[4], mv[2], mv[1], mv[5], S);
+      }
+    }
+    if (tid == 0) {
+      sh.full = 0;
+      S.t_flip += (int64_t)(global_ns() - t0);
+    }
+    __syncthreads();
+    ls_rounds<TWO>(E, arr, S, sh);
+  }
   const int qh = sh.qh, qn = sh.qn, nl = sh.nlog;
   for (int t = tid; t < qn; t += blockDim.x) {
     int i = qh + t;
@@ -508,7 +597,7 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
   S.t_confirm = sh.t_confirm;
   S.t_push = sh.t_push;
   __syncthreads();
-  return sh.fail ? -1 : sh.total;
+  return sh.total;
 }
 
 }  // namespace faco

@@ -77,3 +77,33 @@ def test_initial_search(emulated, n, k, three_opt):
     """Fewer and more nodes than the window, than the nodes read ahead, and
     than the ring they are kept in."""
     emulated(SETUP.format(n=n, k=k, three_opt=three_opt))
+
+
+FULL_TABLES = """
+import numpy as np
+import oracle
+from paper_2203_02228_gb300 import Colony, inputs
+
+xy = inputs.uniform({n}, seed={n})
+kw = dict({kw})
+kept, plain = Colony(xy, {k}, seg_cap={cap}, keep_ant_tours=1, **kw), Colony(xy, {k}, seg_cap={cap}, **kw)
+o = oracle.Colony(xy, {k}, threads=4, **kw)
+last = np.zeros((6, 24), np.int64)
+for _ in range(3):
+    for c in (kept, plain, o):
+        c.iterate(6, 1)
+    np.testing.assert_array_equal(kept.ant_tours()[0], o.ant_tours()[0])
+    np.testing.assert_array_equal(plain.source()[0], o.source()[0])
+    st = kept.ant_stats()
+    full = st[:, 10] > last[:, 10]
+    assert (st[full, 15] != last[full, 15]).all()  # a block's evaluation time: not left to the one-warp kernel
+    last = st
+assert last[:, 10].any()
+"""
+
+
+@pytest.mark.parametrize("n,k,cap,kw", [(250, 16, 24, ""), (400, 24, 40, "min_new_edges=12"),
+                                        (300, 16, 32, "verify_pass=0")])
+def test_search_goes_on_when_its_table_is_full(emulated, n, k, cap, kw):
+    """Tables that hold every tour as constructed and fill up in the search."""
+    emulated(FULL_TABLES.format(n=n, k=k, cap=cap, kw=kw), seed=n)
