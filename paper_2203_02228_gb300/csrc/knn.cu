@@ -376,6 +376,92 @@ __global__ void __launch_bounds__(32 * kKnnWarps, 3) k_knn(const int2* xy, int n
   if (u < n) knn_node(xy, n, g, start, pts, k, bl, cand, backup, eta, dcand, u, s_buf[w]);
 }
 
+// Short lists (K = k + bl <= M) of many nodes: a thread per node, its K nearest
+// so far in order in registers, over the rings of cells around its own until
+// nothing outside them can be nearer.  They are the last K of M entries; those
+// before them stay below every key.
+//
+// A warp per node (above) is bound by the latency of a query's dependent loads,
+// and a short list leaves it nothing to do meanwhile; with a thread per node 32
+// queries share a warp's loads in flight.  With few nodes the warps of threads
+// are too few to fill the chip, and where points cluster the longest query of a
+// warp holds up the others.  The list call at n = 100,000, uniform / clustered
+// points, warps against threads: K = 2 0.228 / 0.275 -> 0.103 / 0.155 ms, 6 0.275 /
+// 0.302 -> 0.126 / 0.188, 8 0.305 / 0.314 -> 0.160 / 0.260, 12 0.329 / 0.337 -> 0.187 /
+// 0.305.  K = 2 at n = 24,000 0.096 / 0.106 against 0.088 / 0.120, at 32,000 0.110 / 0.123
+// against 0.089 / 0.128; K = 8 at 32,000 0.133 / 0.138 against 0.117 / 0.178, at 48,000
+// 0.173 / 0.176 against 0.119 / 0.185, at 64,000 0.218 / 0.227 against 0.130 / 0.205.
+// With 99 % of 100,000 points in one cell threads are ahead (K = 8: 46.7 -> 34.4 ms);
+// with half of them in a few cells they are behind (2.6 -> 5.6 ms).
+constexpr int kFewKnn = 12, kFewerKnn = 6;
+inline bool knn_by_threads(int n, int K) { return K <= kFewKnn && n >= (K <= kFewerKnn ? 32768 : 49152); }
+
+template <int M>
+__global__ void __launch_bounds__(128) k_knn_few(const int2* xy, int n, Grid g, const int32_t* start,
+                                                 const int32_t* pts, int k, int bl, int32_t* cand, int32_t* backup,
+                                                 float* eta, int32_t* dcand) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= n) return;
+  const int K = k + bl;
+  uint64_t bm[M];  // squared distances
+  int32_t bi[M];
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    bm[i] = i < M - K ? 0 : ~0ull;
+    bi[i] = i < M - K ? -1 : INT_MAX;
+  }
+  const int2 q = xy[u];
+  const int cx = (q.x - g.minx) / g.cs, cy = (q.y - g.miny) / g.cs;
+  auto scan = [&](int j, int j1) {
+    for (; j < j1; ++j) {
+      const int v = pts[j];
+      const uint64_t m = sqdist(q, xy[v]);
+      if (v == u || m > bm[M - 1] || (m == bm[M - 1] && v > bi[M - 1])) continue;
+      bool before[M];  // the new key comes before entry i
+#pragma unroll
+      for (int i = 0; i < M; ++i) before[i] = m < bm[i] || (m == bm[i] && v < bi[i]);
+#pragma unroll
+      for (int i = M - 1; i >= 0; --i) {
+        const bool shift = i > 0 && before[i > 0 ? i - 1 : 0];
+        bm[i] = shift ? bm[i > 0 ? i - 1 : 0] : (before[i] ? m : bm[i]);
+        bi[i] = shift ? bi[i > 0 ? i - 1 : 0] : (before[i] ? v : bi[i]);
+      }
+    }
+  };
+  for (int r = 0;; ++r) {
+    const int x0 = max(cx - r, 0), x1 = min(cx + r, g.gx - 1);
+    for (int y = max(cy - r, 0); y <= min(cy + r, g.gy - 1); ++y) {
+      const int32_t* row = start + y * g.gx;
+      if (y == cy - r || y == cy + r) {
+        scan(row[x0], row[x1 + 1]);
+      } else {
+        if (cx - r >= 0) scan(row[cx - r], row[cx - r + 1]);
+        if (cx + r < g.gx) scan(row[cx + r], row[cx + r + 1]);
+      }
+    }
+    const bool lin = cx - r <= 0, rin = cx + r >= g.gx - 1, din = cy - r <= 0, uin = cy + r >= g.gy - 1;
+    if (lin && rin && din && uin) break;  // every cell scanned
+    int64_t dmin = INT64_MAX;  // everything else is at least this far
+    if (!lin) dmin = min(dmin, (int64_t)q.x - ((int64_t)g.minx + (int64_t)(cx - r) * g.cs) + 1);
+    if (!rin) dmin = min(dmin, ((int64_t)g.minx + (int64_t)(cx + r + 1) * g.cs) - q.x);
+    if (!din) dmin = min(dmin, (int64_t)q.y - ((int64_t)g.miny + (int64_t)(cy - r) * g.cs) + 1);
+    if (!uin) dmin = min(dmin, ((int64_t)g.miny + (int64_t)(cy + r + 1) * g.cs) - q.y);
+    if (bm[M - 1] < (uint64_t)(dmin * dmin)) break;
+  }
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const int at = i - (M - K);
+    if (at >= 0 && at < k) {
+      const int32_t d = euc2d_m(bm[i]);
+      cand[(size_t)u * k + at] = bi[i];
+      eta[(size_t)u * k + at] = d > 0 ? __fdiv_rn(1.0f, (float)d) : 1.0f;
+      if (dcand) dcand[(size_t)u * k + at] = d;
+    } else if (at >= k) {
+      backup[(size_t)u * bl + at - k] = bi[i];
+    }
+  }
+}
+
 // ---------------------------------------------------------------------
 // Batch: the same steps for every colony of a batch; each block reads its
 // colony and its block within the colony from a block map.
@@ -495,7 +581,13 @@ cudaError_t build_lists(const int2* xy, int n, int k, int bl, const Grid& g, int
   e = cudaMemcpyAsync(cell_count, cell_start, sizeof(int32_t) * cells, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return e;
   k_cell_fill<<<(n + 255) / 256, 256, 0, s>>>(xy, n, g, cell_count, cell_pts, cell_src);
-  k_knn<<<(n + kKnnWarps - 1) / kKnnWarps, 32 * kKnnWarps, 0, s>>>(xy, n, g, cell_start, cell_pts, k, bl, cand, backup, eta, dcand);
+  if (!knn_by_threads(n, k + bl))
+    k_knn<<<(n + kKnnWarps - 1) / kKnnWarps, 32 * kKnnWarps, 0, s>>>(xy, n, g, cell_start, cell_pts, k, bl, cand, backup,
+                                                                     eta, dcand);
+  else if (k + bl <= kFewerKnn)
+    k_knn_few<kFewerKnn><<<(n + 127) / 128, 128, 0, s>>>(xy, n, g, cell_start, cell_pts, k, bl, cand, backup, eta, dcand);
+  else
+    k_knn_few<kFewKnn><<<(n + 127) / 128, 128, 0, s>>>(xy, n, g, cell_start, cell_pts, k, bl, cand, backup, eta, dcand);
   return cudaGetLastError();
 }
 

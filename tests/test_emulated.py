@@ -107,3 +107,27 @@ assert last[:, 10].any()
 def test_search_goes_on_when_its_table_is_full(emulated, n, k, cap, kw):
     """Tables that hold every tour as constructed and fill up in the search."""
     emulated(FULL_TABLES.format(n=n, k=k, cap=cap, kw=kw), seed=n)
+
+
+SHORT_LISTS = """
+import numpy as np
+from tests.test_gpu_paths import check_short_lists
+import ctypes
+from paper_2203_02228_gb300 import load
+
+def lists(xy, k, bl):
+    n = len(xy)
+    cand, backup = np.zeros((n, k), np.int32), np.zeros((n, max(bl, 1)), np.int32)
+    eta = np.zeros((n, k), np.float32)
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    assert load().faco_lists_noalloc(p(xy), n, k, bl, p(cand), p(backup), p(eta), None) == 0
+    return cand, backup[:, :bl], eta
+
+check_short_lists(lists, {n}, {k}, {bl}, "{kind}")
+"""
+
+
+@pytest.mark.parametrize("n,k,bl,kind", [(32_768, 2, 0, "uniform"), (32_769, 4, 2, "heap"), (49_152, 5, 7, "uniform"),
+                                         (49_152, 7, 0, "far")])
+def test_short_lists_by_threads(emulated, n, k, bl, kind):
+    emulated(SHORT_LISTS.format(n=n, k=k, bl=bl, kind=kind))

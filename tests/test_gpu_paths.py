@@ -125,3 +125,32 @@ def test_lists_over_several_tiles_of_cells(n):
         near = np.argpartition(d2, 12)[:12]
         near = near[np.lexsort((near, d2[near]))][:6]
         np.testing.assert_array_equal(np.concatenate([cand[u], backup[u]]), near)
+
+
+def check_short_lists(lists, n, k, bl, kind):
+    """lists(xy, k, bl) of n points against full distance rows, for 200 of them."""
+    rng = np.random.default_rng(n + k)
+    xy = rng.integers(0, 1_000_000, size=(n, 2))
+    if kind == "heap":   # many coincide, and a cell holds hundreds
+        xy[: n // 8] = 500_000 + rng.integers(0, 25, size=(n // 8, 2))
+    elif kind == "far":  # a few points with nothing near them
+        xy[:5] = (1 << 24) - 1 - rng.integers(0, 1_000_000, size=(5, 2))
+    xy = np.ascontiguousarray(xy, np.int32)
+    cand, backup, eta = lists(xy, k, bl)
+    x = xy.astype(np.int64)
+    for u in np.concatenate([np.arange(8), rng.integers(0, n, 192)]):
+        d2 = ((x - x[u]) ** 2).sum(1)
+        d2[u] = np.iinfo(np.int64).max
+        near = np.flatnonzero(d2 <= np.partition(d2, k + bl - 1)[k + bl - 1])  # with all ties
+        near = near[np.lexsort((near, d2[near]))][: k + bl]
+        np.testing.assert_array_equal(np.concatenate([cand[u], backup[u]]), near)
+        d = np.floor(np.sqrt(d2[near[:k]].astype(np.float64)) + 0.5)
+        np.testing.assert_array_equal(eta[u], (np.float32(1) / np.maximum(d, 1).astype(np.float32)).astype(np.float32))
+
+
+@pytest.mark.parametrize("kind", ["uniform", "heap", "far"])
+@pytest.mark.parametrize("n,k,bl", [(32_767, 4, 2), (32_768, 4, 2), (49_151, 7, 5), (49_152, 7, 5), (49_152, 2, 0),
+                                    (60_000, 8, 5)])
+def test_short_lists_of_many_nodes(n, k, bl, kind):
+    """Both sides of the rule that takes a thread per node instead of a warp."""
+    check_short_lists(lambda xy, k, bl: Colony(xy, k, bl_size=bl).lists(), n, k, bl, kind)
