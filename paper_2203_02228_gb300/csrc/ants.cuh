@@ -355,8 +355,9 @@ __device__ __noinline__ int warp_nearest(const Colony& C, const uint32_t* vis, i
 }
 
 // Backup list, then the globally nearest unvisited node -- with the whole
-// block when it helps (fb; the other warps wait for this request), else by
-// the warp.  Returns the source position of the chosen node.
+// block when it helps (BLOCK: fb; the other warps wait for this request), else
+// by the warp.  Returns the source position of the chosen node.
+template <bool BLOCK>
 __device__ __forceinline__ int fallback_pick(const Colony& C, const uint32_t* vis, Walk& W, FbBlock* fb) {
   int q = backup_pick(C, vis, W.pc);
   if (q >= 0) {
@@ -364,7 +365,7 @@ __device__ __forceinline__ int fallback_pick(const Colony& C, const uint32_t* vi
     return q;
   }
   const uint64_t t0 = global_ns();
-  if (fb) {
+  if constexpr (BLOCK) {
     if (lane_id() == 0) {
       fb->cmd = 1;
       fb->pc = W.pc;
@@ -481,14 +482,14 @@ __device__ __forceinline__ void block_spec(const Colony& C, const uint32_t* vis,
 }
 
 // Up to `nspec` roulette steps, lane t taking the step at pc + t*dir; with
-// the block (fb) and a known direction, up to 32 steps per warp.
-template <int KW>
+// the block (BLOCK: fb) and a known direction, up to 32 steps per warp.
+template <int KW, bool BLOCK>
 __device__ __forceinline__ void aco_steps(const Colony& C, int32_t* route, int32_t* pos, uint32_t* vis,
                                           int32_t* chk, Walk& W, int nspec, uint32_t ant,
                                           uint32_t iter, FbBlock* fb) {
   const int n = C.n, lane = lane_id();
   int f, anyf, qf;
-  if (fb && W.dir != 0 && nspec == 32) {
+  if (BLOCK && W.dir != 0 && nspec == 32) {
     const int nw = blockDim.x >> 5;
     nspec = 32 * nw;
     if (lane == 0) {
@@ -524,20 +525,22 @@ __device__ __forceinline__ void aco_steps(const Colony& C, int32_t* route, int32
     W.aco += f;
   }
   if (f < nspec && W.kf < n) {
-    if (!anyf) qf = fallback_pick(C, vis, W, fb);
+    if (!anyf) qf = fallback_pick<BLOCK>(C, vis, W, fb);
     W.aco++;
     place_step(C, route, pos, vis, chk, W, qf);
   }
 }
 
 // Focused construction of one ant.  Returns the tour length.
-// fb: the block's shared state when the whole block helps with nearest-
-// unvisited searches and speculative roulette steps (the caller then posts
-// cmd 0 when it is done), or null.
-template <int KW>
+// BLOCK: the whole block helps with nearest-unvisited searches and
+// speculative roulette steps, through its shared state fb (the caller then
+// posts cmd 0 when it is done); else fb is null.  A block's kernel makes no
+// calls: what it runs is inlined, and the warp's search is not compiled into
+// it.
+template <int KW, bool BLOCK>
 __device__ __forceinline__ int64_t construct(const Colony& C, int32_t* route, int32_t* pos, uint32_t* vis,
                                              int32_t* chk, Walk& W, uint32_t ant, uint32_t iter,
-                                             FbBlock* fb = nullptr) {
+                                             FbBlock* fb) {
   const int n = C.n, lane = lane_id();
   const int words = (n + 31) >> 5;
   for (int i = lane; i < words; i += 32) vis[i] = 0;
@@ -579,9 +582,9 @@ __device__ __forceinline__ int64_t construct(const Colony& C, int32_t* route, in
         W.kf += c;
       }
       if (W.kf >= n) break;
-      aco_steps<KW>(C, route, pos, vis, chk, W, 1, ant, iter, fb);
+      aco_steps<KW, BLOCK>(C, route, pos, vis, chk, W, 1, ant, iter, fb);
     } else {
-      aco_steps<KW>(C, route, pos, vis, chk, W, W.dir != 0 ? 32 : 1, ant, iter, fb);
+      aco_steps<KW, BLOCK>(C, route, pos, vis, chk, W, W.dir != 0 ? 32 : 1, ant, iter, fb);
     }
   }
   const int64_t L = W.len + run_sum(C, W.run_first, W.dir, W.run_len) +
@@ -591,7 +594,7 @@ __device__ __forceinline__ int64_t construct(const Colony& C, int32_t* route, in
 }
 
 // Writes a list of runs as node ids (warp).
-__device__ void runs_materialize(const Colony& C, const Seg* runs, int S, int32_t* route) {
+__device__ __forceinline__ void runs_materialize(const Colony& C, const Seg* runs, int S, int32_t* route) {
   for (int r = 0; r < S; ++r) {
     const Seg s = runs[r];
     for (int d = lane_id(); d < s.len; d += 32)
@@ -601,7 +604,7 @@ __device__ void runs_materialize(const Colony& C, const Seg* runs, int S, int32_
 }
 
 // Writes the table's tour as node ids (warp).
-__device__ void seg_materialize(const Colony& C, const SegView& V, int32_t* route) {
+__device__ __forceinline__ void seg_materialize(const Colony& C, const SegView& V, int32_t* route) {
   for (int r = 0; r < V.S; ++r) {
     const SegRec s = V.rec(r);
     for (int q = s.lo + lane_id(); q <= s.hi; q += 32) {
@@ -633,7 +636,7 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
   W.runs = nullptr;
   W.cap = 0;
   W.fall_ns = 0;
-  const int64_t pre_len = construct<KW>(C, route, pos, vis, chk, W, (uint32_t)ant, iter);
+  const int64_t pre_len = construct<KW, false>(C, route, pos, vis, chk, W, (uint32_t)ant, iter, nullptr);
   const uint64_t t_cons = global_ns();
   if (A.pre_route) {
     for (int i = lane; i < n; i += 32) A.pre_route[(size_t)ant * n + i] = route[i];
