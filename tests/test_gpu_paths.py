@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_2203_02228_gb300 import Colony, device_selftest, inputs
+from paper_2203_02228_gb300 import Batch, Colony, device_selftest, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -154,3 +154,34 @@ def check_short_lists(lists, n, k, bl, kind):
 def test_short_lists_of_many_nodes(n, k, bl, kind):
     """Both sides of the rule that takes a thread per node instead of a warp."""
     check_short_lists(lambda xy, k, bl: Colony(xy, k, bl_size=bl).lists(), n, k, bl, kind)
+
+
+def sm_count():
+    import torch
+
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("seg_cap", [-1, 28], ids=["tables", "full_tables"])
+@pytest.mark.parametrize("k", [16, 24])
+@pytest.mark.parametrize("more", [0, 1])
+def test_both_register_variants(k, more, seg_cap):
+    """At most two ant blocks per SM run one variant of the per-ant kernel,
+    more run the other; with small tables some searches go on on arrays."""
+    assert_run_equals_oracle(inputs.uniform(700, seed=k), k, 2 * sm_count() + more, 2, seg_cap=seg_cap)
+
+
+def test_wide_batch_with_many_ants_on_tables():
+    """More than two ant blocks per SM with lists wider than 16, in a batch."""
+    xs = [inputs.uniform(n, seed=n) for n in (700, 260, 90, 410, 33)]
+    ants = 2 * sm_count() // len(xs) + 1
+    b = Batch(xs, 32, seeds=[3, 4, 5, 6, 7], plan=0)
+    b.iterate(ants, 3)
+    assert set(b.plan().tolist()) == {0}
+    tours, lens = b.tours()
+    for i, xy in enumerate(xs):
+        o = oracle.Colony(xy, 32, seed=3 + i, threads=8)
+        o.iterate(ants, 3)
+        assert lens[i] == o.best()[1]
+        np.testing.assert_array_equal(tours[i], o.best()[0])
+        assert np.array_equal(b.tau(i).view(np.uint32), o.tau().view(np.uint32))
