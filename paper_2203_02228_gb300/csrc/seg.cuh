@@ -355,8 +355,7 @@ struct LsShared {
   int32_t gain[32];
   int mv[32][8];
   int qh, qn, nlog, changes, moves_round;
-  int full;  // the table filled up: 1 + exchanges of the move that were done
-  int full_mv;  // the move
+  int full;  // the table filled up: 4 * the move + 1 + exchanges of it that were done
   SegState tab;
   int64_t total, t_confirm, t_push;
 };
@@ -510,10 +509,7 @@ __device__ __forceinline__ void ls_rounds(const LsEnv& E, Rep& rep, LsStats& S, 
       }
       if (tid == 0) {
         rep.post(sh);
-        if (full) {
-          sh.full = full;
-          sh.full_mv = first;
-        }
+        if (full) sh.full = 4 * first + full;
         S.t_flip += (int64_t)(global_ns() - t1);
       }
     }
@@ -571,12 +567,13 @@ __device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T
     __syncthreads();
     if (tid < 32) {
       // an Or-opt move's exchanges from the one that did not fit on (ls.cuh: apply_or)
-      const int* mv = sh.mv[sh.full_mv];
+      const int* mv = sh.mv[full >> 2];
+      const int done = (full & 3) - 1;
       if (mv[7] == 0) {
         (void)tour_move2(arr.T, mv[0], mv[1], mv[2], mv[3], S);
       } else {
-        if (full == 1) (void)tour_move2(arr.T, mv[0], mv[1], mv[4], mv[5], S);
-        if (full <= 2) (void)tour_move2(arr.T, mv[0], mv[4], mv[3], mv[2], S);
+        if (done == 0) (void)tour_move2(arr.T, mv[0], mv[1], mv[4], mv[5], S);
+        if (done <= 1) (void)tour_move2(arr.T, mv[0], mv[4], mv[3], mv[2], S);
         if (mv[6]) (void)tour_move2(arr.T, mv[4], mv[2], mv[1], mv[5], S);
       }
     }
