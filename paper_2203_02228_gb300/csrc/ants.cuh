@@ -673,14 +673,14 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 // One block of kAntWarps warps per ant, tour as a segment table in shared
 // memory: warp 0 constructs, then all warps run the local search with
 // speculative in-order pops (ls_run_block).  An ant whose table fills up in
-// construction is marked and redone by the array kernel.  A launch lasts as long as its
-// slowest ant; wider blocks speculate deeper, so the slowest ants finish
+// construction is marked and redone by the array kernel.  A launch lasts as
+// long as its slowest ant; wider blocks speculate deeper, so the slowest ants finish
 // sooner, while fewer blocks fit an SM.  Registers per thread: with
-// kAntMaxRegs three blocks fit an SM and nothing of the evaluation spills;
-// when the launch has no more than two blocks per SM, kAntFewRegs lets them
-// have the rest of the register file.  Measured, ms per iteration (32 ants
-// at n = 1k, 256 at 20k, 256 at 30k with 32-wide lists, 1,024 at 100k, 2,048
-// at 200k):
+// kAntMaxRegs three blocks fit an SM, at 160 bytes of spill stores (424 with
+// lists wider than 16); when the launch has no more than two blocks per SM,
+// kAntFewRegs lets them have the rest of the register file.  Measured when it
+// was chosen, ms per iteration (32 ants at n = 1k, 256 at 20k, 256 at 30k with
+// 32-wide lists, 1,024 at 100k, 2,048 at 200k):
 //   warps x registers    1k     20k    30k    100k   200k
 //   8 x 64              0.267  2.58   3.42   3.88   5.40
 //   8 x 80              0.232  2.10   2.76   3.43   5.10
@@ -690,6 +690,9 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 //   6 x 96              0.235  2.20   2.92   3.54   5.27
 //   10 x 80             0.233  2.04   2.72   3.83   6.00
 //   12 x 128            0.219  1.90   2.63   4.88   8.35
+// The wide lists where more than two blocks per SM run, at 80 / 96 / 128 (n =
+// 30k, k = 32, 512 and 1,024 ants; n = 5k, k = 24, 2,000 ants): 2.37 2.48 2.47; 3.55
+// 3.65 3.62; 3.62 3.87 3.82: a third block is worth more than the spills cost.
 constexpr int kAntWarps = 8;
 constexpr int kAntMaxRegs = 80;
 constexpr int kAntFewRegs = 128;

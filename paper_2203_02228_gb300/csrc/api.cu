@@ -340,9 +340,16 @@ int create_common(const int32_t* coords, int32_t n, int32_t k, const faco_params
 }
 
 // Segments per ant table (one ant per block): the requested size, or (auto)
-// the largest table, up to 1024 segments, that still lets every ant of an
-// iteration be resident at once; with fewer blocks per SM when the visited
-// bits alone are too large for that.  0 (arrays only) when not even 64 fit.
+// up to 1024 segments out of an SM's shared memory divided by the ants per SM
+// (by fewer, until 256 segments fit beside the visited bits).  0 (arrays
+// only) when not even 64 fit.
+// Registers let three blocks reside on an SM, so with many ants this leaves
+// shared memory unused, which then is L1 cache: larger tables are not faster,
+// since a search whose table fills up goes on on arrays.  Iterations in ms, at
+// 256 / 352 / 416 / 640 / 1,024 segments: n = 180,000, 1,536 ants 2.30 2.27 2.34 2.32 2.40
+// (with min_new_edges = 64 13.5 13.5 13.6 13.7 14.2); n = 200,000, 2,048 ants, at 352 /
+// 640 / 1,024: 2.59 2.59 2.69 (18.4 18.5 19.1); n = 100,000, 1,024 ants, at 256 / 544 /
+// 1,024: 1.40 1.40 1.41 (9.7 9.3 9.4).
 int seg_capacity(int n, int m, int requested) {
   if (requested >= 0) return requested;
   int dev = 0, sms = 148;

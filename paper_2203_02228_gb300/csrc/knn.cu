@@ -159,7 +159,7 @@ __global__ void k_cell_fill(const int2* xy, int n, Grid g, int32_t* cursor, int3
 // squared distances stay below 2^32, about 100 x 4 of them per lane and query).  The form it replaced, a thread per
 // node with an insertion sort of K entries in local memory, was bound by
 // that local memory.  Lists of 16 + 64 per node, the whole list call: 8.16 ->
-// 0.85 ms at n = 100,003 (clustered points; 3.9 ms without the thinning, 1.15
+// 0.81 ms at n = 100,003 (clustered points; 3.9 ms without the thinning, 1.15
 // with 96-bit comparisons only), 0.84 -> 0.07 ms at n = 2,000.  Three blocks of
 // 80 registers per SM.
 constexpr int kKnnWarps = 8;     // warps per block, a node each at a time

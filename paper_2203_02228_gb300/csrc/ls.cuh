@@ -444,18 +444,6 @@ __device__ __forceinline__ int ls_push_warp(const LsEnv& E, const int* x, int np
   return qn + __popc(bal);
 }
 
-// FIFO push by lane 0 (the caller broadcasts qn afterwards).
-__device__ __forceinline__ void ls_push0(const LsEnv& E, int x, int qh, int& qn) {
-  const uint8_t f = E.flags[x];
-  if (!(f & 1)) {
-    E.flags[x] = f | 1;
-    int t = qh + qn;
-    if (t >= E.n) t -= E.n;
-    E.queue[t] = x;
-    ++qn;
-  }
-}
-
 // Runs the search from the checklist init[0..ninit) (distinct nodes).
 // Returns the total gain (old length - new length), or -1 if the tour
 // representation ran out of capacity (flags are left clean either way).

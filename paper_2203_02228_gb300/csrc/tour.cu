@@ -223,7 +223,7 @@ __device__ __forceinline__ void cta_reverse(ArrTour& T, Span sp) {
 }
 
 // The local search with every node queued (the initial tour), run by one
-// block of 32 warps over a window of the next kWin queued nodes.  Each
+// block of kWin + 1 warps over a window of the next kWin queued nodes.  Each
 // window entry keeps its evaluation -- the best move from its node on the
 // tour as it was -- together with the tour positions that evaluation read
 // (the node's, the next three and the previous one; each candidate's and its
