@@ -527,7 +527,10 @@ int tuner_run(const std::vector<RunEntry>& entries, size_t smem, cudaStream_t s,
         rc = r.build(v, smem, s);
         float tmin = 1e30f;
         for (int rep = 0; rep < 2 && rc == FACO_OK; ++rep) {
-          if (cudaEventRecord(ev[0], s) != cudaSuccess) rc = FACO_E_CUDA;
+          // the redo list holds the ants of one pass: an iteration's colony
+          // update empties it, and this pass is without one
+          if (cudaMemsetAsync(r.redo_n, 0, sizeof(int32_t), s) != cudaSuccess) rc = FACO_E_CUDA;
+          if (rc == FACO_OK && cudaEventRecord(ev[0], s) != cudaSuccess) rc = FACO_E_CUDA;
           if (rc == FACO_OK) rc = r.enqueue(s, 1);
           if (rc == FACO_OK && cudaEventRecord(ev[1], s) != cudaSuccess) rc = FACO_E_CUDA;
           if (rc == FACO_OK && cudaEventSynchronize(ev[1]) != cudaSuccess) rc = FACO_E_CUDA;

@@ -48,6 +48,7 @@ def _host_source(s):
     for name in WATCHED_STRUCTS:
         s = re.sub(r"struct %s \{.*?\n\};" % name,
                    lambda m: re.sub(r"^  \w+ [^;/]*;", _watch, m.group(0), flags=re.M), s, flags=re.S)
+    s = s.replace("redo_list[atomicAdd(redo_n, 1)] = e", "emu::append_once(redo_list, redo_n, e)")
     s = re.sub(r'asm volatile\("mov.u64 %0, %%globaltimer;"[^;]*;', "static uint64_t ns; t = ++ns;", s)
     s = re.sub(r'asm\("sqrt[^"]*"[^;]*;', "r = sqrtf(x);", s)
     s = re.sub(r'asm volatile\("prefetch[^"]*"[^;]*;', ";", s)

@@ -201,6 +201,15 @@ template <class T, class U>
 inline T atomicMax(T* p, U v) { const T o = *p; *p = max(o, (T)v); return o; }
 template <class T, class U>
 inline T atomicOr(T* p, U v) { const T o = *p; *p = o | (T)v; return o; }
+namespace emu {
+// An entry for a list whose entries are worked on side by side.
+template <class T>
+inline void append_once(T* list, int* count, T e) {
+  for (int i = 0; i < *count; ++i)
+    if (!memcmp(&list[i], &e, sizeof(T))) return report("second entry for the same work in a list");
+  list[(*count)++] = e;
+}
+}  // namespace emu
 inline void __nanosleep(unsigned) { emu::nap(); }
 
 // ---- run time -------------------------------------------------------------------
@@ -225,9 +234,10 @@ inline cudaError_t cudaGetDevice(int* d) { *d = 0; return 0; }
 inline cudaError_t cudaSetDevice(int) { return 0; }
 inline cudaError_t cudaGetDeviceCount(int* d) { *d = 1; return 0; }
 inline cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+  const char* sm_shared = getenv("EMU_SM_SHARED");  // a device with less of it: smaller tables in a batch
   *v = a == cudaDevAttrMaxSharedMemoryPerBlockOptin       ? 232448
        : a == cudaDevAttrMultiProcessorCount              ? 152
-       : a == cudaDevAttrMaxSharedMemoryPerMultiprocessor ? 233472
+       : a == cudaDevAttrMaxSharedMemoryPerMultiprocessor ? (sm_shared ? atoi(sm_shared) : 233472)
        : a == cudaDevAttrReservedSharedMemoryPerBlock     ? 1024
                                                           : 65536;
   return 0;

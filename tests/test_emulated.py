@@ -131,3 +131,18 @@ check_short_lists(lists, {n}, {k}, {bl}, "{kind}")
                                          (49_152, 7, 0, "far")])
 def test_short_lists_by_threads(emulated, n, k, bl, kind):
     emulated(SHORT_LISTS.format(n=n, k=k, bl=bl, kind=kind))
+
+
+def test_tuner_lists_an_ant_once(emulated, monkeypatch):
+    """A batch that times its per-ant kernels first: every table fills up in
+    construction, in each of the timed passes."""
+    monkeypatch.setenv("EMU_SM_SHARED", "17664")  # tables of 64 segments
+    emulated("""
+from paper_2203_02228_gb300 import Batch, inputs
+b = Batch([inputs.uniform(160, seed=7), inputs.uniform(150, seed=8)], 8, seeds=[3, 4], min_new_edges=160)
+b.iterate(3, 1)
+b.sync()
+b.set_plan(0)
+b.iterate(3, 2)
+assert b.stats(0).seg_cap == 64 and b.stats(0).redone_ants > 0
+""")
