@@ -94,6 +94,15 @@ cudaError_t launch_ants_blk_batch(int kw, const Colony* cols, const Ants* ants, 
   return cudaGetLastError();
 }
 
+cudaError_t launch_ants_rest_batch(int kw, const Colony* cols, const Ants* ants, int blocks, const int2* redo_list,
+                                   const int32_t* redo_n, size_t vis_bytes, cudaStream_t s) {
+  if (kw == 16)
+    k_ants_rest_b<16><<<blocks, 32 * kAntWarps, vis_bytes, s>>>(cols, ants, redo_list, redo_n);
+  else
+    k_ants_rest_b<32><<<blocks, 32 * kAntWarps, vis_bytes, s>>>(cols, ants, redo_list, redo_n);
+  return cudaGetLastError();
+}
+
 // Dynamic shared memory of the batch segment-table kernel that still lets
 // as many blocks reside per SM as its registers allow.
 size_t ants_blk_batch_smem(int kw) {
@@ -131,12 +140,11 @@ size_t ants_blk_batch_smem(int kw) {
 }
 
 cudaError_t launch_ants_arr_batch(int kw, int minb, const Colony* cols, const Ants* ants, const int2* map, int nmap,
-                                  int redo_blocks, const int2* redo_list, const int32_t* redo_n,
                                   size_t per_warp, cudaStream_t s) {
   switch (minb) {
-    case 2: return launch_ants_arr_batch_2(kw, cols, ants, map, nmap, redo_blocks, redo_list, redo_n, per_warp, s);
-    case 4: return launch_ants_arr_batch_4(kw, cols, ants, map, nmap, redo_blocks, redo_list, redo_n, per_warp, s);
-    case 8: return launch_ants_arr_batch_8(kw, cols, ants, map, nmap, redo_blocks, redo_list, redo_n, per_warp, s);
+    case 2: return launch_ants_arr_batch_2(kw, cols, ants, map, nmap, per_warp, s);
+    case 4: return launch_ants_arr_batch_4(kw, cols, ants, map, nmap, per_warp, s);
+    case 8: return launch_ants_arr_batch_8(kw, cols, ants, map, nmap, per_warp, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -163,6 +171,9 @@ int ants_batch_resident(int variant, int kw, size_t smem) {
 cudaError_t prepare_ants_batch(int kw, size_t smem_blk, size_t smem_arr) {
   cudaError_t e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel_b(kw, false)), smem_blk);
   if (e == cudaSuccess) e = allow_dyn_smem(reinterpret_cast<const void*>(blk_kernel_b(kw, true)), smem_blk);
+  if (e == cudaSuccess)
+    e = allow_dyn_smem(kw == 16 ? reinterpret_cast<const void*>(k_ants_rest_b<16>)
+                                : reinterpret_cast<const void*>(k_ants_rest_b<32>), smem_arr / 4);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_2(kw, smem_arr);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_4(kw, smem_arr);
   if (e == cudaSuccess) e = prepare_ants_arr_batch_8(kw, smem_arr);

@@ -697,6 +697,11 @@ constexpr int kAntWarps = 8;
 constexpr int kAntMaxRegs = 80;
 constexpr int kAntFewRegs = 128;
 
+// An ant's arrays as a tour over source positions.
+__device__ __forceinline__ ArrTour source_arrays(const Colony& C, const Ants& A, int ant) {
+  return ArrTour{C.n, C.k, A.route + (size_t)ant * C.n, A.pos + (size_t)ant * C.n, C.XYsrc, C.Csrc, C.kw, C.Dcsrc};
+}
+
 // ---------------------------------------------------------------------
 // Kernels.  One colony: the Colony and Ants descriptors are kernel
 // parameters.  A batch of colonies: every block reads its (colony, ant)
@@ -717,7 +722,16 @@ __global__ void __maxnreg__(REGS) k_ants_blk(Colony C, Ants A) {
   const int ant = blockIdx.x;
   if (ant >= A.m) return;
 #define ANTS_BLK_OVERFLOW (void)0
+#define ANTS_BLK_FULL                                    \
+  if (full) {                                            \
+    ArrayRep arr{source_arrays(C, A, ant)};              \
+    ls_to_arrays(tour.view(tab), arr.T, full, S, sh);    \
+    ls_rounds<KW == 32>(E, arr, S, sh);                  \
+  }
+#define ANTS_BLK_LEAVE (void)0
 #include "ants_blk_body.inc"
+#undef ANTS_BLK_LEAVE
+#undef ANTS_BLK_FULL
 #undef ANTS_BLK_OVERFLOW
 }
 
@@ -729,7 +743,10 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, size_t by
 }
 
 // Batch: block b runs ant map[b].y of colony map[b].x; an ant whose table
-// filled up in construction is appended to the redo list.
+// filled up, in construction or in the search, is appended to the redo list,
+// for k_ants_rest_b.  (Going on on arrays in this kernel, as in the one-colony
+// kernel, costs the searches on tables 2 to 6 %, in every form tried: 64
+// instances of 200 to 20,000 nodes, 64 ants, 2.48 -> 2.58 ms an iteration.)
 template <int KW, int REGS>
 __global__ void __maxnreg__(REGS)
     k_ants_blk_b(const Colony* cols, const Ants* ants, const int2* map, int2* redo_list, int32_t* redo_n) {
@@ -745,39 +762,114 @@ __global__ void __maxnreg__(REGS)
   if (ant >= A.m) return;
 #define ANTS_BLK_OVERFLOW \
   if (tid == 0) redo_list[atomicAdd(redo_n, 1)] = e
+#define ANTS_BLK_FULL (void)0
+#define ANTS_BLK_LEAVE             \
+  if (full) {                      \
+    if (tid == 0) A.redo[ant] = 1; \
+    ANTS_BLK_OVERFLOW;             \
+    return;                        \
+  }
 #include "ants_blk_body.inc"
+#undef ANTS_BLK_LEAVE
+#undef ANTS_BLK_FULL
 #undef ANTS_BLK_OVERFLOW
 }
 
-// Batch, arrays: blocks below nmap run the four ants map[b].y + warp of
-// colony map[b].x; the remaining blocks run the redo list, one entry per
-// warp in turn.  per_warp is the shared-memory stride of a warp.
+// The ants on the redo list, built and searched on arrays, a block each in
+// turn (a warp each took 159 ms an iteration, a block 68: 16 instances of
+// 10,000 to 20,000 nodes, 64 ants, min_new_edges = 500, 47 tables of a colony's
+// 64 full).  Visited bits in dynamic shared memory.
+template <int KW>
+__global__ void __maxnreg__(kAntFewRegs)
+    k_ants_rest_b(const Colony* cols, const Ants* ants, const int2* redo_list, const int32_t* redo_n) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ Colony sC;
+  __shared__ Ants sA;
+  __shared__ LsShared sh;
+  __shared__ FbBlock s_fb;
+  __shared__ int s_nchk;
+  __shared__ int64_t s_len;
+  const int tid = threadIdx.x;
+  const int todo = *redo_n;
+  for (int r = blockIdx.x; r < todo; r += gridDim.x) {
+    const int2 e = redo_list[r];
+    __syncthreads();  // the entry before is done with the descriptors
+    copy_words(&sC, cols + e.x, sizeof(Colony), 0, blockDim.x);
+    copy_words(&sA, ants + e.x, sizeof(Ants), 0, blockDim.x);
+    __syncthreads();
+    const Colony& C = sC;
+    const Ants& A = sA;
+    const int ant = e.y, n = C.n;
+    uint32_t* vis = reinterpret_cast<uint32_t*>(smem);
+    int32_t* chk = A.chk + (size_t)ant * n;
+    const uint64_t t_start = global_ns();
+    uint64_t t_cons = t_start;
+    Walk W;
+    W.segs = false;
+    W.runs = nullptr;
+    W.cap = 0;
+    W.fall_ns = 0;
+    W.aco = W.backup = W.global = 0;
+    W.new_edges = W.nchk = 0;
+    LsEnv E{n, C.oropt, C.verify, A.queue + (size_t)ant * n, A.flags + (size_t)ant * n, A.logb + (size_t)ant * n};
+    LsStats S{0, 0, 0, 0, 0};
+    ArrayRep rep{ArrTour{n, C.k, A.route + (size_t)ant * n, A.pos + (size_t)ant * n, C.xy, C.cand, C.k, C.dcand}};
+    const uint32_t iter = (uint32_t)(C.st->iter + 1);
+    if (tid < 32) {
+      const int64_t len =
+          construct<KW, true>(C, rep.T.route, rep.T.pos, vis, chk, W, (uint32_t)ant, iter, &s_fb);
+      if (tid == 0) {
+        s_fb.cmd = 0;
+        s_len = len;
+        s_nchk = C.ls ? W.nchk : 0;
+      }
+      __syncwarp();
+      __syncthreads();  // releases the helpers
+    } else {
+      for (;;) {
+        __syncthreads();  // a request from warp 0, or its end of construction
+        if (s_fb.cmd == 0) break;
+        if (s_fb.cmd == 1)
+          block_nearest(n, C.XYsrc, C.src_route, C.src_pos, C.st, vis, s_fb);
+        else
+          block_spec<KW>(C, vis, s_fb, (uint32_t)ant, iter);
+      }
+    }
+    t_cons = global_ns();
+    ls_begin(E, chk, s_nchk, sh);
+    ls_rounds<KW == 32>(E, rep, S, sh);
+    const int64_t gain = ls_end(E, S, sh);
+    if (tid == 0) {
+      A.nseg[ant] = -1;  // tour in route, as node ids
+      A.len[ant] = s_len - gain;
+      A.redo[ant] = 0;
+      int64_t* st = A.stats + (size_t)ant * kNStats;
+      st[kStAco] += W.aco; st[kStNew] += W.new_edges; st[kStBackup] += W.backup;
+      st[kStGlobal] += W.global; st[kStCheck] += W.nchk; st[kStPops] += S.pops;
+      st[kStMoves2] += S.moves2; st[kStMovesOr] += S.movesor; st[kStFlip] += S.flip;
+      st[kStVerify] += S.verify; st[kStRedo] += 1;
+      st[kStStartNs] = (int64_t)t_start;
+      st[kStDurNs] = (int64_t)(global_ns() - t_start);
+      st[kStConsNs] = (int64_t)(t_cons - t_start);
+      st[kStFallNs] = W.fall_ns;
+    }
+  }
+}
+
+// Batch, arrays: a block runs the four ants map[b].y + warp of colony
+// map[b].x.  per_warp is the shared-memory stride of a warp.
 template <int KW, int MB>
 __global__ void __launch_bounds__(128, MB)
-    k_ants_b(const Colony* cols, const Ants* ants, const int2* map, int nmap, const int2* redo_list,
-             const int32_t* redo_n, size_t per_warp) {
+    k_ants_b(const Colony* cols, const Ants* ants, const int2* map, size_t per_warp) {
   extern __shared__ __align__(16) char smem[];
-  __shared__ Colony sC[4];
-  __shared__ Ants sA[4];
+  __shared__ Colony sC;
+  __shared__ Ants sA;
   const int wib = threadIdx.x >> 5;
-  const bool mapped = (int)blockIdx.x < nmap;
-  const int stride = mapped ? 0 : ((int)gridDim.x - nmap) * 4;
-  for (int r = mapped ? 0 : ((int)blockIdx.x - nmap) * 4 + wib;; r += stride) {
-    int2 e;
-    if (mapped) {
-      e = map[blockIdx.x];
-      e.y += wib;
-    } else {
-      if (r >= *redo_n) break;
-      e = redo_list[r];
-    }
-    copy_words(&sC[wib], cols + e.x, sizeof(Colony), wib * 32, 32);
-    copy_words(&sA[wib], ants + e.x, sizeof(Ants), wib * 32, 32);
-    __syncwarp();
-    ants_arr_body<KW>(sC[wib], sA[wib], e.y, smem + (size_t)wib * per_warp);
-    __syncwarp();
-    if (mapped) break;
-  }
+  const int2 e = map[blockIdx.x];
+  copy_words(&sC, cols + e.x, sizeof(Colony), 0, blockDim.x);
+  copy_words(&sA, ants + e.x, sizeof(Ants), 0, blockDim.x);
+  __syncthreads();
+  ants_arr_body<KW>(sC, sA, e.y + wib, smem + (size_t)wib * per_warp);
 }
 
 }  // namespace

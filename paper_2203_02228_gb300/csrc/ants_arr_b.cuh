@@ -12,15 +12,13 @@ namespace {
 
 template <int MB>
 cudaError_t launch_arr_b_mb(int kw, const Colony* cols, const Ants* ants, const int2* map, int nmap,
-                            int redo_blocks, const int2* redo_list, const int32_t* redo_n, size_t per_warp,
-                            cudaStream_t s) {
-  const int blocks = nmap + redo_blocks;
-  if (blocks <= 0) return cudaSuccess;
+                            size_t per_warp, cudaStream_t s) {
+  if (nmap <= 0) return cudaSuccess;
   const size_t smem = 4 * per_warp;
   if (kw == 16)
-    k_ants_b<16, MB><<<blocks, 128, smem, s>>>(cols, ants, map, nmap, redo_list, redo_n, per_warp);
+    k_ants_b<16, MB><<<nmap, 128, smem, s>>>(cols, ants, map, per_warp);
   else
-    k_ants_b<32, MB><<<blocks, 128, smem, s>>>(cols, ants, map, nmap, redo_list, redo_n, per_warp);
+    k_ants_b<32, MB><<<nmap, 128, smem, s>>>(cols, ants, map, per_warp);
   return cudaGetLastError();
 }
 

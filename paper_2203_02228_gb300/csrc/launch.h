@@ -22,15 +22,17 @@ size_t ants_smem_per_warp(int n, int seg_cap, bool segs);
 int ants_seg_cap_ls(int n, int seg_cap);
 cudaError_t launch_ants_blk_batch(int kw, const Colony* cols, const Ants* ants, const int2* map, int blocks,
                                   int2* redo_list, int32_t* redo_n, size_t smem, cudaStream_t s);
+// The ants that launch left on the redo list (vis_bytes: the most any colony's
+// visited bits take).
+cudaError_t launch_ants_rest_batch(int kw, const Colony* cols, const Ants* ants, int blocks, const int2* redo_list,
+                                   const int32_t* redo_n, size_t vis_bytes, cudaStream_t s);
 // batch array kernel: minb = 2, 4 or 8 blocks per SM (registers per thread
 // 255, 128, 64); one translation unit per bound (ants_arr_bMB.cu)
 cudaError_t launch_ants_arr_batch(int kw, int minb, const Colony* cols, const Ants* ants, const int2* map, int nmap,
-                                  int redo_blocks, const int2* redo_list, const int32_t* redo_n,
                                   size_t per_warp, cudaStream_t s);
 #define FACO_ARR_B_DECL(MB)                                                                                   \
   cudaError_t launch_ants_arr_batch_##MB(int kw, const Colony* cols, const Ants* ants, const int2* map,       \
-                                         int nmap, int redo_blocks, const int2* redo_list,                    \
-                                         const int32_t* redo_n, size_t per_warp, cudaStream_t s);             \
+                                         int nmap, size_t per_warp, cudaStream_t s);                          \
   cudaError_t prepare_ants_arr_batch_##MB(int kw, size_t smem);                                                \
   int occupancy_ants_arr_batch_##MB(int kw, size_t smem);
 FACO_ARR_B_DECL(2)

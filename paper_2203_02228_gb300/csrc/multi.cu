@@ -355,7 +355,6 @@ int Runner::build(const std::vector<RunEntry>& entries, size_t smem, cudaStream_
   nblk = (int)mblk.size();
   for (int v = 0; v < kNVariants; ++v) narr[v] = (int)marr[v].size();
   nmap256 = (int)m256.size();
-  redo_blocks = nblk > 0 ? kRedoBlocks : 0;  // a launch of its own, after the segment-table launch
   // one device block: tables, maps, redo list and count
   Bump B(nullptr);
   B.take<Colony>(C);
@@ -429,10 +428,9 @@ int Runner::enqueue(cudaStream_t s, int parts) const {
       if (u > 0) CK(cudaStreamWaitEvent(q, fork, 0));
       if (v == kVarTable) {
         CK(launch_ants_blk_batch(kw, dC, dA, map_blk, nblk, redo_list, redo_n, smem_blk, q));
-        CK(launch_ants_arr_batch(kw, 2, dC, dA, nullptr, 0, redo_blocks, redo_list, redo_n, per_warp, q));
+        CK(launch_ants_rest_batch(kw, dC, dA, std::min(nblk, kRedoBlocks), redo_list, redo_n, per_warp, q));
       } else {
-        CK(launch_ants_arr_batch(kw, kArrMinBlocks[v], dC, dA, map_arr[v], narr[v], 0, redo_list, redo_n,
-                                 per_warp, q));
+        CK(launch_ants_arr_batch(kw, kArrMinBlocks[v], dC, dA, map_arr[v], narr[v], per_warp, q));
       }
       if (u > 0) CK(cudaEventRecord(join[v], q));
     }

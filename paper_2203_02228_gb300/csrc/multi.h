@@ -21,7 +21,7 @@
 namespace faco {
 
 constexpr int kMultiMaxN = 262144;  // shared-memory visited bits (ants, nearest-neighbour tour)
-constexpr int kRedoBlocks = 38;     // blocks of the array kernel that serve the redo list
+constexpr int kRedoBlocks = 304;    // blocks that serve the redo list (two per SM)
 
 // Device-memory source for arenas (the batch: cudaMalloc; the server: its pool).
 struct DevAlloc {
@@ -84,7 +84,7 @@ enum : int { kVarTable = 0, kVarArr2 = 1, kVarArr4 = 2, kVarArr8 = 3, kNVariants
 constexpr int kArrMinBlocks[kNVariants] = {0, 2, 4, 8};
 
 struct Runner {
-  int count = 0, kw = 16, nblk = 0, nmap256 = 0, redo_blocks = 0;
+  int count = 0, kw = 16, nblk = 0, nmap256 = 0;
   int narr[kNVariants] = {0, 0, 0, 0};
   size_t smem_blk = 0, per_warp = 0;
   char* mem = nullptr;          // one cudaMalloc: tables, maps, redo list

@@ -399,7 +399,7 @@ struct ArrayRep {
   __device__ __forceinline__ void fetch(const LsShared&, int) {}
 };
 
-// The rounds of ls_run_block, until the search ends or the table is full
+// The rounds of the block search, until the search ends or the table is full
 // (sh.full).  In each, warp w evaluates the w-th queued node; entries are
 // popped in queue order up to and including the first one whose evaluation
 // found a move, which is applied.  Nothing changes the tour between the
@@ -519,12 +519,11 @@ __device__ __forceinline__ void ls_rounds(const LsEnv& E, Rep& rep, LsStats& S, 
   __syncthreads();
 }
 
-// The search of ls_run by a block on one tour.  A table that fills up (rare:
-// the tables are sized for it not to) is written out to arrays_of(), a tour over
-// source positions, the rest of the move that did not fit is applied there,
-// and the rounds go on with the same queue.  Must be called by every thread of
-// the block; tab: the table's state, the same on every thread.  Returns the
-// gain, and whether the tour is in the arrays.
+// The search of ls_run by a block on one tour: ls_begin with the checklist,
+// ls_rounds on the table, ls_end, each by every thread of the block.  When the
+// rounds end with the table full (rare: the tables are sized for it not to),
+// ls_to_arrays writes it out as arrays of source positions and applies the rest
+// of the move that did not fit, and the rounds go on there with the same queue.
 //
 // (A launch lasts as long as its slowest ant, and an ant that one warp builds
 // and searches again from the start takes several times as long as it had.
@@ -532,58 +531,54 @@ __device__ __forceinline__ void ls_rounds(const LsEnv& E, Rep& rep, LsStats& S, 
 // took 36.6 ms with min_new_edges = 64 (53 ants' tables fill up) and 197 ms with
 // 256 (963); going on takes 16.4 and 66.5 ms.  256 ants at n = 20,000 with
 // 64-segment tables: 4.0 against 1.16 ms.)
-template <bool TWO, class Arrays>
-__device__ __forceinline__ int64_t ls_run_block(const LsEnv& E, const SegTour& T, SegState& tab, Arrays arrays_of,
-                                                const int32_t* init, int ninit, LsStats& S, LsShared& sh,
-                                                bool& arrays) {
-  const int n = E.n, tid = threadIdx.x;
-  for (int i = tid; i < ninit; i += blockDim.x) {
+__device__ __forceinline__ void ls_begin(const LsEnv& E, const int32_t* init, int ninit, LsShared& sh) {
+  for (int i = threadIdx.x; i < ninit; i += blockDim.x) {
     const int x = init[i];
     E.queue[i] = x;
     E.flags[x] = 1;
   }
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     sh.qh = 0; sh.qn = ninit; sh.nlog = 0; sh.changes = 0; sh.moves_round = 0; sh.full = 0;
     sh.total = 0; sh.t_confirm = 0; sh.t_push = 0;
   }
   __syncthreads();
-  TableRep rep{T, tab};
-  ls_rounds<TWO>(E, rep, S, sh);
-  tab = rep.tab;
-  const int full = sh.full;
-  arrays = full != 0;
-  if (arrays) {
-    const uint64_t t0 = tid == 0 ? global_ns() : 0;
-    const SegView V = T.view(tab);
-    ArrayRep arr{arrays_of()};
-    for (int r = 0; r < V.S; ++r) {
-      const SegRec g = V.rec(r);
-      for (int q = g.lo + tid; q <= g.hi; q += blockDim.x) {
-        const int t = g.pos(q, n);
-        arr.T.route[t] = q;
-        arr.T.pos[q] = t;
-      }
+}
+
+// full: sh.full as the rounds left it; it is cleared.
+__device__ __forceinline__ void ls_to_arrays(const SegView& V, ArrTour& T, int full, LsStats& S, LsShared& sh) {
+  const int n = V.n, tid = threadIdx.x;
+  const uint64_t t0 = tid == 0 ? global_ns() : 0;
+  for (int r = 0; r < V.S; ++r) {
+    const SegRec g = V.rec(r);
+    for (int q = g.lo + tid; q <= g.hi; q += blockDim.x) {
+      const int t = g.pos(q, n);
+      T.route[t] = q;
+      T.pos[q] = t;
     }
-    __syncthreads();
-    if (tid < 32) {
-      // an Or-opt move's exchanges from the one that did not fit on (ls.cuh: apply_or)
-      const int* mv = sh.mv[full >> 2];
-      const int done = (full & 3) - 1;
-      if (mv[7] == 0) {
-        (void)tour_move2(arr.T, mv[0], mv[1], mv[2], mv[3], S);
-      } else {
-        if (done == 0) (void)tour_move2(arr.T, mv[0], mv[1], mv[4], mv[5], S);
-        if (done <= 1) (void)tour_move2(arr.T, mv[0], mv[4], mv[3], mv[2], S);
-        if (mv[6]) (void)tour_move2(arr.T, mv[4], mv[2], mv[1], mv[5], S);
-      }
-    }
-    if (tid == 0) {
-      sh.full = 0;
-      S.t_flip += (int64_t)(global_ns() - t0);
-    }
-    __syncthreads();
-    ls_rounds<TWO>(E, arr, S, sh);
   }
+  __syncthreads();
+  if (tid < 32) {
+    // an Or-opt move's exchanges from the one that did not fit on (ls.cuh: apply_or)
+    const int* mv = sh.mv[full >> 2];
+    const int done = (full & 3) - 1;
+    if (mv[7] == 0) {
+      (void)tour_move2(T, mv[0], mv[1], mv[2], mv[3], S);
+    } else {
+      if (done == 0) (void)tour_move2(T, mv[0], mv[1], mv[4], mv[5], S);
+      if (done <= 1) (void)tour_move2(T, mv[0], mv[4], mv[3], mv[2], S);
+      if (mv[6]) (void)tour_move2(T, mv[4], mv[2], mv[1], mv[5], S);
+    }
+  }
+  if (tid == 0) {
+    sh.full = 0;
+    S.t_flip += (int64_t)(global_ns() - t0);
+  }
+  __syncthreads();
+}
+
+// Leaves the flags clean.  Returns the gain.
+__device__ __forceinline__ int64_t ls_end(const LsEnv& E, LsStats& S, const LsShared& sh) {
+  const int n = E.n, tid = threadIdx.x;
   const int qh = sh.qh, qn = sh.qn, nl = sh.nlog;
   for (int t = tid; t < qn; t += blockDim.x) {
     int i = qh + t;

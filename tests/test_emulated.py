@@ -146,3 +146,25 @@ b.set_plan(0)
 b.iterate(3, 2)
 assert b.stats(0).seg_cap == 64 and b.stats(0).redone_ants > 0
 """)
+
+
+@pytest.mark.parametrize("k,new_edges", [(16, 34), (24, 30)])
+def test_batch_tables_full(emulated, monkeypatch, k, new_edges):
+    """Tables of 64 segments that fill up in construction, in the search, or
+    not at all."""
+    monkeypatch.setenv("EMU_SM_SHARED", "17664")
+    emulated("""
+import numpy as np
+import oracle
+from paper_2203_02228_gb300 import Batch, inputs
+xs = [inputs.uniform(400, seed=7), inputs.uniform(150, seed=8)]
+b = Batch(xs, {k}, seeds=[3, 4], min_new_edges={e}, plan=0)
+b.iterate(5, 2)
+tours, lens = b.tours()
+for i, x in enumerate(xs):
+    o = oracle.Colony(x, {k}, seed=3 + i, min_new_edges={e}, threads=4)
+    o.iterate(5, 2)
+    np.testing.assert_array_equal(tours[i], o.best()[0])
+    assert np.array_equal(b.tau(i).view(np.uint32), o.tau().view(np.uint32))
+assert b.stats(0).seg_cap == 64 and b.stats(0).redone_ants > 0
+""".format(k=k, e=new_edges), seed=k)

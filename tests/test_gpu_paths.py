@@ -185,3 +185,21 @@ def test_wide_batch_with_many_ants_on_tables():
         assert lens[i] == o.best()[1]
         np.testing.assert_array_equal(tours[i], o.best()[0])
         assert np.array_equal(b.tau(i).view(np.uint32), o.tau().view(np.uint32))
+
+
+@pytest.mark.parametrize("k,new_edges", [(16, 350), (16, 900), (20, 350), (16, 600), (20, 600), (16, 1500)])
+def test_batch_tables_full(k, new_edges):
+    """A batch whose tables (1,024 segments and more) do not fill up, do in the
+    search or in construction: the ants go on, or are built again, on arrays."""
+    xs = [inputs.uniform(2500, seed=91), inputs.uniform(1800, seed=92), inputs.uniform(60, seed=93)]
+    b = Batch(xs, k, seeds=[5, 6, 7], min_new_edges=new_edges, plan=0)
+    b.iterate(24, 3)
+    tours, lens = b.tours()
+    for i, xy in enumerate(xs):
+        o = oracle.Colony(xy, k, seed=5 + i, min_new_edges=new_edges, threads=8)
+        o.iterate(24, 3)
+        assert lens[i] == o.best()[1]
+        np.testing.assert_array_equal(tours[i], o.best()[0])
+        assert np.array_equal(b.tau(i).view(np.uint32), o.tau().view(np.uint32))
+    if new_edges >= 900:
+        assert b.stats(0).redone_ants > 0
