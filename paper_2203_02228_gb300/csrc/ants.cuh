@@ -672,7 +672,7 @@ __device__ __forceinline__ void ants_arr_body(const Colony& C, const Ants& A, in
 
 // One block of kAntWarps warps per ant, tour as a segment table in shared
 // memory: warp 0 constructs, then all warps run the local search with
-// speculative in-order pops (ls_run_block).  An ant whose table fills up in
+// speculative in-order pops (seg.cuh).  An ant whose table fills up in
 // construction is marked and redone by the array kernel.  A launch lasts as
 // long as its slowest ant; wider blocks speculate deeper, so the slowest ants finish
 // sooner, while fewer blocks fit an SM.  Registers per thread: with
