@@ -857,19 +857,28 @@ __global__ void __maxnreg__(kAntFewRegs)
 }
 
 // Batch, arrays: a block runs the four ants map[b].y + warp of colony
-// map[b].x.  per_warp is the shared-memory stride of a warp.
+// map[b].x, for every b of its stride (a launch has a block for each).  per_warp
+// is the shared-memory stride of a warp.
+// Descriptors by warp and the loop are what the compiler does best with.  One
+// descriptor per block, without the loop: 512 instances 146 -> 142 ms (8 blocks
+// per SM) and 154 -> 147 (4), but 42 small ones, a wave that the slowest ant
+// ends, 11.0 -> 11.4; with the loop 150, 160 and 10.8.
 template <int KW, int MB>
 __global__ void __launch_bounds__(128, MB)
-    k_ants_b(const Colony* cols, const Ants* ants, const int2* map, size_t per_warp) {
+    k_ants_b(const Colony* cols, const Ants* ants, const int2* map, int nmap, size_t per_warp) {
   extern __shared__ __align__(16) char smem[];
-  __shared__ Colony sC;
-  __shared__ Ants sA;
+  __shared__ Colony sC[4];
+  __shared__ Ants sA[4];
   const int wib = threadIdx.x >> 5;
-  const int2 e = map[blockIdx.x];
-  copy_words(&sC, cols + e.x, sizeof(Colony), 0, blockDim.x);
-  copy_words(&sA, ants + e.x, sizeof(Ants), 0, blockDim.x);
-  __syncthreads();
-  ants_arr_body<KW>(sC, sA, e.y + wib, smem + (size_t)wib * per_warp);
+  for (int b = blockIdx.x; b < nmap; b += gridDim.x) {
+    int2 e = map[b];
+    e.y += wib;
+    copy_words(&sC[wib], cols + e.x, sizeof(Colony), wib * 32, 32);
+    copy_words(&sA[wib], ants + e.x, sizeof(Ants), wib * 32, 32);
+    __syncwarp();
+    ants_arr_body<KW>(sC[wib], sA[wib], e.y, smem + (size_t)wib * per_warp);
+    __syncwarp();
+  }
 }
 
 }  // namespace

@@ -16,9 +16,9 @@ cudaError_t launch_arr_b_mb(int kw, const Colony* cols, const Ants* ants, const 
   if (nmap <= 0) return cudaSuccess;
   const size_t smem = 4 * per_warp;
   if (kw == 16)
-    k_ants_b<16, MB><<<nmap, 128, smem, s>>>(cols, ants, map, per_warp);
+    k_ants_b<16, MB><<<nmap, 128, smem, s>>>(cols, ants, map, nmap, per_warp);
   else
-    k_ants_b<32, MB><<<nmap, 128, smem, s>>>(cols, ants, map, per_warp);
+    k_ants_b<32, MB><<<nmap, 128, smem, s>>>(cols, ants, map, nmap, per_warp);
   return cudaGetLastError();
 }
 
